@@ -1132,7 +1132,7 @@ int launch_batches(nk_graph *g, const int32_t *d_src, int32_t k, double *d_score
     constexpr int B = 64 * W;
     // sources without arcs add nothing: the batches take the others (the error-bounded
     // estimate keeps its slots, which are tied to their targets)
-    Tmp csrc, ccnt;
+    Tmp csrc, ccnt, osrc, okey;
     if (!cfg.rk_t) {
         NK_TRY(csrc.alloc(sizeof(int32_t) * (size_t)k, s));
         NK_TRY(ccnt.alloc(sizeof(int32_t), s));
@@ -1149,6 +1149,15 @@ int launch_batches(nk_graph *g, const int32_t *d_src, int32_t k, double *d_score
                 st->batch = B;
             }
             return NK_OK;
+        }
+        // more than one batch: similar sources share one.  R-MAT 18, 670 sources by 128: 65.2M
+        // rows gathered in the order of the ids, 42.8M in this order, 18.3 -> 13.4 ms; R-MAT 24,
+        // 271 sources: 493 -> 348 ms; BA 10^6, 512 sources: 40.2 -> 36.9 ms; ER (no hubs) equal
+        if (k > B && !cfg.keep_order) {
+            NK_TRY(osrc.alloc(sizeof(int32_t) * (size_t)k, s));
+            NK_TRY(okey.alloc(sizeof(unsigned long long) * (size_t)k, s));
+            NK_TRY(order_sources(g, d_src, k, ccnt.as<int32_t>(), okey.as<unsigned long long>(), osrc.as<int32_t>(), s));
+            d_src = osrc.as<int32_t>();
         }
     }
     HeavyView hw;
@@ -1357,9 +1366,10 @@ int enqueue_batches(nk_graph *g, const int32_t *d_src, int32_t k, double *d_scor
     if (lcap < 4) return set_error(NK_ERR_NOMEM, "not enough device memory for a batch of %d sources", B);
     const int nb = (k + B - 1) / B;
     const Layout L = layout(g, B, lcap, hw.chunk);
-    // status words of the nb batches, then the compacted sources and their count
-    const size_t ctrl_bytes = align_up(sizeof(Ctrl) * nb);
-    const size_t bctrl_bytes = ctrl_bytes + align_up(sizeof(int32_t) * (size_t)k) + 256;
+    // status words of the nb batches, then the compacted sources and their count; with more
+    // than one batch also the ordered sources and their keys
+    const size_t ctrl_bytes = align_up(sizeof(Ctrl) * nb), src_bytes = align_up(sizeof(int32_t) * (size_t)k);
+    const size_t bctrl_bytes = ctrl_bytes + src_bytes + 256 + (nb > 1 ? src_bytes + sizeof(unsigned long long) * (size_t)k : 0);
     if (prepare_only) {
         NK_TRY(ws[WS_BATCH].ensure(L.total));
         NK_TRY(ws[WS_BCTRL].ensure(bctrl_bytes));
@@ -1415,10 +1425,16 @@ int enqueue_batches(nk_graph *g, const int32_t *d_src, int32_t k, double *d_scor
     a.dir = cfg.direction;
     Ctrl *ctrls = ws[WS_BCTRL].as<Ctrl>();
     int32_t *csrc = reinterpret_cast<int32_t *>(ws[WS_BCTRL].as<char>() + ctrl_bytes);
-    int32_t *ccnt = reinterpret_cast<int32_t *>(ws[WS_BCTRL].as<char>() + ctrl_bytes + align_up(sizeof(int32_t) * (size_t)k));
+    int32_t *ccnt = reinterpret_cast<int32_t *>(ws[WS_BCTRL].as<char>() + ctrl_bytes + src_bytes);
     NK_CUDA(cudaMemsetAsync(ctrls, 0, sizeof(Ctrl) * nb, s));
     // sources without arcs add nothing: compacted on the device, each batch reads the count
     NK_TRY(compact_sources(g, d_src, k, csrc, ccnt, s));
+    if (nb > 1) {
+        char *ob = ws[WS_BCTRL].as<char>() + ctrl_bytes + src_bytes + 256;
+        int32_t *osrc = reinterpret_cast<int32_t *>(ob);
+        NK_TRY(order_sources(g, csrc, k, ccnt, reinterpret_cast<unsigned long long *>(ob + src_bytes), osrc, s));
+        csrc = osrc;
+    }
     a.ksrc = ccnt;
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeCooperative;

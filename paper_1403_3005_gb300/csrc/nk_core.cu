@@ -311,6 +311,65 @@ int compact_sources(const nk_graph *g, const int32_t *d_src, int32_t k, int32_t 
     return NK_OK;
 }
 
+// ---------------------------------------------------------------- similar sources together
+namespace {
+constexpr int kKeyArcs = 2048;      // arcs of a source that its key looks at
+constexpr int kRankSegment = 32768; // sources ranked against one another
+
+// key[i] = number of walks of length two from source i (the sum of its neighbours' degrees),
+// a warp per source.  Of longer rows every stride-th arc is read and the sum multiplied by
+// the stride.
+__global__ void __launch_bounds__(256)
+k_source_keys(const int32_t *rp, const int32_t *col, const int32_t *src, const int32_t *count,
+              unsigned long long *key)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (i >= *count) return;
+    const int v = src[i], beg = rp[v], deg = rp[v + 1] - beg;
+    const int stride = (deg + kKeyArcs - 1) / kKeyArcs;
+    unsigned long long t = 0;
+    for (int64_t j = (int64_t)lane * stride; j < deg; j += 32ll * stride) {
+        const int c = __ldg(col + beg + j);
+        t += (unsigned)(__ldg(rp + c + 1) - __ldg(rp + c));
+    }
+    t = dev::group_sum<32>(t) * (unsigned)stride;
+    if (lane == 0) key[i] = t;
+}
+
+// Sources in the order of falling keys (equal keys: as they were), a warp per source, which
+// counts the sources before it.  Lists above kRankSegment are ordered segment by segment.
+__global__ void __launch_bounds__(256)
+k_source_rank(const int32_t *src, const int32_t *count, const unsigned long long *key, int32_t *out)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int k = *count;
+    if (i >= k) return;
+    const int64_t lo = i / kRankSegment * kRankSegment, hi = min(lo + kRankSegment, (int64_t)k);
+    const unsigned long long x = key[i];
+    int before = 0;
+    for (int64_t j = lo + lane; j < hi; j += 32) {
+        const unsigned long long y = __ldg(key + j);
+        before += y > x || (y == x && j < i);
+    }
+    before = dev::group_sum<32>(before);
+    if (lane == 0) out[lo + before] = src[i];
+}
+}  // namespace
+
+int order_sources(const nk_graph *g, const int32_t *d_src, int32_t k, const int32_t *d_count,
+                  unsigned long long *d_key, int32_t *d_out, cudaStream_t s)
+{
+    const unsigned blocks = (unsigned)(((int64_t)k + 7) / 8);
+    k_source_keys<<<blocks, 256, 0, s>>>(g->rp.as<int32_t>(), g->col.as<int32_t>(), d_src, d_count, d_key);
+    ::nk::count_launch();
+    k_source_rank<<<blocks, 256, 0, s>>>(d_src, d_count, d_key, d_out);
+    ::nk::count_launch();
+    NK_CUDA(cudaGetLastError());
+    return NK_OK;
+}
+
 // ---------------------------------------------------------------- vector scale
 namespace {
 __global__ void k_scale(double *d, int32_t n, double s)

@@ -234,6 +234,7 @@ struct RunCfg {
     double *edge = nullptr;               // edge betweenness: per-arc sums (device, A), or null
     int chunk = 0;                        // batched sweep: arcs per hub chunk (0: kHeavyChunk)
     bool relabel = false;                 // betweenness entry: use the relabelled copy
+    bool keep_order = false;              // batched sweep: batches in the order the sources are given
     // error-bounded estimate: per source index i, the target of its random shortest path,
     // the key of the walk's random stream, and the per-vertex counts of interior vertices
     const int32_t *rk_t = nullptr;
@@ -287,6 +288,14 @@ size_t batched_bytes_lcap(const nk_graph *g, int B, int lcap);
 // One CTA, no allocation (usable inside a stream capture); the ids must be in range.
 int compact_sources(const nk_graph *g, const int32_t *d_src, int32_t k, int32_t *d_out, int32_t *d_count,
                     cudaStream_t s);
+
+// Orders the sources d_src[0..*d_count) (device; k is an upper bound of the count) so that
+// consecutive ones have similar BFS trees: by the number of two-step walks from them, largest
+// first.  A batch of the multi-source sweep reads a neighbour's row once for all sources that
+// have it on the same level, so a batch of similar sources reads fewer rows.  d_key: k words
+// of scratch.  No allocation (usable inside a stream capture); the order is deterministic.
+int order_sources(const nk_graph *g, const int32_t *d_src, int32_t k, const int32_t *d_count,
+                  unsigned long long *d_key, int32_t *d_out, cudaStream_t s);
 
 // Scale a device vector in place.
 int scale_vector(double *d, int32_t n, double scale, cudaStream_t s);

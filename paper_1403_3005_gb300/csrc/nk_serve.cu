@@ -254,6 +254,7 @@ int run_pack(nk_server *S, const std::vector<Request *> &rs, cudaStream_t st, do
     RunCfg cfg;
     cfg.mode = NK_MODE_BATCHED;
     cfg.batch = k_u > 64 ? kPackWidth : 64;
+    cfg.keep_order = true;  // the members' sources stay together: a batch of several graphs shares no rows
     cfg.ws = ws;
     cfg.grid_ctas = (int)std::min<int64_t>(std::max<int64_t>(A_u / 8192, 128), 1 << 20);
     cfg.grid_div = 2;
