@@ -55,8 +55,9 @@ constexpr int kStartLevels = 48; // level slabs of a first attempt
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int kTraceCap = 1024;
 constexpr int kChunk = kHeavyChunk;  // default arcs per work item; longer rows are split
-constexpr int kGrabQ = 8;            // queue entries a warp takes at a time
-constexpr int kGrabV = 32;           // vertices a warp scans at a time (one ballot window)
+constexpr int kGrabV = 32;           // most vertices a warp takes at a time (one per lane)
+constexpr int kGrabArcs = 256;       // arcs, by the graph's average, a warp takes at a time
+constexpr int kGrabShare = 4;        // a warp takes at most 1/kGrabShare of its share of a phase
 constexpr int kGrabCMax = 16;        // most heavy chunks a warp takes at a time
 // work-counter slots of a level
 enum { WQ_BU = 0, WQ_BU_C, WQ_PUSH, WQ_PUSH_C, WQ_PULL, WQ_PULL_C, WQ_BACK, WQ_BACK_C };
@@ -160,7 +161,7 @@ __device__ __forceinline__ int deg_of(const int32_t *rp, int v) { return __ldg(r
 // batch.  Slot k of lane L is source G L + k: bit G L + k of the batch's bitsets (word
 // (G L + k) / 64) and entry G L + k of a vertex's row of B values, so that one contiguous load
 // moves all of a lane's values of a row, and the lane's bits of a bitset are one field of one
-// word.
+// byte.
 template <int W> __device__ __forceinline__ int slot_off(int k, int lane) { return 2 * W * lane + k; }
 
 // The word of a bitset that holds the lane's slots (selected without indexing the register
@@ -175,16 +176,21 @@ template <int W> __device__ __forceinline__ unsigned long long lane_word(const B
     return w;
 }
 
-template <int W> __device__ __forceinline__ bool has_slot(const Bits<W> &b, int k, int lane)
-{
-    return (lane_word<W>(b, lane) >> ((2 * W * lane + k) & 63)) & 1ull;
-}
-
-// The lane's 2W bits of a bitset of W words.
+// The lane's 2W bits of a bitset of W words in shared memory: a field of one byte.
 template <int W> __device__ __forceinline__ unsigned lane_bits(const unsigned long long *w, int lane)
 {
     const int s = 2 * W * lane;
-    return (unsigned)(w[s >> 6] >> (s & 63)) & ((1u << (2 * W)) - 1u);
+    return ((unsigned)reinterpret_cast<const unsigned char *>(w)[s >> 3] >> (s & 7)) & ((1u << (2 * W)) - 1u);
+}
+
+// Every lane's 2W bits stored as a bitset of W words in shared memory: the lanes of a byte
+// join their fields, the first of them stores it.
+template <int W> __device__ __forceinline__ void store_lane_bits(unsigned long long *w, unsigned f, int lane)
+{
+    constexpr int LPB = 8 / (2 * W);  // lanes of a byte: 4, 2, 1
+#pragma unroll
+    for (int o = 1; o < LPB; o <<= 1) f |= __shfl_down_sync(FULL, f, o) << (2 * W * o);
+    if (lane % LPB == 0) reinterpret_cast<unsigned char *>(w)[lane / LPB] = (unsigned char)f;
 }
 
 // acc += x with the carry out of bit 63 counted in carry (a path-count overflow).
@@ -203,28 +209,32 @@ __device__ __forceinline__ void check_failed(const BArgs &a, int code, int where
     }
 }
 
-// One warp's list of the relevant neighbours of the current 32-arc window of a gather:
-// their ids, masked source bits and arc indices, in shared memory.
-template <int W> struct Nbrs {
-    unsigned long long f[32][W];
-    int c[32];
-    int j[32];
-    double e[32];  // edge variant: each listed arc's share of the window
+// One warp's shared memory: the group of vertices it works on, and the list of the relevant
+// neighbours of the current window of 32 arcs.
+template <int W, bool EDGE> struct WarpBuf {
+    unsigned long long f[32][W];  // list: bits the neighbour shares with its vertex
+    unsigned long long t[32][W];  // group: the bits a vertex gathers (a pull leaves its new bits here)
+    int c[32];                    // list: neighbour
+    int o[32];                    // list: its vertex's place in the group
+    int off[32];                  // group: first arc, less the arcs of the vertices before
+    int v[32];                    // group: vertex
+    unsigned long long until;     // deadline of the phase
+    double e[EDGE ? 32 : 1];      // list, edge variant: the arc's share
 };
 
-// sum_k sv[k] * x[k] over the lane's G slots (x: double-single pairs packed in 64 bits, zero
-// for slots that are not relevant), as a compensated dot product (Ogita, Rump and Oishi's
-// Dot2): the leading products hi*hi are summed by TwoSum, and their exact FMA errors, the
-// cross terms hi*lo and lo*hi and the TwoSum errors are gathered in one float instead of
-// renormalising the pair after every term.  All terms are non-negative (sigma and psi are),
-// so the gathered float stays a small fraction of the sum.
+// sum_k sv[k] * x[k] over the lane's G slots (x: double-single pairs, zero for slots that are
+// not relevant), as a compensated dot product (Ogita, Rump and Oishi's Dot2): the leading
+// products hi*hi are summed by TwoSum, and their exact FMA errors, the cross terms hi*lo and
+// lo*hi and the TwoSum errors are gathered in one float instead of renormalising the pair
+// after every term.  All terms are non-negative (sigma and psi are), so the gathered float
+// stays a small fraction of the sum.
 template <int G>
-__device__ __forceinline__ dev::ff edge_dot(const dev::ff *sv, const unsigned long long (&x)[G])
+__device__ __forceinline__ dev::ff edge_dot(const dev::ff (&sv)[G], const dev::ff (&x)[G])
 {
     float s = 0.0f, c = 0.0f;
 #pragma unroll
     for (int k = 0; k < G; ++k) {
-        const dev::ff b = dev::ff_unpack(x[k]);
+        const dev::ff b = x[k];
         const float p = __fmul_rn(sv[k].hi, b.hi);
         c = __fmaf_rn(sv[k].hi, b.lo, __fmaf_rn(sv[k].lo, b.hi, __fadd_rn(c, __fmaf_rn(sv[k].hi, b.hi, -p))));
         const float t = __fadd_rn(s, p);
@@ -246,169 +256,257 @@ __device__ __forceinline__ dev::ff edge_sum2(dev::ff a, dev::ff b)
     return {t, __fadd_rn(__fadd_rn(a.lo, b.lo), e)};
 }
 
-// For the warp's vertex with adjacency [beg, end): per source slot, the sum of sp over
-// the neighbours c whose Fsel[c] & tgt holds that source bit; uint64 sums (sigma, with
-// carry detection) or double-single sums (psi).  Lanes over arcs find the relevant
-// neighbours of a 32-arc window and list them in shared memory; then the lanes, each on
-// its source pairs, read two listed neighbours' rows per round with 16-byte loads (both
-// neighbours' loads in flight together) and add the relevant entries.
-// With EDGE (backward only) the warp's vertex v also hands every relevant arc (v, c) its
-// share sum_b sigma_b(v) * psi_b(c) over the gathered source bits (sv holds sigma_b(v) of
-// the lane's slots): a warp sum per neighbour, parked in shared memory, then added to
-// edge[j] by the lane that listed the arc, which loaded the old value when it listed it (the
-// load is in flight during the rounds, so no round waits on a read-modify-write).  The arc
-// is owned by v's warp at this level, so no atomics are needed.
-template <int W, bool PSI, bool EDGE = false, bool S32 = false>
-__device__ __forceinline__ void gather(const BArgs &a, int beg, int end,
-                                       const unsigned long long *Fsel, const Bits<W> &tgt,
-                                       unsigned long long (&acc)[2 * W], dev::ff (&facc)[2 * W],
-                                       bool &ovf, Nbrs<W> &st, const dev::ff *sv = nullptr)
+// 16- and 8-byte loads that bypass L1, zeros where `on` is zero.  Written out so that a load is
+// predicated: the compiler made it a branch, and R-MAT 18 took 13.6 instead of 12.5 ms.  (Reading
+// a dummy address instead takes 33 ms: the lanes of all warps meet in one L2 slice.)
+__device__ __forceinline__ void load16_if(unsigned on, const void *p, unsigned &x, unsigned &y, unsigned &z, unsigned &w)
 {
-    constexpr int B = 64 * W;
+    x = y = z = w = 0;
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t@p ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%5];\n\t}"
+                 : "+r"(x), "+r"(y), "+r"(z), "+r"(w) : "r"(on), "l"(p));
+}
+__device__ __forceinline__ void load8_if(unsigned on, const void *p, unsigned &x, unsigned &y)
+{
+    x = y = 0;
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p ld.global.cg.v2.u32 {%0, %1}, [%3];\n\t}"
+                 : "+r"(x), "+r"(y) : "r"(on), "l"(p));
+}
+
+// acc += x where on is not zero
+__device__ __forceinline__ void add_if(unsigned on, unsigned long long &acc, unsigned x)
+{
+    asm("{\n\t.reg .pred p;\n\t.reg .b64 t;\n\tsetp.ne.u32 p, %1, 0;\n\tcvt.u64.u32 t, %2;\n\t@p add.u64 %0, %0, t;\n\t}"
+        : "+l"(acc) : "r"(on), "r"(x));
+}
+
+// dev::ff_add(a, {hi, lo}), operation by operation, where on is not zero: only the two results
+// are predicated, which replaces the two selections of an addition of zero
+__device__ __forceinline__ void ff_add_if(unsigned on, dev::ff &a, unsigned hi, unsigned lo)
+{
+    asm("{\n\t.reg .pred p;\n\t.reg .f32 s, v, e, t;\n\t"
+        "setp.ne.u32 p, %2, 0;\n\t"
+        "add.rn.f32 s, %0, %3;\n\t"
+        "sub.rn.f32 v, s, %0;\n\t"
+        "sub.rn.f32 e, s, v;\n\t"
+        "sub.rn.f32 e, %0, e;\n\t"
+        "sub.rn.f32 v, %3, v;\n\t"
+        "add.rn.f32 e, e, v;\n\t"
+        "add.rn.f32 t, %1, %4;\n\t"
+        "add.rn.f32 t, e, t;\n\t"
+        "@p add.rn.f32 %0, s, t;\n\t"
+        "sub.rn.f32 v, %0, s;\n\t"
+        "@p sub.rn.f32 %1, t, v;\n\t}"
+        : "+f"(a.hi), "+f"(a.lo) : "r"(on), "f"(__uint_as_float(hi)), "f"(__uint_as_float(lo)));
+}
+
+// A lane's 2W values of a vertex's row, loaded in 16-byte pieces, each only if one of its
+// entries is relevant (nib); the values of other entries are undefined.
+template <int W, bool S32> struct RowPart {
+    static constexpr int G = 2 * W;
+    unsigned u[S32 ? G : 2 * G];
+    __device__ __forceinline__ void load(const BArgs &a, int c, int lane, unsigned nib)
+    {
+        if constexpr (S32) {
+            const unsigned *row = a.sp32 + (size_t)c * (64 * W) + G * lane;
+            if constexpr (G == 2) {
+                load8_if(nib, row, u[0], u[1]);
+            } else {
+#pragma unroll
+                for (int h = 0; h < G / 4; ++h)
+                    load16_if(nib & (15u << (4 * h)), row + 4 * h, u[4 * h], u[4 * h + 1], u[4 * h + 2], u[4 * h + 3]);
+            }
+        } else {
+            const unsigned long long *row = a.sp + (size_t)c * (64 * W) + G * lane;
+#pragma unroll
+            for (int h = 0; h < G / 2; ++h)
+                load16_if(nib & (3u << (2 * h)), row + 2 * h, u[4 * h], u[4 * h + 1], u[4 * h + 2], u[4 * h + 3]);
+        }
+    }
+    __device__ __forceinline__ unsigned long long u64(int k) const
+    {
+        if constexpr (S32) return u[k];
+        else return ((unsigned long long)u[2 * k + 1] << 32) | u[2 * k];
+    }
+    // a path count as a double-single number
+    __device__ __forceinline__ dev::ff count(int k) const
+    {
+        if constexpr (S32) return dev::ff_from_u32(u[k]);
+        else return dev::ff_from_u64(u64(k));
+    }
+};
+
+// Gathers, for a group of up to 32 vertices (lane L's vertex v with arcs [beg, beg + dg) and
+// bits t, where `on`), per source slot the sum of sp over the neighbours c whose Fsel[c] & t
+// holds that source's bit: uint64 sums (sigma, with carry detection) or double-single sums
+// (psi).  The warp walks the concatenated arcs of the group in windows of 32, lanes over arcs:
+// a window's column ids, then their level bits, are read in one step whatever the rows'
+// lengths, and the neighbours that share a bit with their vertex are listed in shared memory
+// in the order of the arcs.  Then the lanes, each on its own source slots, read the rows of
+// NB listed neighbours at a time (all of their loads in flight together) and add the relevant
+// entries.  When the list comes to another vertex, flush(o) takes the sums of the vertex at
+// place o and clears them, and begin(o) is called for the next.  One vertex at a time, a row
+// of 8 arcs used 8 of 32 lanes and paid the chain of column, bits and row reads by itself: ER
+// 200003 (degree 8) k = 300 in batches of 128 takes 5.1 ms in groups, 8.0 ms without.  What bounds
+// it is instruction issue and the latency of its reads (R-MAT 20: issue active 56 %, DRAM 7 %).
+// Vertices without a relevant neighbour are never flushed.  Returns the places flushed; pos:
+// the lane's vertex's place, or -1.
+// With EDGE (psi only) every relevant arc (v, c) also gets its share sum_b sigma_b(v) *
+// psi_b(c) (sv: sigma_b of the vertex's slots, set by begin): a warp sum per neighbour, parked
+// in shared memory, then added to edge[j] by the lane that listed the arc, which loaded the old
+// value when it listed it.  The arc is owned by this warp at this level: no atomics.
+template <int W, bool PSI, bool EDGE, bool S32, class Buf, class Begin, class Flush>
+__device__ __forceinline__ unsigned gather(const BArgs &a, bool on, int v, int beg, int dg, const Bits<W> &t,
+                                           const unsigned long long *Fsel, Buf &st,
+                                           unsigned long long (&acc)[2 * W], dev::ff (&facc)[2 * W],
+                                           dev::ff (&sv)[2 * W], bool &ovf, int &pos, Begin begin, Flush flush)
+{
+    // rows in flight.  With 2 instead of 4 rows of 32-bit counts R-MAT 18 and BA 10^6 (128 sources)
+    // go from 13.2 to 13.5 and 33.5 to 35.7 ms; with 4 rows of psi the W = 2 and 4 kernels run out of
+    // registers (256 sources: 12.7 -> 14.7, 33.0 -> 45.6 ms), the W = 1 one gains (15.9 -> 15.4,
+    // 41.5 -> 36.0 ms)
+    constexpr int G = 2 * W, NB = S32 || (PSI && !EDGE && W == 1) ? 4 : 2;
     const int lane = threadIdx.x & 31;
     unsigned carry = 0;
-    if (beg < 0 || end < beg || (long long)end > a.A) {  // warp-uniform
-        if (lane == 0) check_failed(a, kErrCheck, 1, beg);
-        return;
+    if (on && (beg < 0 || dg < 0 || (long long)beg + dg > a.A)) {
+        check_failed(a, kErrCheck, 1, beg);
+        on = false;
     }
-    for (int base = beg; base < end; base += 32) {
-        const int j = base + lane;
-        int c = 0;
+    const int d0 = on ? dg : 0;
+    int incl = d0;
+#pragma unroll
+    for (int s = 1; s < 32; s <<= 1) {
+        const int y = __shfl_up_sync(FULL, incl, s);
+        if (lane >= s) incl += y;
+    }
+    const int total = __shfl_sync(FULL, incl, 31), pre = incl - d0;
+    const unsigned members = __ballot_sync(FULL, d0 > 0);
+    pos = d0 > 0 ? __popc(members & dev::lanemask_lt()) : -1;
+    __syncwarp();  // the group before is done with the buffer
+    if (d0 > 0) {
+        st.v[pos] = v;
+        st.off[pos] = beg - pre;
+#pragma unroll
+        for (int q = 0; q < W; ++q) st.t[pos][q] = t.w[q];
+    }
+    __syncwarp();
+    int cur = -1, before = 0;
+    unsigned done = 0;
+    for (int base = 0; base < total; base += 32) {
+        // the vertices whose arcs start in this window mark their first arc; an arc's vertex is
+        // the number of marks up to it
+        const unsigned marks = __reduce_or_sync(FULL, d0 > 0 && (unsigned)(pre - base) < 32u ? 1u << (pre - base) : 0u);
+        const int o = before + __popc(marks & (dev::lanemask_lt() << 1 | 1u)) - 1;
+        before += __popc(marks);
+        int c = 0, j = 0;
         Bits<W> f;
 #pragma unroll
         for (int q = 0; q < W; ++q) f.w[q] = 0;
-        if (j < end) {
+        if (base + lane < total) {
+            j = st.off[o] + base + lane;
             c = __ldg(a.col + j);
             const Bits<W> fc = load_bits<W>(Fsel + (size_t)c * W);
 #pragma unroll
-            for (int q = 0; q < W; ++q) f.w[q] = fc.w[q] & tgt.w[q];
+            for (int q = 0; q < W; ++q) f.w[q] = fc.w[q] & st.t[o][q];
         }
         const bool mine = any_bits<W>(f);
         const unsigned rel = __ballot_sync(FULL, mine);
         if (!rel) continue;
-        const int pos = __popc(rel & dev::lanemask_lt());
+        const int at = __popc(rel & dev::lanemask_lt()), cnt = __popc(rel);
+        // list entries whose vertex is not that of the entry before
+        const int lead = __shfl_sync(FULL, o, 31 - __clz(rel & dev::lanemask_lt()));
+        const unsigned fresh = __reduce_or_sync(FULL, mine && o != (at ? lead : cur) ? 1u << at : 0u);
         double eold = 0.0;
         if (mine) {
-            st.c[pos] = c;
-            st.j[pos] = j;
+            st.c[at] = c;
+            st.o[at] = o;
 #pragma unroll
-            for (int q = 0; q < W; ++q) st.f[pos][q] = f.w[q];
+            for (int q = 0; q < W; ++q) st.f[at][q] = f.w[q];
             if constexpr (EDGE) eold = __ldcg(a.edge + j);
         }
+        if (lane >= cnt && lane < ((cnt + NB - 1) & ~(NB - 1))) {  // the last round's empty places
+            st.c[lane] = 0;
+#pragma unroll
+            for (int q = 0; q < W; ++q) st.f[lane][q] = 0;
+        }
         __syncwarp();
-        // NB relevant neighbours per round (two for the edge variant): every load of the
-        // round is issued before any addition, so their latencies overlap
-        constexpr int NB = 2;
-        unsigned left = rel;
-        while (left) {
-            int idx[NB];
-            bool on[NB];
-#pragma unroll
-            for (int r = 0; r < NB; ++r) {
-                on[r] = left != 0;
-                const int sr = on[r] ? __ffs(left) - 1 : 0;
-                if (on[r]) left &= left - 1;
-                idx[r] = on[r] ? __popc(rel & ((1u << sr) - 1u)) : 0;
-            }
-            // the lane's 2W bits of each listed neighbour, then one contiguous stretch of its row
-            // per neighbour: 2W entries of 4 bytes (32-bit sigma) or 8 bytes, in 16-byte loads,
-            // each issued only if one of its entries is relevant
-            constexpr int G = 2 * W;
+        for (int i = 0; i < cnt; i += NB) {
             unsigned nib[NB];
-            unsigned long long x[NB][G];
+            RowPart<W, S32> x[NB];
 #pragma unroll
             for (int r = 0; r < NB; ++r) {
-                nib[r] = on[r] ? lane_bits<W>(st.f[idx[r]], lane) : 0u;
-                if constexpr (S32) {
-                    const unsigned *row = a.sp32 + (size_t)st.c[idx[r]] * B + G * lane;
-                    if constexpr (G == 2) {
-                        unsigned long long p = 0ull;
-                        if (nib[r]) p = __ldcg(reinterpret_cast<const unsigned long long *>(row));
-                        x[r][0] = p & 0xffffffffull;
-                        x[r][1] = p >> 32;
-                    } else {
+                nib[r] = lane_bits<W>(st.f[i + r], lane);
+                x[r].load(a, st.c[i + r], lane, nib[r]);
+            }
+            dev::ff e[NB];
+            auto add = [&](int r) {
+                if constexpr (PSI && EDGE) {
+                    dev::ff y[G];
 #pragma unroll
-                        for (int h = 0; h < G / 4; ++h) {
-                            uint4 p = make_uint4(0u, 0u, 0u, 0u);
-                            if ((nib[r] >> (4 * h)) & 15u) p = __ldcg(reinterpret_cast<const uint4 *>(row) + h);
-                            x[r][4 * h] = p.x;
-                            x[r][4 * h + 1] = p.y;
-                            x[r][4 * h + 2] = p.z;
-                            x[r][4 * h + 3] = p.w;
-                        }
+                    for (int k = 0; k < G; ++k) {
+                        y[k] = (nib[r] >> k) & 1u ? dev::ff_unpack(x[r].u64(k)) : dev::ff_zero();
+                        facc[k] = dev::ff_add(facc[k], y[k]);
                     }
-                } else {
-                    const unsigned long long *row = a.sp + (size_t)st.c[idx[r]] * B + G * lane;
+                    e[r] = edge_dot<G>(sv, y);
+                } else if constexpr (PSI) {
 #pragma unroll
-                    for (int h = 0; h < G / 2; ++h) {
-                        ulonglong2 p = make_ulonglong2(0ull, 0ull);
-                        if ((nib[r] >> (2 * h)) & 3u) p = __ldcg(reinterpret_cast<const ulonglong2 *>(row) + h);
-                        x[r][2 * h] = p.x;
-                        x[r][2 * h + 1] = p.y;
+                    for (int k = 0; k < G; ++k) ff_add_if(nib[r] & (1u << k), facc[k], x[r].u[2 * k], x[r].u[2 * k + 1]);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < G; ++k) {
+                        // 32-bit counts: a row of under 2^31 of them cannot overflow 64 bits
+                        if constexpr (S32) add_if(nib[r] & (1u << k), acc[k], x[r].u[k]);
+                        else add_carry(acc[k], carry, (nib[r] >> k) & 1u ? x[r].u64(k) : 0ull);
                     }
                 }
-            }
+            };
+            if (!((fresh >> i) & ((1u << NB) - 1u))) {  // warp-uniform: all of one vertex
 #pragma unroll
-            for (int r = 0; r < NB; ++r)
-#pragma unroll
-                for (int k = 0; k < G; ++k)
-                    if (!((nib[r] >> k) & 1u)) x[r][k] = 0ull;
-#pragma unroll
-            for (int k = 0; k < 2 * W; ++k) {
+                for (int r = 0; r < NB; ++r) add(r);
+            } else {
 #pragma unroll
                 for (int r = 0; r < NB; ++r) {
-                    if constexpr (PSI) {
-                        facc[k] = dev::ff_add(facc[k], dev::ff_unpack(x[r][k]));
-                    } else {
-                        add_carry(acc[k], carry, x[r][k]);
+                    if ((fresh >> i) & (1u << r)) {
+                        if (cur >= 0) {
+                            flush(cur);
+                            done |= 1u << cur;
+                        }
+                        cur = st.o[i + r];
+                        begin(cur);
                     }
+                    add(r);
                 }
             }
             if constexpr (EDGE) {
-                const dev::ff e0 = edge_dot<G>(sv, x[0]), e1 = edge_dot<G>(sv, x[NB - 1]);
                 // both sums at once: one exchange leaves neighbour 0's partials in the low
                 // half-warp and neighbour 1's in the high half, then each half reduces alone
                 const bool lo = lane < 16;
-                dev::ff mine = lo ? e0 : e1, other = lo ? e1 : e0;
+                dev::ff own = lo ? e[0] : e[1], other = lo ? e[1] : e[0];
                 dev::ff recv;
                 recv.hi = __shfl_xor_sync(FULL, other.hi, 16);
                 recv.lo = __shfl_xor_sync(FULL, other.lo, 16);
-                mine = edge_sum2(mine, recv);
+                own = edge_sum2(own, recv);
 #pragma unroll
-                for (int o = 8; o > 0; o >>= 1) {
+                for (int s = 8; s > 0; s >>= 1) {
                     dev::ff y;
-                    y.hi = __shfl_xor_sync(FULL, mine.hi, o);
-                    y.lo = __shfl_xor_sync(FULL, mine.lo, o);
-                    mine = edge_sum2(mine, y);
+                    y.hi = __shfl_xor_sync(FULL, own.hi, s);
+                    y.lo = __shfl_xor_sync(FULL, own.lo, s);
+                    own = edge_sum2(own, y);
                 }
-                if (lane == 0) st.e[idx[0]] = dev::ff_to_double(mine);
-                if (on[NB - 1] && lane == 16) st.e[idx[NB - 1]] = dev::ff_to_double(mine);
+                if (lane == 0) st.e[i] = dev::ff_to_double(own);
+                if (i + 1 < cnt && lane == 16) st.e[i + 1] = dev::ff_to_double(own);
             }
         }
         __syncwarp();
         if constexpr (EDGE) {
-            if (mine) a.edge[j] = eold + st.e[pos];
+            if (mine) a.edge[j] = eold + st.e[at];
         }
     }
+    if (cur >= 0) {
+        flush(cur);
+        done |= 1u << cur;
+    }
     if (!PSI) ovf |= carry != 0;
-}
-
-template <int W> __device__ __forceinline__ Bits<W> nonzero_bits(const unsigned long long (&acc)[2 * W])
-{
-    // the lane's 2W-bit field, shifted into its place in its word, OR-reduced over the 32/W
-    // lanes that share the word, then every word broadcast from its first lane
-    constexpr int G = 2 * W, LPW = 32 / W;  // slots per lane, lanes per word
-    const int lane = threadIdx.x & 31;
-    unsigned f = 0u;
-#pragma unroll
-    for (int k = 0; k < G; ++k) f |= (acc[k] != 0ull ? 1u : 0u) << k;
-    unsigned long long v = (unsigned long long)f << ((G * lane) & 63);
-#pragma unroll
-    for (int o = 1; o < LPW; o <<= 1) v |= __shfl_xor_sync(FULL, v, o);
-    Bits<W> r;
-#pragma unroll
-    for (int q = 0; q < W; ++q) r.w[q] = __shfl_sync(FULL, v, q * LPW);
-    return r;
+    return done;
 }
 
 struct BlockCnt {
@@ -416,128 +514,166 @@ struct BlockCnt {
     unsigned long long mf, dmu;
 };
 
-// Vertex w joined level d+1 for the sources in nb (vold = its visited set before):
-// writes its sigma row and visited set (and F_{d+1} when Fn is given), and counts it.
-// Called by the whole warp with warp-uniform arguments.
-template <int W, bool S32 = false>
-__device__ __forceinline__ void settle(const BArgs &a, int w, const Bits<W> &vold, const Bits<W> &nb,
-                                       const Bits<W> &act, const unsigned long long (&acc)[2 * W],
-                                       unsigned long long *Fn, BlockCnt *bc)
+// Writes the new counts acc of the lane's slots nib of vertex w's sigma row.
+template <int W, bool S32>
+__device__ __forceinline__ void store_sigma(const BArgs &a, int w, unsigned nib, int lane,
+                                            const unsigned long long (&acc)[2 * W])
 {
     constexpr int B = 64 * W;
-    const int lane = threadIdx.x & 31;
     if constexpr (S32) {
         // a count that does not fit 32 bits sends the batch back to the 64-bit kernel
         unsigned *row = a.sp32 + (size_t)w * B;
-        bool wide = false;
+        unsigned wide = 0;
 #pragma unroll
         for (int k = 0; k < 2 * W; ++k)
-            if (has_slot<W>(nb, k, lane)) {
+            if ((nib >> k) & 1u) {
                 row[slot_off<W>(k, lane)] = (unsigned)acc[k];
-                wide |= (acc[k] >> 32) != 0;
+                wide |= (unsigned)(acc[k] >> 32);
             }
         if (wide) atomicCAS(&a.ctrl->err, 0, kErrWide);
     } else {
         unsigned long long *row = a.sp + (size_t)w * B;
 #pragma unroll
         for (int k = 0; k < 2 * W; ++k)
-            if (has_slot<W>(nb, k, lane)) row[slot_off<W>(k, lane)] = acc[k];
-    }
-    bool full = true;
-#pragma unroll
-    for (int q = 0; q < W; ++q) {
-        const unsigned long long nv = vold.w[q] | nb.w[q];
-        full &= nv == act.w[q];
-        if (lane == q) {
-            a.vis[(size_t)w * W + q] = nv;
-            if (Fn) Fn[(size_t)w * W + q] = nb.w[q];
-        }
-    }
-    if (lane == 0) {
-        const unsigned long long dg = (unsigned long long)deg_of(a.rp, w);
-        atomicAdd(&bc->v, 1);
-        atomicAdd(&bc->mf, dg);
-        if (full) atomicAdd(&bc->dmu, dg);
+            if ((nib >> k) & 1u) row[slot_off<W>(k, lane)] = acc[k];
     }
 }
 
-// Calls fn(v) with the whole warp for every vertex of a level: the queued entries
-// queue[qo, qo+nq) or, if qo < 0, every v with Fl[v] != 0 (scanned 32 at a time; nq is
-// then the level's vertex count).
-// Calls fn(v) with the whole warp for every vertex of a level: the queued entries
-// queue[qo, qo+nq) or, if qo < 0, every v with Fl[v] != 0 (scanned 32 at a time; nq is
-// then the level's vertex count).  Warps
-// take work dynamically from the zeroed counter *ctr (8 entries or 64 vertices at a
-// time), so that power-law degrees do not leave a few warps finishing long after the
-// rest.
-template <int W, class Fn>
-__device__ __forceinline__ void for_level(const BArgs &a, int qo, int nq,
-                                          const unsigned long long *Fl, int32_t *ctr, Fn fn)
+template <int W> __device__ __forceinline__ void store_bits(unsigned long long *p, const Bits<W> &b)
+{
+    if constexpr (W == 1) {
+        *p = b.w[0];
+    } else {
+#pragma unroll
+        for (int q = 0; q < W; q += 2) *reinterpret_cast<ulonglong2 *>(p + q) = make_ulonglong2(b.w[q], b.w[q + 1]);
+    }
+}
+
+// Lane L's vertex w (where `on`) joined level d+1 for the sources nb: writes its visited set
+// and F_{d+1}, and counts the warp's vertices in the block's counters.
+template <int W>
+__device__ __forceinline__ void join_level(const BArgs &a, bool on, int w, int dg, const Bits<W> &nb,
+                                           const Bits<W> &act, unsigned long long *Fn, BlockCnt *bc)
+{
+    bool full = on;
+    if (on) {
+        Bits<W> nv = load_bits<W>(a.vis + (size_t)w * W);
+#pragma unroll
+        for (int q = 0; q < W; ++q) {
+            nv.w[q] |= nb.w[q];
+            full &= nv.w[q] == act.w[q];
+        }
+        store_bits<W>(a.vis + (size_t)w * W, nv);
+        store_bits<W>(Fn + (size_t)w * W, nb);
+    }
+    const unsigned m = __ballot_sync(FULL, on);
+    const unsigned df = __reduce_add_sync(FULL, on ? (unsigned)dg : 0u);
+    const unsigned dd = __reduce_add_sync(FULL, full ? (unsigned)dg : 0u);
+    if ((threadIdx.x & 31) == 0 && m) {
+        atomicAdd(&bc->v, __popc(m));
+        atomicAdd(&bc->mf, (unsigned long long)df);
+        if (dd) atomicAdd(&bc->dmu, (unsigned long long)dd);
+    }
+}
+
+// Vertices a warp takes at a time (a power of two up to the 32 lanes) of the n of a phase: about
+// kGrabArcs arcs by the graph's average, and at most 1/kGrabShare of the warp's share.  Always 32
+// vertices left most warps idle on small graphs (63 of 4864 worked on ER 2000: a launch of 64
+// sources 680 us, now 200) and made long tails on others: BA 10^6 (16 arcs a vertex), 128 sources,
+// 128 arcs a grab 34.1 ms, 256 33.7, 512 42.6; R-MAT 24 (31) 398, 372, 361 (the counter's atomics).
+__device__ __forceinline__ int grab_size(const BArgs &a, int n, int nw)
+{
+    const int by_arcs = (int)((long long)a.n * kGrabArcs / max((long long)a.A, 1ll));
+    const int most = min(by_arcs, n / (kGrabShare * nw));
+    return most >= kGrabV ? kGrabV : most <= 1 ? 1 : 1 << (31 - __clz(most));
+}
+
+// How a phase finds its vertices: entries [qo, qo + nq) of the queue, or a scan of all
+// vertices (the callee looks at their bits).  nq: the number of vertices expected.
+struct Level {
+    int qo;   // -1: scan
+    int nq;
+};
+
+// Calls fn(on, v, beg, dg, chunk) with the whole warp for all work of a phase.  First the
+// chunks of the heavy vertices, whose work is largest (chunk >= 0: lane 0 holds the vertex and
+// the chunk's arcs), then groups of light vertices, one per lane (chunk = -1).  Warps take work
+// dynamically from the two zeroed counters, each grab requested while the one before is worked
+// on; scans of sparse levels (under n/32 vertices) are static.  Loops are bounded in time: lane
+// 0 checks the phase's deadline (kept in shared memory) once per item and the warp leaves together (the status is read
+// at the next barrier).
+template <class Fn>
+__device__ __forceinline__ void for_work(const BArgs &a, Level lv, int32_t *ctr, int32_t *ctr_c,
+                                         unsigned long long &deadline, Fn fn)
 {
     const int lane = threadIdx.x & 31;
-    // every loop below is also bounded in time: lane 0 checks the phase deadline once per
-    // grab or tile and the warp leaves together (the status is read at the next barrier)
-    const uint64_t deadline = dev::globaltimer() + a.limit_ns;
-    auto expired = [&]() {
-        int e = 0;
-        if (lane == 0 && dev::globaltimer() > deadline) {
-            check_failed(a, NK_ERR_TIMEOUT, 2, nq);
-            e = 1;
+    const int nw = (int)(((long long)gridDim.x * blockDim.x) >> 5);
+    if (lane == 0) deadline = dev::globaltimer() + a.limit_ns;
+    // about C / (32 warps) chunks per grab, 1..16: few chunks stay spread over many warps,
+    // millions of chunks cost few atomics
+    const int gc = max(1, min(kGrabCMax, a.C / (32 * nw)));
+    const bool fixed = lv.qo < 0 && lv.nq < a.n / 32;
+    const int gv = fixed ? kGrabV : grab_size(a, lv.qo >= 0 ? lv.nq : a.n, nw);
+    const int step = fixed ? nw * kGrabV : 0;
+    const unsigned end = lv.qo >= 0 ? lv.nq : a.n;
+    int c = 0, cend = 0;
+    unsigned next = 0;  // lane 0: the grab under way
+    bool chunks = a.C > 0;
+    auto grab = [&]() {
+        if (lane == 0) {
+            if (chunks) next = (unsigned)atomicAdd(ctr_c, gc);
+            else next = step ? next + step : (unsigned)atomicAdd(ctr, gv);
         }
-        return __shfl_sync(FULL, e, 0) != 0;
     };
-    if (qo >= 0) {
-        // up to kGrabQ entries per grab, fewer when the level is short (level 0, deep
-        // levels), so that its entries spread over many warps
-        const long long nwq = ((long long)gridDim.x * blockDim.x) >> 5;
-        const int gq = (int)max(1LL, min((long long)kGrabQ, (long long)nq / nwq));
-        for (;;) {
-            int i0 = 0;
-            if (lane == 0) i0 = atomicAdd(ctr, gq);
-            i0 = __shfl_sync(FULL, i0, 0);
-            if (i0 >= nq || expired()) break;
-            const int i1 = min(i0 + gq, nq);
-            for (int i = i0; i < i1; ++i) {
-                const int v = __ldcg(a.queue + qo + i);
-                if ((unsigned)v >= (unsigned)a.n) {  // warp-uniform
-                    if (lane == 0) check_failed(a, kErrCheck, 3, v);
+    auto first = [&]() {  // of the scan
+        if (lane == 0) next = step ? (unsigned)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kGrabV
+                                   : (unsigned)atomicAdd(ctr, gv);
+    };
+    if (chunks) grab();
+    else first();
+    for (;;) {
+        bool on = false;
+        int v = 0, beg = 0, dg = 0, chunk = -1;
+        if (chunks) {
+            if (c >= cend) {
+                c = __shfl_sync(FULL, (int)next, 0);
+                if (c >= a.C) {
+                    chunks = false;
+                    first();
                     continue;
                 }
-                fn(v);
+                cend = min(c + gc, a.C);
+                grab();
+            }
+            const int i = __ldg(a.chunk_h + c);
+            v = __ldg(a.hv + i);
+            beg = __ldg(a.rp + v) + (c - __ldg(a.hfirst + i)) * a.chunk;
+            dg = min(a.chunk, __ldg(a.rp + v + 1) - beg);
+            on = lane == 0;
+            chunk = c++;
+        } else {
+            const unsigned i = __shfl_sync(FULL, next, 0) + lane;
+            if (i - lane >= end) break;
+            grab();
+            on = lane < gv && i < end;
+            if (on) v = lv.qo >= 0 ? __ldcg(a.queue + lv.qo + i) : (int)i;
+            if (on && (unsigned)v >= (unsigned)a.n) {
+                check_failed(a, kErrCheck, 3, v);
+                on = false;
+            }
+            if (on) {
+                beg = __ldg(a.rp + v);
+                dg = __ldg(a.rp + v + 1) - beg;
+                on = dg > 0 && dg <= a.chunk;
             }
         }
-    } else if ((long long)nq * 32 < a.n) {
-        // a sparse level (fewer than n/32 vertices): a static scan, no counter traffic
-        const long long wid = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-        const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
-        for (long long base = wid * 32; base < a.n; base += nw * 32) {
-            if (expired()) break;
-            const long long v = base + lane;
-            const bool nz = v < a.n && any_bits<W>(load_bits<W>(Fl + (size_t)v * W));
-            unsigned m = __ballot_sync(FULL, nz);
-            while (m) {
-                const int t = __ffs(m) - 1;
-                m &= m - 1;
-                fn((int)(base + t));
-            }
+        int late = 0;
+        if (lane == 0 && dev::globaltimer() > deadline) {
+            check_failed(a, NK_ERR_TIMEOUT, 2, lv.nq);
+            late = 1;
         }
-    } else {
-        for (;;) {
-            int t0 = 0;
-            if (lane == 0) t0 = atomicAdd(ctr, kGrabV);
-            t0 = __shfl_sync(FULL, t0, 0);
-            if (t0 >= a.n || expired()) break;
-            for (int base = t0; base < min(t0 + kGrabV, a.n); base += 32) {
-                const int v = base + lane;
-                const bool nz = v < a.n && any_bits<W>(load_bits<W>(Fl + (size_t)v * W));
-                unsigned m = __ballot_sync(FULL, nz);
-                while (m) {
-                    const int t = __ffs(m) - 1;
-                    m &= m - 1;
-                    fn(base + t);
-                }
-            }
-        }
+        if (__shfl_sync(FULL, late, 0)) break;
+        fn(on, v, beg, dg, chunk);
     }
 }
 
@@ -551,38 +687,6 @@ __device__ __forceinline__ void trace_mark(const BArgs &a, int &ti, int level, i
         a.trace[2 * ti] = (unsigned long long)(level * 16 + phase);
         a.trace[2 * ti + 1] = dev::globaltimer();
         ++ti;
-    }
-}
-
-// Work on the chunks of heavy vertices: fn(c, h, j0, j1) per chunk, with the whole warp;
-// chunks are taken dynamically from the zeroed counter *ctr, and the loop is bounded in
-// time like the others.
-template <class Fn> __device__ __forceinline__ void for_chunks(const BArgs &a, int32_t *ctr, Fn fn)
-{
-    const int lane = threadIdx.x & 31;
-    const uint64_t deadline = dev::globaltimer() + a.limit_ns;
-    // grab about C / (32 warps) chunks, 1..16: few chunks stay spread over many warps,
-    // millions of chunks cost few atomics
-    const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
-    const int gc = (int)max(1LL, min((long long)kGrabCMax, (long long)a.C / (32 * nw)));
-    for (;;) {
-        int c0 = 0;
-        if (lane == 0) {
-            c0 = atomicAdd(ctr, gc);
-            if (c0 < a.C && dev::globaltimer() > deadline) {
-                check_failed(a, NK_ERR_TIMEOUT, 4, c0);
-                c0 = a.C;
-            }
-        }
-        c0 = __shfl_sync(FULL, c0, 0);
-        if (c0 >= a.C) break;
-        for (int c = c0; c < min(c0 + gc, a.C); ++c) {
-            const int i = __ldg(a.chunk_h + c);
-            const int h = __ldg(a.hv + i);
-            const int j0 = __ldg(a.rp + h) + (c - __ldg(a.hfirst + i)) * a.chunk;
-            const int j1 = min(j0 + a.chunk, __ldg(a.rp + h + 1));
-            fn(c, h, j0, j1);
-        }
     }
 }
 
@@ -603,7 +707,30 @@ __device__ __forceinline__ void store_part(const BArgs &a, int c, const unsigned
     for (int k = 0; k < 2 * W; ++k) row[slot_off<W>(k, threadIdx.x & 31)] = acc[k];
 }
 
-__device__ __forceinline__ bool heavy(const BArgs &a, int v) { return deg_of(a.rp, v) > a.chunk; }
+// Sums of a heavy vertex's chunks [c0, c1) in chunk order, four loads in flight at a time.
+template <int W, class Add> __device__ __forceinline__ void sum_parts(const BArgs &a, int c0, int c1, Add add)
+{
+    const unsigned long long *p = a.part + (size_t)c0 * (64 * W) + slot_off<W>(0, threadIdx.x & 31);
+    constexpr int U = W == 1 ? 4 : 2;
+    int c = c0;
+    for (; c + U <= c1; c += U, p += U * 64 * W) {
+        ulonglong2 y[U][W];
+#pragma unroll
+        for (int r = 0; r < U; ++r)
+#pragma unroll
+            for (int h = 0; h < W; ++h) y[r][h] = __ldcg(reinterpret_cast<const ulonglong2 *>(p + r * 64 * W) + h);
+#pragma unroll
+        for (int r = 0; r < U; ++r)
+#pragma unroll
+            for (int h = 0; h < W; ++h) {
+                add(2 * h, y[r][h].x);
+                add(2 * h + 1, y[r][h].y);
+            }
+    }
+    for (; c < c1; ++c, p += 64 * W)
+#pragma unroll
+        for (int k = 0; k < 2 * W; ++k) add(k, __ldcg(p + k));
+}
 
 // CTAs per SM that the launch bounds ask for: 4 for 64 and 128 sources (64 registers), 3 for
 // the 128-source edge sweep (its per-arc shares need 80 registers, which 64 would spill), 2
@@ -616,7 +743,7 @@ __global__ void __launch_bounds__(kThreads, min_ctas<W, EDGE>()) k_batch(BArgs a
     constexpr int B = 64 * W;
     __shared__ BlockCnt bc;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    Nbrs<W> &st = reinterpret_cast<Nbrs<W> *>(smem_raw)[threadIdx.x >> 5];
+    WarpBuf<W, EDGE> &st = reinterpret_cast<WarpBuf<W, EDGE> *>(smem_raw)[threadIdx.x >> 5];
     const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long nthr = (long long)gridDim.x * blockDim.x;
     const int lane = threadIdx.x & 31;
@@ -704,88 +831,49 @@ __global__ void __launch_bounds__(kThreads, min_ctas<W, EDGE>()) k_batch(BArgs a
                             (a.dir == NK_DIR_AUTO && a.alpha * (double)mf > (double)mu);
         bool queued = false;
         int nq1 = 0;
-        if (use_bu) {
-            // ---- bottom-up (a): light vertices with unvisited sources pull from level d;
-            //      chunks of heavy vertices store partial sums
-            const uint64_t bu_deadline = dev::globaltimer() + a.limit_ns;
-            for (int t0 = 0;;) {
-                if (lane == 0) {
-                    t0 = atomicAdd(a.wq + (size_t)d * 8 + WQ_BU, 32);
-                    if (t0 < a.n && dev::globaltimer() > bu_deadline) {
-                        check_failed(a, NK_ERR_TIMEOUT, 5, t0);
-                        t0 = a.n;
+        int32_t *wq = a.wq + (size_t)d * 8;
+        if (!use_bu) {
+            // ---- top-down (a): push the frontier's bits, queue each new vertex once; lanes over
+            //      the concatenated arcs of a group of frontier vertices, or of a heavy one's chunk
+            for_work(a, {qo, nq}, wq + WQ_PUSH, wq + WQ_PUSH_C, st.until, [&](bool on, int v, int beg, int dg, int) {
+                Bits<W> t;
+                if (on) {
+                    t = load_bits<W>(Fd + (size_t)v * W);
+                    on = any_bits<W>(t);
+                }
+                const int d0 = on ? dg : 0;
+                int incl = d0;
+#pragma unroll
+                for (int s = 1; s < 32; s <<= 1) {
+                    const int y = __shfl_up_sync(FULL, incl, s);
+                    if (lane >= s) incl += y;
+                }
+                const int total = __shfl_sync(FULL, incl, 31), pre = incl - d0;
+                const unsigned members = __ballot_sync(FULL, d0 > 0);
+                __syncwarp();
+                if (d0 > 0) {
+                    const int pos = __popc(members & dev::lanemask_lt());
+                    st.off[pos] = beg - pre;
+#pragma unroll
+                    for (int q = 0; q < W; ++q) st.t[pos][q] = t.w[q];
+                }
+                __syncwarp();
+                int before = 0;
+                for (int base = 0; base < total; base += 32) {
+                    const unsigned marks = __reduce_or_sync(FULL, d0 > 0 && (unsigned)(pre - base) < 32u ? 1u << (pre - base) : 0u);
+                    const int o = before + __popc(marks & (dev::lanemask_lt() << 1 | 1u)) - 1;
+                    before += __popc(marks);
+                    if (base + lane >= total) continue;
+                    const int c = __ldg(a.col + st.off[o] + base + lane);
+                    const Bits<W> vc = load_bits<W>(a.vis + (size_t)c * W);
+                    bool any = false;
+#pragma unroll
+                    for (int q = 0; q < W; ++q) {
+                        const unsigned long long m = st.t[o][q] & ~vc.w[q];
+                        any |= m != 0;
+                        if (m) atomicOr(Fn + (size_t)c * W + q, m);
                     }
-                }
-                t0 = __shfl_sync(FULL, t0, 0);
-                if (t0 >= a.n) break;
-                const long long base = t0;
-                const long long v = base + lane;
-                Bits<W> vv = act;
-                if (v < a.n && !heavy(a, (int)v)) vv = load_bits<W>(a.vis + (size_t)v * W);
-                unsigned m = __ballot_sync(FULL, any_bits<W>(andnot<W>(act, vv)));
-                while (m) {
-                    const int t = __ffs(m) - 1;
-                    m &= m - 1;
-                    const int w = (int)(base + t);
-                    const Bits<W> vold = shfl_bits<W>(vv, t);
-                    const Bits<W> u = andnot<W>(act, vold);
-                    unsigned long long acc[2 * W];
-                    dev::ff facc[2 * W];
-#pragma unroll
-                    for (int k = 0; k < 2 * W; ++k) acc[k] = 0;
-                    gather<W, false, false, S32>(a, __ldg(a.rp + w), __ldg(a.rp + w + 1), Fd, u, acc, facc, ovf, st);
-                    const Bits<W> nb = nonzero_bits<W>(acc);
-                    if (any_bits<W>(nb)) settle<W, S32>(a, w, vold, nb, act, acc, Fn, &bc);
-                }
-            }
-            for_chunks(a, a.wq + (size_t)d * 8 + WQ_BU_C, [&](int c, int h, int j0, int j1) {
-                const Bits<W> u = andnot<W>(act, load_bits<W>(a.vis + (size_t)h * W));
-                if (!any_bits<W>(u)) return;
-                unsigned long long acc[2 * W];
-                dev::ff facc[2 * W];
-#pragma unroll
-                for (int k = 0; k < 2 * W; ++k) acc[k] = 0;
-                gather<W, false, false, S32>(a, j0, j1, Fd, u, acc, facc, ovf, st);
-                store_part<W>(a, c, acc);
-            });
-            if (a.H > 0 && !dev::grid_barrier(a.ctrl, a.limit_ns)) return;
-            trace_mark(a, ti, d, PH_BU_A);
-            // ---- bottom-up (b): heavy vertices sum their chunks in chunk order
-            for_heavy(a, [&](int i, int h, int c0, int c1) {
-                const Bits<W> vold = load_bits<W>(a.vis + (size_t)h * W);
-                if (!any_bits<W>(andnot<W>(act, vold))) return;
-                unsigned long long acc[2 * W];
-#pragma unroll
-                for (int k = 0; k < 2 * W; ++k) acc[k] = 0;
-                for (int c = c0; c < c1; ++c) {
-                    const unsigned long long *row = a.part + (size_t)c * B;
-#pragma unroll
-                    for (int k = 0; k < 2 * W; ++k) {
-                        const unsigned long long y = acc[k] + __ldcg(row + slot_off<W>(k, lane));
-                        ovf |= y < acc[k];
-                        acc[k] = y;
-                    }
-                }
-                const Bits<W> nb = nonzero_bits<W>(acc);
-                if (any_bits<W>(nb)) settle<W, S32>(a, h, vold, nb, act, acc, Fn, &bc);
-            });
-            flush_counts(d + 1);
-            if (tid == 0) a.qoff[d + 1] = -1;
-            if (!dev::grid_barrier(a.ctrl, a.limit_ns)) return;
-            trace_mark(a, ti, d, PH_BU_B);
-        } else {
-            // ---- top-down (a): push the frontier's bits, queue each new vertex once;
-            //      heavy frontier vertices push chunk by chunk
-            auto push = [&](int v, int j0, int j1) {
-                const Bits<W> f = load_bits<W>(Fd + (size_t)v * W);
-                for (int j = j0 + lane; j < j1; j += 32) {
-                    const int c = __ldg(a.col + j);
-                    const Bits<W> m = andnot<W>(f, load_bits<W>(a.vis + (size_t)c * W));
-                    if (!any_bits<W>(m)) continue;
-#pragma unroll
-                    for (int q = 0; q < W; ++q)
-                        if (m.w[q]) atomicOr(Fn + (size_t)c * W + q, m.w[q]);
-                    if (__ldcg(a.qmark + c) != d + 1 && atomicExch(a.qmark + c, d + 1) != d + 1) {
+                    if (any && __ldcg(a.qmark + c) != d + 1 && atomicExch(a.qmark + c, d + 1) != d + 1) {
                         cg::coalesced_group g = cg::coalesced_threads();
                         int pos = 0;
                         if (g.thread_rank() == 0) pos = atomicAdd(a.qcnt + d + 1, (int)g.size());
@@ -793,66 +881,85 @@ __global__ void __launch_bounds__(kThreads, min_ctas<W, EDGE>()) k_batch(BArgs a
                         if (qtail + pos < a.qcap) a.queue[qtail + pos] = c;
                     }
                 }
-            };
-            for_level<W>(a, qo, nq, Fd, a.wq + (size_t)d * 8 + WQ_PUSH, [&](int v) {
-                if (heavy(a, v)) return;
-                push(v, __ldg(a.rp + v), __ldg(a.rp + v + 1));
-            });
-            for_chunks(a, a.wq + (size_t)d * 8 + WQ_PUSH_C, [&](int c, int h, int j0, int j1) {
-                if (any_bits<W>(load_bits<W>(Fd + (size_t)h * W))) push(h, j0, j1);
             });
             if (!dev::grid_barrier(a.ctrl, a.limit_ns)) return;
             trace_mark(a, ti, d, PH_TD_A);
-            // ---- top-down (b): every new vertex pulls sigma for its new bits
             nq1 = __ldcg(a.qcnt + d + 1);
             queued = qtail + nq1 <= a.qcap;
-            for_level<W>(a, queued ? (int)qtail : -1, nq1, Fn, a.wq + (size_t)d * 8 + WQ_PULL, [&](int w) {
-                if (heavy(a, w)) return;
-                const Bits<W> t = load_bits<W>(Fn + (size_t)w * W);
-                const Bits<W> vold = load_bits<W>(a.vis + (size_t)w * W);
-                unsigned long long acc[2 * W];
-                dev::ff facc[2 * W];
-#pragma unroll
-                for (int k = 0; k < 2 * W; ++k) acc[k] = 0;
-                gather<W, false, false, S32>(a, __ldg(a.rp + w), __ldg(a.rp + w + 1), Fd, t, acc, facc, ovf, st);
-                settle<W, S32>(a, w, vold, t, act, acc, nullptr, &bc);
-            });
-            for_chunks(a, a.wq + (size_t)d * 8 + WQ_PULL_C, [&](int c, int h, int j0, int j1) {
-                const Bits<W> t = load_bits<W>(Fn + (size_t)h * W);
-                if (!any_bits<W>(t)) return;
-                unsigned long long acc[2 * W];
-                dev::ff facc[2 * W];
-#pragma unroll
-                for (int k = 0; k < 2 * W; ++k) acc[k] = 0;
-                gather<W, false, false, S32>(a, j0, j1, Fd, t, acc, facc, ovf, st);
-                store_part<W>(a, c, acc);
-            });
-            if (a.H > 0 && !dev::grid_barrier(a.ctrl, a.limit_ns)) return;
-            trace_mark(a, ti, d, PH_TD_B);
-            // ---- top-down (c): heavy new vertices sum their chunks in chunk order
-            for_heavy(a, [&](int i, int h, int c0, int c1) {
-                const Bits<W> t = load_bits<W>(Fn + (size_t)h * W);
-                if (!any_bits<W>(t)) return;
-                const Bits<W> vold = load_bits<W>(a.vis + (size_t)h * W);
-                unsigned long long acc[2 * W];
-#pragma unroll
-                for (int k = 0; k < 2 * W; ++k) acc[k] = 0;
-                for (int c = c0; c < c1; ++c) {
-                    const unsigned long long *row = a.part + (size_t)c * B;
-#pragma unroll
-                    for (int k = 0; k < 2 * W; ++k) {
-                        const unsigned long long y = acc[k] + __ldcg(row + slot_off<W>(k, lane));
-                        ovf |= y < acc[k];
-                        acc[k] = y;
-                    }
-                }
-                settle<W, S32>(a, h, vold, t, act, acc, nullptr, &bc);
-            });
-            flush_counts(d + 1);
-            if (tid == 0) a.qoff[d + 1] = queued ? (int)qtail : -1;
-            if (!dev::grid_barrier(a.ctrl, a.limit_ns)) return;
-            trace_mark(a, ti, d, PH_TD_C);
         }
+        // ---- pull sigma from level d: bottom-up every vertex with unvisited sources, for all of
+        //      them; top-down (b) every new vertex for its new bits.  Chunks of heavy vertices
+        //      store partial sums.
+        const Level pull = use_bu ? Level{-1, a.n} : Level{queued ? (int)qtail : -1, nq1};
+        for_work(a, pull, wq + (use_bu ? WQ_BU : WQ_PULL), wq + (use_bu ? WQ_BU_C : WQ_PULL_C), st.until,
+                 [&](bool on, int v, int beg, int dg, int chunk) {
+            Bits<W> t;
+            if (on) {
+                t = load_bits<W>((use_bu ? (const unsigned long long *)a.vis : Fn) + (size_t)v * W);
+                if (use_bu) t = andnot<W>(act, t);
+                on = any_bits<W>(t);
+            }
+            if (!__any_sync(FULL, on)) return;
+            unsigned long long acc[2 * W];
+            dev::ff facc[2 * W];
+#pragma unroll
+            for (int k = 0; k < 2 * W; ++k) acc[k] = 0;
+            int pos;
+            const unsigned done = gather<W, false, false, S32>(
+                a, on, v, beg, dg, t, Fd, st, acc, facc, facc, ovf, pos, [](int) {},
+                [&](int o) {
+                    if (chunk >= 0) return;  // stored below
+                    unsigned nib = 0;
+#pragma unroll
+                    for (int k = 0; k < 2 * W; ++k) nib |= (acc[k] != 0ull ? 1u : 0u) << k;
+                    store_sigma<W, S32>(a, st.v[o], nib, lane, acc);
+                    store_lane_bits<W>(st.t[o], nib, lane);
+#pragma unroll
+                    for (int k = 0; k < 2 * W; ++k) acc[k] = 0;
+                });
+            if (chunk >= 0) {
+                store_part<W>(a, chunk, acc);
+                return;
+            }
+            __syncwarp();
+            Bits<W> nb;
+#pragma unroll
+            for (int q = 0; q < W; ++q) nb.w[q] = 0;
+            if (pos >= 0 && ((done >> pos) & 1u))
+#pragma unroll
+                for (int q = 0; q < W; ++q) nb.w[q] = st.t[pos][q];
+            join_level<W>(a, any_bits<W>(nb), v, dg, nb, act, Fn, &bc);
+        });
+        if (a.H > 0 && !dev::grid_barrier(a.ctrl, a.limit_ns)) return;
+        trace_mark(a, ti, d, use_bu ? PH_BU_A : PH_TD_B);
+        // ---- heavy vertices sum their chunks in chunk order
+        for_heavy(a, [&](int i, int h, int c0, int c1) {
+            const Bits<W> t = use_bu ? andnot<W>(act, load_bits<W>(a.vis + (size_t)h * W)) : load_bits<W>(Fn + (size_t)h * W);
+            if (!any_bits<W>(t)) return;
+            unsigned long long acc[2 * W];
+#pragma unroll
+            for (int k = 0; k < 2 * W; ++k) acc[k] = 0;
+            sum_parts<W>(a, c0, c1, [&](int k, unsigned long long x) {
+                const unsigned long long y = acc[k] + x;
+                ovf |= y < x;
+                acc[k] = y;
+            });
+            unsigned nib = 0;
+#pragma unroll
+            for (int k = 0; k < 2 * W; ++k) nib |= (acc[k] != 0ull ? 1u : 0u) << k;
+            store_sigma<W, S32>(a, h, nib, lane, acc);
+            __syncwarp();
+            store_lane_bits<W>(st.t[0], nib, lane);
+            __syncwarp();
+            Bits<W> nb;
+#pragma unroll
+            for (int q = 0; q < W; ++q) nb.w[q] = st.t[0][q];
+            join_level<W>(a, lane == 0 && any_bits<W>(nb), h, deg_of(a.rp, h), nb, act, Fn, &bc);
+        });
+        flush_counts(d + 1);
+        if (tid == 0) a.qoff[d + 1] = queued ? (int)qtail : -1;
+        if (!dev::grid_barrier(a.ctrl, a.limit_ns)) return;
+        trace_mark(a, ti, d, use_bu ? PH_BU_B : PH_TD_C);
         const int c = __ldcg(a.vcnt + d + 1);
         if (use_bu) {
             ++bu;
@@ -968,75 +1075,91 @@ __global__ void __launch_bounds__(kThreads, min_ctas<W, EDGE>()) k_batch(BArgs a
         const unsigned long long *Fs = a.F + (size_t)(l + 1) * slab;
         const int ql = __ldcg(a.qoff + l);
         const int nl = ql >= 0 ? __ldcg(a.qcnt + l) : __ldcg(a.vcnt + l);
-        // delta/psi/score of vertex v from its successor sums facc (whole warp)
-        // psi_v = 1/sigma_v + acc and delta_v = sigma_v * acc (Brandes' recurrence with
-        // sigma_v factored out), in double-single; the vertex's delta summed over its
-        // source slots goes to the FP64 score once per vertex and level
-        auto finish = [&](int v, const Bits<W> &mv, const dev::ff (&facc)[2 * W]) {
+        // delta/psi/score of vertex v from its successor sums facc (whole warp; the lane's slots
+        // nib, its path counts sg): psi_v = 1/sigma_v + acc and delta_v = sigma_v * acc (Brandes'
+        // recurrence with sigma_v factored out), in double-single; the vertex's delta summed over
+        // its source slots goes to the FP64 score once per vertex and level.  One warp adds to a
+        // vertex's score per level, so the atomic addition, which returns nothing and is not
+        // waited for, keeps the order of the additions.
+        auto finish = [&](int v, unsigned nib, const RowPart<W, S32> &sg, const dev::ff (&facc)[2 * W]) {
             dev::ff part = dev::ff_zero();
             unsigned long long *row = a.sp + (size_t)v * B;
 #pragma unroll
             for (int k = 0; k < 2 * W; ++k) {
-                if (has_slot<W>(mv, k, lane)) {
-                    const unsigned long long sg = S32 ? (unsigned long long)__ldcg(a.sp32 + (size_t)v * B + slot_off<W>(k, lane))
-                                                      : __ldcg(row + slot_off<W>(k, lane));
-                    const dev::ff sv = dev::ff_from_u64(sg);
-                    const dev::ff delta = dev::ff_mul(sv, facc[k]);
-                    row[slot_off<W>(k, lane)] = dev::ff_pack(dev::ff_add(dev::ff_rcp(sv), facc[k]));
-                    part = dev::ff_add(part, delta);
+                if ((nib >> k) & 1u) {
+                    const dev::ff s = sg.count(k);
+                    row[slot_off<W>(k, lane)] = dev::ff_pack(dev::ff_add(dev::ff_rcp(s), facc[k]));
+                    part = dev::ff_add(part, dev::ff_mul(s, facc[k]));
                 }
             }
             part = dev::group_sum_ff<32>(part);
-            if (lane == 0 && part.hi != 0.0f && l > 0) a.scores[v] += dev::ff_to_double(part);
+            if (lane == 0 && part.hi != 0.0f && l > 0) atomicAdd(a.scores + v, dev::ff_to_double(part));
         };
-        // sigma_b(v) of the lane's slots in mv (edge betweenness only), read before psi
-        // replaces it
-        auto sigma_row = [&](int v, const Bits<W> &mv, dev::ff (&sv)[2 * W]) {
-            const unsigned long long *row = a.sp + (size_t)v * B;
-#pragma unroll
-            for (int k = 0; k < 2 * W; ++k)
-                sv[k] = has_slot<W>(mv, k, lane) ? dev::ff_from_u64(__ldcg(row + slot_off<W>(k, lane))) : dev::ff_zero();
-        };
-        for_level<W>(a, ql, nl, Fl, a.wq + (size_t)l * 8 + WQ_BACK, [&](int v) {
-            if (heavy(a, v)) return;
-            const Bits<W> mv = load_bits<W>(Fl + (size_t)v * W);
+        for_work(a, {ql, nl}, a.wq + (size_t)l * 8 + WQ_BACK, a.wq + (size_t)l * 8 + WQ_BACK_C, st.until,
+                 [&](bool on, int v, int beg, int dg, int chunk) {
+            Bits<W> t;
+            if (on) {
+                t = load_bits<W>(Fl + (size_t)v * W);
+                on = any_bits<W>(t);
+            }
+            const unsigned members = __ballot_sync(FULL, on);
+            if (!members) return;
             unsigned long long acc[2 * W];
             dev::ff facc[2 * W], sv[2 * W];
+            RowPart<W, S32> sg;
 #pragma unroll
             for (int k = 0; k < 2 * W; ++k) facc[k] = dev::ff_zero();
-            if constexpr (EDGE) sigma_row(v, mv, sv);
             bool dummy = false;
-            gather<W, true, EDGE>(a, __ldg(a.rp + v), __ldg(a.rp + v + 1), Fs, mv, acc, facc, dummy, st, sv);
-            finish(v, mv, facc);
-        });
-        for_chunks(a, a.wq + (size_t)l * 8 + WQ_BACK_C, [&](int c, int h, int j0, int j1) {
-            const Bits<W> mv = load_bits<W>(Fl + (size_t)h * W);
-            if (!any_bits<W>(mv)) return;
-            unsigned long long acc[2 * W];
-            dev::ff facc[2 * W], sv[2 * W];
+            int pos;
+            const unsigned done = gather<W, true, EDGE, false>(
+                a, on, v, beg, dg, t, Fs, st, acc, facc, sv, dummy, pos,
+                [&](int o) {
+                    if (!EDGE && chunk >= 0) return;
+                    const unsigned nib = lane_bits<W>(st.t[o], lane);
+                    sg.load(a, st.v[o], lane, nib);  // in flight while the vertex's rows are gathered
+                    if constexpr (EDGE) {
 #pragma unroll
-            for (int k = 0; k < 2 * W; ++k) facc[k] = dev::ff_zero();
-            if constexpr (EDGE) sigma_row(h, mv, sv);
-            bool dummy = false;
-            gather<W, true, EDGE>(a, j0, j1, Fs, mv, acc, facc, dummy, st, sv);
+                        for (int k = 0; k < 2 * W; ++k) sv[k] = (nib >> k) & 1u ? sg.count(k) : dev::ff_zero();
+                    }
+                },
+                [&](int o) {
+                    if (chunk >= 0) return;  // stored below
+                    finish(st.v[o], lane_bits<W>(st.t[o], lane), sg, facc);
 #pragma unroll
-            for (int k = 0; k < 2 * W; ++k) acc[k] = dev::ff_pack(facc[k]);
-            store_part<W>(a, c, acc);
+                    for (int k = 0; k < 2 * W; ++k) facc[k] = dev::ff_zero();
+                });
+            if (chunk >= 0) {
+#pragma unroll
+                for (int k = 0; k < 2 * W; ++k) acc[k] = dev::ff_pack(facc[k]);
+                store_part<W>(a, chunk, acc);
+                return;
+            }
+            // vertices without successors: psi = 1 / sigma
+            unsigned rest = ((2u << (__popc(members) - 1)) - 1u) & ~done;
+            while (rest) {
+                const int o = __ffs(rest) - 1;
+                rest &= rest - 1;
+                const unsigned nib = lane_bits<W>(st.t[o], lane);
+                unsigned long long *row = a.sp + (size_t)st.v[o] * B;
+                sg.load(a, st.v[o], lane, nib);
+#pragma unroll
+                for (int k = 0; k < 2 * W; ++k)
+                    if ((nib >> k) & 1u) row[slot_off<W>(k, lane)] = dev::ff_pack(dev::ff_rcp(sg.count(k)));
+            }
         });
         if (a.H > 0 && !dev::grid_barrier(a.ctrl, a.limit_ns)) return;
         trace_mark(a, ti, l, PH_BK_A);
         for_heavy(a, [&](int i, int h, int c0, int c1) {
             const Bits<W> mv = load_bits<W>(Fl + (size_t)h * W);
             if (!any_bits<W>(mv)) return;
+            const unsigned nib = (unsigned)(lane_word<W>(mv, lane) >> ((2 * W * lane) & 63)) & ((1u << (2 * W)) - 1u);
+            RowPart<W, S32> sg;
+            sg.load(a, h, lane, nib);
             dev::ff facc[2 * W];
 #pragma unroll
             for (int k = 0; k < 2 * W; ++k) facc[k] = dev::ff_zero();
-            for (int c = c0; c < c1; ++c) {
-                const unsigned long long *row = a.part + (size_t)c * B;
-#pragma unroll
-                for (int k = 0; k < 2 * W; ++k) facc[k] = dev::ff_add(facc[k], dev::ff_unpack(__ldcg(row + slot_off<W>(k, lane))));
-            }
-            finish(h, mv, facc);
+            sum_parts<W>(a, c0, c1, [&](int k, unsigned long long x) { facc[k] = dev::ff_add(facc[k], dev::ff_unpack(x)); });
+            finish(h, nib, sg, facc);
         });
         if (!dev::grid_barrier(a.ctrl, a.limit_ns)) return;
         trace_mark(a, ti, l, PH_BK_B);
@@ -1045,7 +1168,7 @@ __global__ void __launch_bounds__(kThreads, min_ctas<W, EDGE>()) k_batch(BArgs a
 
 // ------------------------------------------------------------------ host side
 // Dynamic shared memory of one CTA: a neighbour list per warp.
-template <int W> constexpr size_t smem_bytes() { return (size_t)(kThreads / 32) * sizeof(Nbrs<W>); }
+template <int W, bool EDGE> constexpr size_t smem_bytes() { return (size_t)(kThreads / 32) * sizeof(WarpBuf<W, EDGE>); }
 
 // Co-resident CTAs per SM of k_batch<W, EDGE> with its shared memory (the shared-memory
 // attribute is set on the first call, outside any stream capture).
@@ -1053,9 +1176,9 @@ template <int W, bool EDGE = false, bool S32 = false> int blocks_per_sm()
 {
     static int b = -1;
     if (b < 0) {
-        NK_CUDA(cudaFuncSetAttribute(k_batch<W, EDGE, S32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<W>()));
+        NK_CUDA(cudaFuncSetAttribute(k_batch<W, EDGE, S32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes<W, EDGE>()));
         int v = 0;
-        NK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_batch<W, EDGE, S32>, kThreads, smem_bytes<W>()));
+        NK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_batch<W, EDGE, S32>, kThreads, smem_bytes<W, EDGE>()));
         b = v;
     }
     return b;
@@ -1256,7 +1379,7 @@ int launch_batches(nk_graph *g, const int32_t *d_src, int32_t k, double *d_score
             a.rk_key = cfg.rk_key ? cfg.rk_key + (size_t)bi * B : nullptr;
             a.trace = (trace_on && bi == todo.front()) ? trace_buf.as<unsigned long long>() : nullptr;
             void *args[] = {&a};
-            NK_CUDA(cudaLaunchCooperativeKernel(kfn, dim3(grid), dim3(kThreads), args, smem_bytes<W>(), s));
+            NK_CUDA(cudaLaunchCooperativeKernel(kfn, dim3(grid), dim3(kThreads), args, edge ? smem_bytes<W, true>() : smem_bytes<W, false>(), s));
             ::nk::count_launch();
         }
         if (cfg.time_kernels) NK_CUDA(cudaEventRecord(e1, s));
@@ -1442,7 +1565,7 @@ int enqueue_batches(nk_graph *g, const int32_t *d_src, int32_t k, double *d_scor
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(grid);
     lc.blockDim = dim3(kThreads);
-    lc.dynamicSmemBytes = smem_bytes<W>();
+    lc.dynamicSmemBytes = smem_bytes<W, false>();
     lc.stream = s;
     lc.attrs = &attr;
     lc.numAttrs = 1;

@@ -2,6 +2,9 @@
 import numpy as np
 import pytest
 
+import graphs as G
+import oracle
+
 pytestmark = pytest.mark.gpu
 
 
@@ -50,3 +53,31 @@ def test_sources_ordered_over_batches(nk, with_arcs):
     for batch in (64, 128):
         got = nk.betweenness_sources(g, np.arange(n, dtype=np.int32), 0.5, nk.run_opts(mode=nk.MODE_BATCHED, batch=batch))
         assert np.allclose(got, score, rtol=1e-9, atol=1e-12)
+
+
+# rows of 31..33 and 64, 65 arcs (windows of 32), 255..257 and 512 (chunks of 256) among short ones
+# and isolated vertices; a graph of under 32 vertices; one whose groups are full (32 vertices a warp)
+GROUPS = {
+    "rows": G.with_hubs(G.disjoint_union(G.complete(1), G.gnp(600, 0.01, 3)), [31, 32, 33, 64, 65, 255, 256, 257, 512], 5),
+    "tiny": G.gnp(20, 0.3, 2),
+    "many": G.gnp(30000, 0.0001, 7),
+}
+
+
+@pytest.mark.parametrize("name", list(GROUPS))
+@pytest.mark.parametrize("batch", [64, 128, 256])
+def test_groups_of_rows(nk, name, batch):
+    """The batched sweep, which walks the concatenated rows of groups of vertices, in both
+    directions and with small chunks, against the oracle."""
+    n, u, v = GROUPS[name]
+    g = nk.graph_from_edges(n, u, v)
+    rp, col = oracle.csr_build(n, u, v)
+    k = min(n, 150)
+    ref = oracle.betweenness_sampled(rp, col, 3, k)
+    far = oracle.closeness_sampled(rp, col, 3, k)
+    edges = oracle.edge_betweenness_sampled(rp, col, 3, k)
+    for kw in (dict(direction=1), dict(direction=2), dict(alpha=2.0, chunk=32)):
+        o = nk.run_opts(mode=nk.MODE_BATCHED, batch=batch, **kw)
+        assert np.allclose(nk.betweenness_sampled(g, 3, k, o), ref, rtol=1e-9, atol=1e-12)
+        assert np.allclose(nk.edge_betweenness_sampled(g, 3, k, o), edges, rtol=1e-9, atol=1e-12)
+        assert all(np.array_equal(x, y) for x, y in zip(nk.closeness_sampled(g, 3, k, o), far))
