@@ -41,27 +41,21 @@
 
 #include "nk_device.cuh"
 #include "nk_internal.h"
+#include "nk_sweep.cuh"
 
 namespace cg = cooperative_groups;
 
 namespace nk {
 namespace {
 
+using namespace sweep;
+
 constexpr int kThreads = 256;
 constexpr int kErrDepth = 100;  // internal status: BFS deeper than the level slabs
-constexpr int kErrCheck = 101;  // internal status: a device-side range check failed
 constexpr int kErrWide = 102;   // internal status: a path count did not fit the 32-bit sigma rows
 constexpr int kStartLevels = 48; // level slabs of a first attempt
-constexpr unsigned FULL = 0xffffffffu;
 constexpr int kTraceCap = 1024;
 constexpr int kChunk = kHeavyChunk;  // default arcs per work item; longer rows are split
-constexpr int kGrabV = 32;           // most vertices a warp takes at a time (one per lane)
-constexpr int kGrabArcs = 256;       // arcs, by the graph's average, a warp takes at a time
-constexpr int kGrabShare = 4;        // a warp takes at most 1/kGrabShare of its share of a phase
-constexpr int kGrabCMax = 16;        // most heavy chunks a warp takes at a time
-// work-counter slots of a level
-enum { WQ_BU = 0, WQ_BU_C, WQ_PUSH, WQ_PUSH_C, WQ_PULL, WQ_PULL_C, WQ_BACK, WQ_BACK_C };
-
 struct BArgs {
     int32_t n;
     int64_t A;
@@ -100,9 +94,7 @@ struct BArgs {
     int32_t H, C;
     unsigned long long *part;    // [C][B] per-chunk partial sums (uint64 or double)
     unsigned long long *trace;   // [kTraceCap][2] (code, globaltimer) after each barrier, or null
-    unsigned long long *far;     // [n] closeness: sums of distances from the batch's sources, or null
-    unsigned long long *reach;   // [n] closeness: number of the batch's sources that reach v
-    int backward;                // 0: forward sweep only (closeness)
+    int backward;                // 0: forward sweep only (error-bounded estimate)
     double *edge;                // [A] edge betweenness: per-arc shares, or null
     // error-bounded estimate (forward sweep only): per source slot, the target of its
     // random shortest path and the key of the walk's stream; counts of interior vertices
@@ -110,52 +102,6 @@ struct BArgs {
     const unsigned long long *rk_key;
     unsigned long long *rk_count;
 };
-
-template <int W> struct Bits {
-    unsigned long long w[W];
-};
-
-template <int W> __device__ __forceinline__ Bits<W> load_bits(const unsigned long long *p)
-{
-    Bits<W> r;
-    if constexpr (W == 1) {
-        r.w[0] = __ldcg(p);
-    } else {
-#pragma unroll
-        for (int q = 0; q < W; q += 2) {
-            const ulonglong2 x = __ldcg(reinterpret_cast<const ulonglong2 *>(p + q));
-            r.w[q] = x.x;
-            r.w[q + 1] = x.y;
-        }
-    }
-    return r;
-}
-
-template <int W> __device__ __forceinline__ bool any_bits(const Bits<W> &b)
-{
-    unsigned long long o = 0;
-#pragma unroll
-    for (int q = 0; q < W; ++q) o |= b.w[q];
-    return o != 0;
-}
-
-template <int W> __device__ __forceinline__ Bits<W> shfl_bits(const Bits<W> &b, int src)
-{
-    Bits<W> r;
-#pragma unroll
-    for (int q = 0; q < W; ++q) r.w[q] = __shfl_sync(FULL, b.w[q], src);
-    return r;
-}
-
-template <int W> __device__ __forceinline__ Bits<W> andnot(const Bits<W> &x, const Bits<W> &y)
-{
-    Bits<W> r;
-#pragma unroll
-    for (int q = 0; q < W; ++q) r.w[q] = x.w[q] & ~y.w[q];
-    return r;
-}
-
-__device__ __forceinline__ int deg_of(const int32_t *rp, int v) { return __ldg(rp + v + 1) - __ldg(rp + v); }
 
 // Source slots of a lane: lane L owns the G = 2W consecutive sources [G L, G L + G) of the
 // batch.  Slot k of lane L is source G L + k: bit G L + k of the batch's bitsets (word
@@ -197,16 +143,6 @@ template <int W> __device__ __forceinline__ void store_lane_bits(unsigned long l
 __device__ __forceinline__ void add_carry(unsigned long long &acc, unsigned &carry, unsigned long long x)
 {
     asm("add.cc.u64 %0, %0, %2;\n\taddc.u32 %1, %1, 0;" : "+l"(acc), "+r"(carry) : "l"(x));
-}
-
-// Records the first failed device-side check (code, where, offending value); every CTA
-// then leaves at its next grid barrier and the host reports the status.
-__device__ __forceinline__ void check_failed(const BArgs &a, int code, int where, int value)
-{
-    if (atomicCAS(&a.ctrl->err, 0, code) == 0) {
-        a.ctrl->where = where;
-        a.ctrl->bad_id = value;
-    }
 }
 
 // One warp's shared memory: the group of vertices it works on, and the list of the relevant
@@ -371,37 +307,25 @@ __device__ __forceinline__ unsigned gather(const BArgs &a, bool on, int v, int b
         check_failed(a, kErrCheck, 1, beg);
         on = false;
     }
-    const int d0 = on ? dg : 0;
-    int incl = d0;
-#pragma unroll
-    for (int s = 1; s < 32; s <<= 1) {
-        const int y = __shfl_up_sync(FULL, incl, s);
-        if (lane >= s) incl += y;
-    }
-    const int total = __shfl_sync(FULL, incl, 31), pre = incl - d0;
-    const unsigned members = __ballot_sync(FULL, d0 > 0);
-    pos = d0 > 0 ? __popc(members & dev::lanemask_lt()) : -1;
+    Rows rows(on ? dg : 0);
+    pos = rows.place();
     __syncwarp();  // the group before is done with the buffer
-    if (d0 > 0) {
+    if (pos >= 0) {
         st.v[pos] = v;
-        st.off[pos] = beg - pre;
+        st.off[pos] = beg - rows.pre;
 #pragma unroll
         for (int q = 0; q < W; ++q) st.t[pos][q] = t.w[q];
     }
     __syncwarp();
-    int cur = -1, before = 0;
+    int cur = -1;
     unsigned done = 0;
-    for (int base = 0; base < total; base += 32) {
-        // the vertices whose arcs start in this window mark their first arc; an arc's vertex is
-        // the number of marks up to it
-        const unsigned marks = __reduce_or_sync(FULL, d0 > 0 && (unsigned)(pre - base) < 32u ? 1u << (pre - base) : 0u);
-        const int o = before + __popc(marks & (dev::lanemask_lt() << 1 | 1u)) - 1;
-        before += __popc(marks);
+    for (int base = 0; base < rows.total; base += 32) {
+        const int o = rows.owner(base);
         int c = 0, j = 0;
         Bits<W> f;
 #pragma unroll
         for (int q = 0; q < W; ++q) f.w[q] = 0;
-        if (base + lane < total) {
+        if (base + lane < rows.total) {
             j = st.off[o] + base + lane;
             c = __ldg(a.col + j);
             const Bits<W> fc = load_bits<W>(Fsel + (size_t)c * W);
@@ -509,11 +433,6 @@ __device__ __forceinline__ unsigned gather(const BArgs &a, bool on, int v, int b
     return done;
 }
 
-struct BlockCnt {
-    int v;
-    unsigned long long mf, dmu;
-};
-
 // Writes the new counts acc of the lane's slots nib of vertex w's sigma row.
 template <int W, bool S32>
 __device__ __forceinline__ void store_sigma(const BArgs &a, int w, unsigned nib, int lane,
@@ -536,16 +455,6 @@ __device__ __forceinline__ void store_sigma(const BArgs &a, int w, unsigned nib,
 #pragma unroll
         for (int k = 0; k < 2 * W; ++k)
             if ((nib >> k) & 1u) row[slot_off<W>(k, lane)] = acc[k];
-    }
-}
-
-template <int W> __device__ __forceinline__ void store_bits(unsigned long long *p, const Bits<W> &b)
-{
-    if constexpr (W == 1) {
-        *p = b.w[0];
-    } else {
-#pragma unroll
-        for (int q = 0; q < W; q += 2) *reinterpret_cast<ulonglong2 *>(p + q) = make_ulonglong2(b.w[q], b.w[q + 1]);
     }
 }
 
@@ -576,107 +485,6 @@ __device__ __forceinline__ void join_level(const BArgs &a, bool on, int w, int d
     }
 }
 
-// Vertices a warp takes at a time (a power of two up to the 32 lanes) of the n of a phase: about
-// kGrabArcs arcs by the graph's average, and at most 1/kGrabShare of the warp's share.  Always 32
-// vertices left most warps idle on small graphs (63 of 4864 worked on ER 2000: a launch of 64
-// sources 680 us, now 200) and made long tails on others: BA 10^6 (16 arcs a vertex), 128 sources,
-// 128 arcs a grab 34.1 ms, 256 33.7, 512 42.6; R-MAT 24 (31) 398, 372, 361 (the counter's atomics).
-__device__ __forceinline__ int grab_size(const BArgs &a, int n, int nw)
-{
-    const int by_arcs = (int)((long long)a.n * kGrabArcs / max((long long)a.A, 1ll));
-    const int most = min(by_arcs, n / (kGrabShare * nw));
-    return most >= kGrabV ? kGrabV : most <= 1 ? 1 : 1 << (31 - __clz(most));
-}
-
-// How a phase finds its vertices: entries [qo, qo + nq) of the queue, or a scan of all
-// vertices (the callee looks at their bits).  nq: the number of vertices expected.
-struct Level {
-    int qo;   // -1: scan
-    int nq;
-};
-
-// Calls fn(on, v, beg, dg, chunk) with the whole warp for all work of a phase.  First the
-// chunks of the heavy vertices, whose work is largest (chunk >= 0: lane 0 holds the vertex and
-// the chunk's arcs), then groups of light vertices, one per lane (chunk = -1).  Warps take work
-// dynamically from the two zeroed counters, each grab requested while the one before is worked
-// on; scans of sparse levels (under n/32 vertices) are static.  Loops are bounded in time: lane
-// 0 checks the phase's deadline (kept in shared memory) once per item and the warp leaves together (the status is read
-// at the next barrier).
-template <class Fn>
-__device__ __forceinline__ void for_work(const BArgs &a, Level lv, int32_t *ctr, int32_t *ctr_c,
-                                         unsigned long long &deadline, Fn fn)
-{
-    const int lane = threadIdx.x & 31;
-    const int nw = (int)(((long long)gridDim.x * blockDim.x) >> 5);
-    if (lane == 0) deadline = dev::globaltimer() + a.limit_ns;
-    // about C / (32 warps) chunks per grab, 1..16: few chunks stay spread over many warps,
-    // millions of chunks cost few atomics
-    const int gc = max(1, min(kGrabCMax, a.C / (32 * nw)));
-    const bool fixed = lv.qo < 0 && lv.nq < a.n / 32;
-    const int gv = fixed ? kGrabV : grab_size(a, lv.qo >= 0 ? lv.nq : a.n, nw);
-    const int step = fixed ? nw * kGrabV : 0;
-    const unsigned end = lv.qo >= 0 ? lv.nq : a.n;
-    int c = 0, cend = 0;
-    unsigned next = 0;  // lane 0: the grab under way
-    bool chunks = a.C > 0;
-    auto grab = [&]() {
-        if (lane == 0) {
-            if (chunks) next = (unsigned)atomicAdd(ctr_c, gc);
-            else next = step ? next + step : (unsigned)atomicAdd(ctr, gv);
-        }
-    };
-    auto first = [&]() {  // of the scan
-        if (lane == 0) next = step ? (unsigned)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kGrabV
-                                   : (unsigned)atomicAdd(ctr, gv);
-    };
-    if (chunks) grab();
-    else first();
-    for (;;) {
-        bool on = false;
-        int v = 0, beg = 0, dg = 0, chunk = -1;
-        if (chunks) {
-            if (c >= cend) {
-                c = __shfl_sync(FULL, (int)next, 0);
-                if (c >= a.C) {
-                    chunks = false;
-                    first();
-                    continue;
-                }
-                cend = min(c + gc, a.C);
-                grab();
-            }
-            const int i = __ldg(a.chunk_h + c);
-            v = __ldg(a.hv + i);
-            beg = __ldg(a.rp + v) + (c - __ldg(a.hfirst + i)) * a.chunk;
-            dg = min(a.chunk, __ldg(a.rp + v + 1) - beg);
-            on = lane == 0;
-            chunk = c++;
-        } else {
-            const unsigned i = __shfl_sync(FULL, next, 0) + lane;
-            if (i - lane >= end) break;
-            grab();
-            on = lane < gv && i < end;
-            if (on) v = lv.qo >= 0 ? __ldcg(a.queue + lv.qo + i) : (int)i;
-            if (on && (unsigned)v >= (unsigned)a.n) {
-                check_failed(a, kErrCheck, 3, v);
-                on = false;
-            }
-            if (on) {
-                beg = __ldg(a.rp + v);
-                dg = __ldg(a.rp + v + 1) - beg;
-                on = dg > 0 && dg <= a.chunk;
-            }
-        }
-        int late = 0;
-        if (lane == 0 && dev::globaltimer() > deadline) {
-            check_failed(a, NK_ERR_TIMEOUT, 2, lv.nq);
-            late = 1;
-        }
-        if (__shfl_sync(FULL, late, 0)) break;
-        fn(on, v, beg, dg, chunk);
-    }
-}
-
 // Phase trace (diagnostics): CTA 0 records (code, %globaltimer) after a grid barrier.
 // code = level * 16 + phase.
 enum { PH_INIT = 1, PH_BU_A, PH_BU_B, PH_TD_A, PH_TD_B, PH_TD_C, PH_BK_A, PH_BK_B };
@@ -688,15 +496,6 @@ __device__ __forceinline__ void trace_mark(const BArgs &a, int &ti, int level, i
         a.trace[2 * ti + 1] = dev::globaltimer();
         ++ti;
     }
-}
-
-// fn(i, h, c0, c1) per heavy vertex (chunks [c0, c1)), with the whole warp.
-template <class Fn> __device__ __forceinline__ void for_heavy(const BArgs &a, Fn fn)
-{
-    const long long wid = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
-    for (long long i = wid; i < a.H; i += nw)
-        fn((int)i, __ldg(a.hv + i), __ldg(a.hfirst + i), __ldg(a.hfirst + i + 1));
 }
 
 template <int W>
@@ -841,29 +640,18 @@ __global__ void __launch_bounds__(kThreads, min_ctas<W, EDGE>()) k_batch(BArgs a
                     t = load_bits<W>(Fd + (size_t)v * W);
                     on = any_bits<W>(t);
                 }
-                const int d0 = on ? dg : 0;
-                int incl = d0;
-#pragma unroll
-                for (int s = 1; s < 32; s <<= 1) {
-                    const int y = __shfl_up_sync(FULL, incl, s);
-                    if (lane >= s) incl += y;
-                }
-                const int total = __shfl_sync(FULL, incl, 31), pre = incl - d0;
-                const unsigned members = __ballot_sync(FULL, d0 > 0);
+                Rows rows(on ? dg : 0);
+                const int pos = rows.place();
                 __syncwarp();
-                if (d0 > 0) {
-                    const int pos = __popc(members & dev::lanemask_lt());
-                    st.off[pos] = beg - pre;
+                if (pos >= 0) {
+                    st.off[pos] = beg - rows.pre;
 #pragma unroll
                     for (int q = 0; q < W; ++q) st.t[pos][q] = t.w[q];
                 }
                 __syncwarp();
-                int before = 0;
-                for (int base = 0; base < total; base += 32) {
-                    const unsigned marks = __reduce_or_sync(FULL, d0 > 0 && (unsigned)(pre - base) < 32u ? 1u << (pre - base) : 0u);
-                    const int o = before + __popc(marks & (dev::lanemask_lt() << 1 | 1u)) - 1;
-                    before += __popc(marks);
-                    if (base + lane >= total) continue;
+                for (int base = 0; base < rows.total; base += 32) {
+                    const int o = rows.owner(base);
+                    if (base + lane >= rows.total) continue;
                     const int c = __ldg(a.col + st.off[o] + base + lane);
                     const Bits<W> vc = load_bits<W>(a.vis + (size_t)c * W);
                     bool any = false;
@@ -1039,30 +827,6 @@ __global__ void __launch_bounds__(kThreads, min_ctas<W, EDGE>()) k_batch(BArgs a
                 if (z < 0) break;  // only with a wrapped path count (reported as an overflow)
                 if (lane == 0) atomicAdd(a.rk_count + z, 1ull);
                 w = z;
-            }
-        }
-    }
-    if (a.far) {
-        // closeness: v is at distance l from the sources of F_l[v]; one thread per vertex
-        // adds its level sums once the whole sweep has stayed within the slabs (a batch
-        // that ran out of levels returned above and adds nothing).  A bottom-up level takes
-        // its new bits from non-zero path sums, which a sum that wrapped past 2^64 could
-        // hide: a batch with an overflow adds nothing either and the host reruns it.
-        if (!dev::grid_barrier(a.ctrl, a.limit_ns)) return;
-        if (dev::ld_volatile(&a.ctrl->ovf) != 0) return;
-        for (long long v = tid; v < a.n; v += nthr) {
-            unsigned long long fs = 0, rs = 0;
-            for (int l = 1; l <= D; ++l) {
-                const Bits<W> f = load_bits<W>(a.F + (size_t)l * slab + (size_t)v * W);
-                unsigned long long cnt = 0;
-#pragma unroll
-                for (int q = 0; q < W; ++q) cnt += (unsigned long long)__popcll(f.w[q]);
-                fs += cnt * (unsigned long long)l;
-                rs += cnt;
-            }
-            if (rs) {
-                a.far[v] += fs;
-                a.reach[v] += rs;
             }
         }
     }
@@ -1354,8 +1118,6 @@ int launch_batches(nk_graph *g, const int32_t *d_src, int32_t k, double *d_score
         a.chunk = hw.chunk;
         a.part = reinterpret_cast<unsigned long long *>(base + L.off_part);
         a.trace = nullptr;
-        a.far = cfg.far;
-        a.reach = cfg.reach;
         a.backward = cfg.backward ? 1 : 0;
         a.edge = edge ? cfg.edge : nullptr;
         a.rk_count = cfg.rk_count;
@@ -1448,12 +1210,9 @@ int launch_batches(nk_graph *g, const int32_t *d_src, int32_t k, double *d_score
             ovf |= h[bi].ovf != 0;
             if (h[bi].err == kErrDepth) deep.push_back(bi);
         }
-        if (ovf && !cfg.far) return set_error(NK_ERR_OVERFLOW, "a shortest-path count exceeded 2^64 - 1");
-        if (cfg.far)  // closeness: batches with a wrapped path count go to the per-source form
-            for (int bi : todo)
-                if (h[bi].ovf && h[bi].err != kErrDepth) deep.push_back(bi);
+        if (ovf) return set_error(NK_ERR_OVERFLOW, "a shortest-path count exceeded 2^64 - 1");
         if (deep.empty()) return NK_OK;
-        if (lcap < lmax && !(cfg.far && ovf)) {
+        if (lcap < lmax) {
             todo = deep;
             lcap = lmax;
             continue;
@@ -1536,8 +1295,6 @@ int enqueue_batches(nk_graph *g, const int32_t *d_src, int32_t k, double *d_scor
     a.chunk = hw.chunk;
     a.part = reinterpret_cast<unsigned long long *>(base + L.off_part);
     a.trace = nullptr;
-    a.far = cfg.far;
-    a.reach = cfg.reach;
     a.backward = cfg.backward ? 1 : 0;
     a.edge = nullptr;  // the captured form serves vertex scores only
     a.rk_t = nullptr;

@@ -347,7 +347,7 @@ int closeness_entry(const nk_graph *gc, bool sample, uint64_t seed, int32_t k, d
     int mode = cfg.mode == NK_MODE_AUTO ? (k >= 16 ? NK_MODE_BATCHED : NK_MODE_PER_SOURCE) : cfg.mode;
     int rc;
     if (mode == NK_MODE_BATCHED) {
-        rc = run_batched(g, dsrc.as<int32_t>(), k, nullptr, cfg, &t_stats, s);
+        rc = run_levels(g, dsrc.as<int32_t>(), k, cfg, &t_stats, s);
         if (rc == NK_ERR_NOMEM && cfg.mode == NK_MODE_AUTO) {
             NK_CUDA(cudaMemsetAsync(sums.p, 0, sizeof(unsigned long long) * 2 * (size_t)n, s));
             t_stats = RunStats();

@@ -268,6 +268,10 @@ int run_weighted(nk_graph *g, const int32_t *d_src, int32_t k, double *d_scores,
 int run_batched(nk_graph *g, const int32_t *d_src, int32_t k, double *d_scores,
                 const RunCfg &cfg, RunStats *st, cudaStream_t s);
 
+// Batched closeness sweeps (nk_levels.cu): cfg.far and cfg.reach (device) += the distance sums and
+// reach counts of the k device sources, in batches of cfg.batch sources (0: by k).
+int run_levels(nk_graph *g, const int32_t *d_src, int32_t k, const RunCfg &cfg, RunStats *st, cudaStream_t s);
+
 // Capturable pieces of the batched form: prepare_only sizes and allocates the scratch
 // (outside any stream capture); otherwise the status reset and the launches are enqueued
 // without host synchronisation, and *ctrls / *nb give the per-batch status words.

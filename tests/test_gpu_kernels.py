@@ -81,3 +81,18 @@ def test_groups_of_rows(nk, name, batch):
         assert np.allclose(nk.betweenness_sampled(g, 3, k, o), ref, rtol=1e-9, atol=1e-12)
         assert np.allclose(nk.edge_betweenness_sampled(g, 3, k, o), edges, rtol=1e-9, atol=1e-12)
         assert all(np.array_equal(x, y) for x, y in zip(nk.closeness_sampled(g, 3, k, o), far))
+
+
+@pytest.mark.parametrize("batch", [0, 64, 128, 256])
+def test_closeness_levels(nk, batch):
+    """Closeness from level bitsets: a search far deeper than the levels kept at a time, and
+    source counts at the edges of the batch widths, against sums in closed form."""
+    n = 700
+    i = np.arange(n)
+    g = nk.graph_from_edges(*G.path(n))
+    for k in (63, 64, 65, 128, 129, 256, 257, n):
+        src = oracle.sample_sources(n, 8, k)
+        for direction in (0, 1, 2):
+            far, reach = nk.closeness_sampled(g, 8, k, nk.run_opts(mode=nk.MODE_BATCHED, batch=batch, direction=direction))
+            assert np.array_equal(far, np.abs(i[:, None] - src).sum(1) * (n / k))
+            assert np.array_equal(reach, (i[:, None] != src).sum(1) * (n / k))
