@@ -214,8 +214,8 @@ int nk_betweenness_sources(const nk_graph *g, const int32_t *src, int32_t k, dou
 int nk_last_run_stats(nk_run_stats *out);
 
 /* Autotuner (no counterpart in the paper; it tunes the batched GPU sweep, which is this
- * library's own design): on one launch of up to 256 of the run's own sources (seed, k), times the
- * batched sweep with 64/128/256 sources per launch, then alpha in {0.25, 1, 4, 16}, then hub
+ * library's own design): on up to 256 of the run's own sources (seed, k), times the
+ * batched sweep with batches of 64 and 128 sources, then alpha in {0.25, 1, 4, 16}, then hub
  * chunks of 128 arcs against 256, then the relabelled copy (NK_RUN_RELABEL) with alpha in
  * {0.25, 4, 16}; writes the fastest into *best (flags: NK_RUN_RELABEL or NK_RUN_NO_RELABEL).
  * The choice is cached on the graph: later calls with batch/alpha/chunk = 0 and neither

@@ -35,6 +35,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <climits>
 #include <cstdio>
 #include <cstdlib>
 #include <vector>
@@ -56,18 +57,20 @@ constexpr int kErrWide = 102;   // internal status: a path count did not fit the
 constexpr int kStartLevels = 48; // level slabs of a first attempt
 constexpr int kTraceCap = 1024;
 constexpr int kChunk = kHeavyChunk;  // default arcs per work item; longer rows are split
+// The arrays below hold the state of every team (blockIdx.y) side by side: [n] stands for
+// [teams][n], and a team's row of vertex v is row team * n + v.
 struct BArgs {
     int32_t n;
     int64_t A;
     const int32_t *rp, *col;
     const int32_t *src;
-    int32_t nsrc;
+    int32_t nsrc;                // sources of the whole run
+    int32_t b0;                  // this launch's first batch
     // when set (captured calls), the number of sources of the whole run is *ksrc, read on
-    // the device, and this batch has min(B, *ksrc - boff) of them (none: it returns at once)
+    // the device
     const int32_t *ksrc;
-    int32_t boff;
     int32_t lcap;                // levels 0..lcap may be non-empty; slabs 0..lcap+1
-    unsigned long long *F;       // [lcap+2][n][W]
+    unsigned long long *F;       // [lcap+2][teams][n][W]
     unsigned long long *vis;     // [n][W]
     unsigned long long *sp;      // [n][B]
     unsigned *sp32;              // [n][B] sigma in 32 bits during the forward sweep (kernels with S32)
@@ -81,7 +84,7 @@ struct BArgs {
     unsigned long long *dmu;     // [lcap+3] degrees of vertices completed at level d
     int32_t *wq;                 // [lcap+3][8] work counters of the phases of level d
     double *scores;
-    Ctrl *ctrl;
+    Ctrl *ctrl;                  // [batches of the run]
     uint64_t limit_ns;
     double alpha;
     int dir;
@@ -101,6 +104,8 @@ struct BArgs {
     const int32_t *rk_t;
     const unsigned long long *rk_key;
     unsigned long long *rk_count;
+
+    __device__ __forceinline__ Ctrl *status() const { return ctrl + b0 + blockIdx.y; }
 };
 
 // Source slots of a lane: lane L owns the G = 2W consecutive sources [G L, G L + G) of the
@@ -150,11 +155,11 @@ __device__ __forceinline__ void add_carry(unsigned long long &acc, unsigned &car
 template <int W, bool EDGE> struct WarpBuf {
     unsigned long long f[32][W];  // list: bits the neighbour shares with its vertex
     unsigned long long t[32][W];  // group: the bits a vertex gathers (a pull leaves its new bits here)
-    int c[32];                    // list: neighbour
+    unsigned c[32];               // list: the neighbour's row
     int o[32];                    // list: its vertex's place in the group
     int off[32];                  // group: first arc, less the arcs of the vertices before
-    int v[32];                    // group: vertex
-    unsigned long long until;     // deadline of the phase
+    unsigned v[32];               // group: the vertex's row
+    Hand hand;
     double e[EDGE ? 32 : 1];      // list, edge variant: the arc's share
 };
 
@@ -235,12 +240,19 @@ __device__ __forceinline__ void ff_add_if(unsigned on, dev::ff &a, unsigned hi, 
         : "+f"(a.hi), "+f"(a.lo) : "r"(on), "f"(__uint_as_float(hi)), "f"(__uint_as_float(lo)));
 }
 
+// F_d of the block's team, and its queue
+__device__ __forceinline__ unsigned long long *level_bits(const BArgs &a, int d, size_t slab)
+{
+    return a.F + ((size_t)d * gridDim.y + blockIdx.y) * slab;
+}
+__device__ __forceinline__ int32_t *queue_of(const BArgs &a) { return a.queue + (size_t)blockIdx.y * a.qcap; }
+
 // A lane's 2W values of a vertex's row, loaded in 16-byte pieces, each only if one of its
 // entries is relevant (nib); the values of other entries are undefined.
 template <int W, bool S32> struct RowPart {
     static constexpr int G = 2 * W;
     unsigned u[S32 ? G : 2 * G];
-    __device__ __forceinline__ void load(const BArgs &a, int c, int lane, unsigned nib)
+    __device__ __forceinline__ void load(const BArgs &a, unsigned c, int lane, unsigned nib)
     {
         if constexpr (S32) {
             const unsigned *row = a.sp32 + (size_t)c * (64 * W) + G * lane;
@@ -294,7 +306,7 @@ template <int W, bool PSI, bool EDGE, bool S32, class Buf, class Begin, class Fl
 __device__ __forceinline__ unsigned gather(const BArgs &a, bool on, int v, int beg, int dg, const Bits<W> &t,
                                            const unsigned long long *Fsel, Buf &st,
                                            unsigned long long (&acc)[2 * W], dev::ff (&facc)[2 * W],
-                                           dev::ff (&sv)[2 * W], bool &ovf, int &pos, Begin begin, Flush flush)
+                                           dev::ff (&sv)[2 * W], int &pos, Begin begin, Flush flush)
 {
     // rows in flight.  With 2 instead of 4 rows of 32-bit counts R-MAT 18 and BA 10^6 (128 sources)
     // go from 13.2 to 13.5 and 33.5 to 35.7 ms; with 4 rows of psi the W = 2 and 4 kernels run out of
@@ -302,16 +314,17 @@ __device__ __forceinline__ unsigned gather(const BArgs &a, bool on, int v, int b
     // 41.5 -> 36.0 ms)
     constexpr int G = 2 * W, NB = S32 || (PSI && !EDGE && W == 1) ? 4 : 2;
     const int lane = threadIdx.x & 31;
+    const unsigned tn = blockIdx.y * (unsigned)a.n;
     unsigned carry = 0;
     if (on && (beg < 0 || dg < 0 || (long long)beg + dg > a.A)) {
-        check_failed(a, kErrCheck, 1, beg);
+        check_failed(a.status(), kErrCheck, 1, beg);
         on = false;
     }
     Rows rows(on ? dg : 0);
     pos = rows.place();
     __syncwarp();  // the group before is done with the buffer
     if (pos >= 0) {
-        st.v[pos] = v;
+        st.v[pos] = tn + v;
         st.off[pos] = beg - rows.pre;
 #pragma unroll
         for (int q = 0; q < W; ++q) st.t[pos][q] = t.w[q];
@@ -341,11 +354,11 @@ __device__ __forceinline__ unsigned gather(const BArgs &a, bool on, int v, int b
         const unsigned fresh = __reduce_or_sync(FULL, mine && o != (at ? lead : cur) ? 1u << at : 0u);
         double eold = 0.0;
         if (mine) {
-            st.c[at] = c;
+            st.c[at] = tn + c;
             st.o[at] = o;
 #pragma unroll
             for (int q = 0; q < W; ++q) st.f[at][q] = f.w[q];
-            if constexpr (EDGE) eold = __ldcg(a.edge + j);
+            if constexpr (EDGE) eold = __ldcg(a.edge + (size_t)blockIdx.y * a.A + j);
         }
         if (lane >= cnt && lane < ((cnt + NB - 1) & ~(NB - 1))) {  // the last round's empty places
             st.c[lane] = 0;
@@ -422,20 +435,20 @@ __device__ __forceinline__ unsigned gather(const BArgs &a, bool on, int v, int b
         }
         __syncwarp();
         if constexpr (EDGE) {
-            if (mine) a.edge[j] = eold + st.e[at];
+            if (mine) a.edge[(size_t)blockIdx.y * a.A + j] = eold + st.e[at];
         }
     }
     if (cur >= 0) {
         flush(cur);
         done |= 1u << cur;
     }
-    if (!PSI) ovf |= carry != 0;
+    if (!PSI && !S32 && carry != 0) atomicOr(&a.status()->ovf, 1);
     return done;
 }
 
 // Writes the new counts acc of the lane's slots nib of vertex w's sigma row.
 template <int W, bool S32>
-__device__ __forceinline__ void store_sigma(const BArgs &a, int w, unsigned nib, int lane,
+__device__ __forceinline__ void store_sigma(const BArgs &a, unsigned w, unsigned nib, int lane,
                                             const unsigned long long (&acc)[2 * W])
 {
     constexpr int B = 64 * W;
@@ -449,7 +462,7 @@ __device__ __forceinline__ void store_sigma(const BArgs &a, int w, unsigned nib,
                 row[slot_off<W>(k, lane)] = (unsigned)acc[k];
                 wide |= (unsigned)(acc[k] >> 32);
             }
-        if (wide) atomicCAS(&a.ctrl->err, 0, kErrWide);
+        if (wide) atomicCAS(&a.status()->err, 0, kErrWide);
     } else {
         unsigned long long *row = a.sp + (size_t)w * B;
 #pragma unroll
@@ -464,15 +477,16 @@ template <int W>
 __device__ __forceinline__ void join_level(const BArgs &a, bool on, int w, int dg, const Bits<W> &nb,
                                            const Bits<W> &act, unsigned long long *Fn, BlockCnt *bc)
 {
+    const unsigned tn = blockIdx.y * (unsigned)a.n;
     bool full = on;
     if (on) {
-        Bits<W> nv = load_bits<W>(a.vis + (size_t)w * W);
+        Bits<W> nv = load_bits<W>(a.vis + (size_t)(tn + w) * W);
 #pragma unroll
         for (int q = 0; q < W; ++q) {
             nv.w[q] |= nb.w[q];
             full &= nv.w[q] == act.w[q];
         }
-        store_bits<W>(a.vis + (size_t)w * W, nv);
+        store_bits<W>(a.vis + (size_t)(tn + w) * W, nv);
         store_bits<W>(Fn + (size_t)w * W, nb);
     }
     const unsigned m = __ballot_sync(FULL, on);
@@ -491,7 +505,7 @@ enum { PH_INIT = 1, PH_BU_A, PH_BU_B, PH_TD_A, PH_TD_B, PH_TD_C, PH_BK_A, PH_BK_
 
 __device__ __forceinline__ void trace_mark(const BArgs &a, int &ti, int level, int phase)
 {
-    if (a.trace && blockIdx.x == 0 && threadIdx.x == 0 && ti < kTraceCap) {
+    if (a.trace && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 && ti < kTraceCap) {
         a.trace[2 * ti] = (unsigned long long)(level * 16 + phase);
         a.trace[2 * ti + 1] = dev::globaltimer();
         ++ti;
@@ -501,7 +515,7 @@ __device__ __forceinline__ void trace_mark(const BArgs &a, int &ti, int level, i
 template <int W>
 __device__ __forceinline__ void store_part(const BArgs &a, int c, const unsigned long long (&acc)[2 * W])
 {
-    unsigned long long *row = a.part + (size_t)c * (64 * W);
+    unsigned long long *row = a.part + (size_t)(blockIdx.y * (unsigned)a.C + c) * (64 * W);
 #pragma unroll
     for (int k = 0; k < 2 * W; ++k) row[slot_off<W>(k, threadIdx.x & 31)] = acc[k];
 }
@@ -509,7 +523,7 @@ __device__ __forceinline__ void store_part(const BArgs &a, int c, const unsigned
 // Sums of a heavy vertex's chunks [c0, c1) in chunk order, four loads in flight at a time.
 template <int W, class Add> __device__ __forceinline__ void sum_parts(const BArgs &a, int c0, int c1, Add add)
 {
-    const unsigned long long *p = a.part + (size_t)c0 * (64 * W) + slot_off<W>(0, threadIdx.x & 31);
+    const unsigned long long *p = a.part + (size_t)(blockIdx.y * (unsigned)a.C + c0) * (64 * W) + slot_off<W>(0, threadIdx.x & 31);
     constexpr int U = W == 1 ? 4 : 2;
     int c = c0;
     for (; c + U <= c1; c += U, p += U * 64 * W) {
@@ -536,76 +550,95 @@ template <int W, class Add> __device__ __forceinline__ void sum_parts(const BArg
 // for 256 sources
 template <int W, bool EDGE> constexpr int min_ctas() { return W >= 4 ? 2 : (EDGE && W == 2) ? 3 : 4; }
 
+// One batch per team: batch b0 + blockIdx.y by the gridDim.x blocks of that row of the grid.
 template <int W, bool EDGE, bool S32>
 __global__ void __launch_bounds__(kThreads, min_ctas<W, EDGE>()) k_batch(BArgs a)
 {
     constexpr int B = 64 * W;
+    // what changes from level to level, kept by thread 0 (in registers it would cost every thread of
+    // the gathers about twenty)
     __shared__ BlockCnt bc;
+    __shared__ struct {
+        unsigned long long act[W];  // bits of the batch's sources
+        long long mu, mf;           // arcs of vertices not yet visited by every source, of the level's
+        long long qtail;            // queue entries of all levels so far
+        int qo, nq;                 // the level's queue entries (qo < 0: found by a scan)
+        int td, bu, ti;
+    } lv;
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int bi = a.b0 + blockIdx.y;
     WarpBuf<W, EDGE> &st = reinterpret_cast<WarpBuf<W, EDGE> *>(smem_raw)[threadIdx.x >> 5];
     const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long nthr = (long long)gridDim.x * blockDim.x;
     const int lane = threadIdx.x & 31;
     const size_t slab = (size_t)a.n * W;
-    const int nsrc = a.ksrc ? max(0, min(B, __ldg(a.ksrc) - a.boff)) : a.nsrc;
-    if (nsrc == 0) return;  // uniform over the grid: no barrier is entered
-    Bits<W> act;
-#pragma unroll
-    for (int q = 0; q < W; ++q) {
-        const int left = nsrc - 64 * q;
-        act.w[q] = left >= 64 ? ~0ull : (left <= 0 ? 0ull : ((1ull << left) - 1));
+    const unsigned tn = blockIdx.y * (unsigned)a.n;           // the team's first row
+    const size_t lv0 = (size_t)blockIdx.y * (a.lcap + 3);      // its first level counter
+    const int nsrc = max(0, min(B, (a.ksrc ? __ldg(a.ksrc) : a.nsrc) - bi * B));
+    if (nsrc == 0) return;  // uniform over the team: no barrier is entered
+    if (threadIdx.x < W) {
+        const int left = nsrc - 64 * (int)threadIdx.x;
+        lv.act[threadIdx.x] = left >= 64 ? ~0ull : (left <= 0 ? 0ull : ((1ull << left) - 1));
     }
-    bool ovf = false;
-    int ti = 0;
-    trace_mark(a, ti, 0, 0);
+    if (threadIdx.x == 0) lv.ti = 0;
+    auto active = [&]() {
+        Bits<W> r;
+#pragma unroll
+        for (int q = 0; q < W; ++q) r.w[q] = lv.act[q];
+        return r;
+    };
+    trace_mark(a, lv.ti, 0, 0);
     auto flush_counts = [&](int lvl) {
         __syncthreads();
         if (threadIdx.x == 0) {
-            if (bc.v) atomicAdd(a.vcnt + lvl, bc.v);
-            if (bc.mf) atomicAdd(a.mfv + lvl, bc.mf);
-            if (bc.dmu) atomicAdd(a.dmu + lvl, bc.dmu);
+            if (bc.v) atomicAdd(a.vcnt + lv0 + lvl, bc.v);
+            if (bc.mf) atomicAdd(a.mfv + lv0 + lvl, bc.mf);
+            if (bc.dmu) atomicAdd(a.dmu + lv0 + lvl, bc.dmu);
         }
     };
 
     // ---- init: empty visited sets, F_0 and F_1, queue marks, level-0..2 counters
     for (size_t i = tid; i < slab; i += nthr) {
-        a.vis[i] = 0;
-        a.F[i] = 0;
-        a.F[slab + i] = 0;
+        a.vis[(size_t)tn * W + i] = 0;
+        level_bits(a, 0, slab)[i] = 0;
+        level_bits(a, 1, slab)[i] = 0;
     }
-    for (long long i = tid; i < a.n; i += nthr) a.qmark[i] = -1;
-    if (tid < 3 * 8) a.wq[tid] = 0;
+    for (long long i = tid; i < a.n; i += nthr) a.qmark[tn + i] = -1;
+    if (tid < 3 * 8) a.wq[lv0 * 8 + tid] = 0;
     if (tid < 3) {
-        a.vcnt[tid] = 0;
-        a.qcnt[tid] = 0;
-        a.qoff[tid] = -1;
-        a.mfv[tid] = 0;
-        a.dmu[tid] = 0;
+        a.vcnt[lv0 + tid] = 0;
+        a.qcnt[lv0 + tid] = 0;
+        a.qoff[lv0 + tid] = -1;
+        a.mfv[lv0 + tid] = 0;
+        a.dmu[lv0 + tid] = 0;
     }
-    if (!dev::grid_barrier(a.ctrl, a.limit_ns)) return;
-    trace_mark(a, ti, 0, PH_INIT);
+    if (!dev::grid_barrier(a.status(), a.limit_ns)) return;
+    trace_mark(a, lv.ti, 0, PH_INIT);
     if (tid < nsrc) {
-        const int s = __ldg(a.src + tid);
+        const int s = __ldg(a.src + (size_t)bi * B + tid);
         const unsigned long long bit = 1ull << (tid & 63);
-        atomicOr(a.F + (size_t)s * W + (tid >> 6), bit);
-        atomicOr(a.vis + (size_t)s * W + (tid >> 6), bit);
-        if constexpr (S32) a.sp32[(size_t)s * B + tid] = 1u;
-        else a.sp[(size_t)s * B + tid] = 1ull;
-        a.queue[tid] = s;
-        atomicAdd(a.mfv, (unsigned long long)deg_of(a.rp, s));
-        if (nsrc == 1) a.dmu[0] = (unsigned long long)deg_of(a.rp, s);
+        atomicOr(level_bits(a, 0, slab) + (size_t)s * W + (tid >> 6), bit);
+        atomicOr(a.vis + (size_t)(tn + s) * W + (tid >> 6), bit);
+        if constexpr (S32) a.sp32[(size_t)(tn + s) * B + tid] = 1u;
+        else a.sp[(size_t)(tn + s) * B + tid] = 1ull;
+        queue_of(a)[tid] = s;
+        atomicAdd(a.mfv + lv0, (unsigned long long)deg_of(a.rp, s));
+        if (nsrc == 1) a.dmu[lv0] = (unsigned long long)deg_of(a.rp, s);
     }
     if (tid == 0) {
-        a.vcnt[0] = nsrc;
-        a.qcnt[0] = nsrc;
-        a.qoff[0] = 0;
+        a.vcnt[lv0] = nsrc;
+        a.qcnt[lv0] = nsrc;
+        a.qoff[lv0] = 0;
     }
-    if (!dev::grid_barrier(a.ctrl, a.limit_ns)) return;
+    if (!dev::grid_barrier(a.status(), a.limit_ns)) return;
 
-    long long mu = a.A - (long long)__ldcg(a.dmu);
-    long long mf = (long long)__ldcg(a.mfv);
-    int d = 0, qo = 0, nq = nsrc, td = 0, bu = 0;
-    long long qtail = nsrc;
+    if (threadIdx.x == 0) {
+        lv.mu = a.A - (long long)__ldcg(a.dmu + lv0);
+        lv.mf = (long long)__ldcg(a.mfv + lv0);
+        lv.qtail = lv.nq = nsrc;
+        lv.qo = lv.td = lv.bu = 0;
+    }
+    int d = 0;
     for (;;) {
         if (threadIdx.x == 0) {
             bc.v = 0;
@@ -613,28 +646,28 @@ __global__ void __launch_bounds__(kThreads, min_ctas<W, EDGE>()) k_batch(BArgs a
             bc.dmu = 0;
         }
         if (tid == 0) {
-            a.vcnt[d + 2] = 0;
-            a.qcnt[d + 2] = 0;
-            a.mfv[d + 2] = 0;
-            a.dmu[d + 2] = 0;
+            a.vcnt[lv0 + d + 2] = 0;
+            a.qcnt[lv0 + d + 2] = 0;
+            a.mfv[lv0 + d + 2] = 0;
+            a.dmu[lv0 + d + 2] = 0;
         }
-        if (tid < 8) a.wq[(size_t)(d + 2) * 8 + tid] = 0;
+        if (tid < 8) a.wq[(lv0 + d + 2) * 8 + tid] = 0;
         {
-            unsigned long long *Fz = a.F + (size_t)(d + 2) * slab;
+            unsigned long long *Fz = level_bits(a, d + 2, slab);
             for (size_t i = tid; i < slab; i += nthr) Fz[i] = 0;
         }
         __syncthreads();
-        const unsigned long long *Fd = a.F + (size_t)d * slab;
-        unsigned long long *Fn = a.F + (size_t)(d + 1) * slab;
+        const unsigned long long *Fd = level_bits(a, d, slab);
+        unsigned long long *Fn = level_bits(a, d + 1, slab);
         const bool use_bu = a.dir == NK_DIR_BOTTOM_UP ||
-                            (a.dir == NK_DIR_AUTO && a.alpha * (double)mf > (double)mu);
+                            (a.dir == NK_DIR_AUTO && a.alpha * (double)lv.mf > (double)lv.mu);
         bool queued = false;
         int nq1 = 0;
-        int32_t *wq = a.wq + (size_t)d * 8;
+        int32_t *wq = a.wq + (lv0 + d) * 8;
         if (!use_bu) {
             // ---- top-down (a): push the frontier's bits, queue each new vertex once; lanes over
             //      the concatenated arcs of a group of frontier vertices, or of a heavy one's chunk
-            for_work(a, {qo, nq}, wq + WQ_PUSH, wq + WQ_PUSH_C, st.until, [&](bool on, int v, int beg, int dg, int) {
+            for_work(a, {lv.qo >= 0 ? queue_of(a) + lv.qo : nullptr, lv.nq}, wq + WQ_PUSH, st.hand, [&](bool on, int v, int beg, int dg, int) {
                 Bits<W> t;
                 if (on) {
                     t = load_bits<W>(Fd + (size_t)v * W);
@@ -653,7 +686,7 @@ __global__ void __launch_bounds__(kThreads, min_ctas<W, EDGE>()) k_batch(BArgs a
                     const int o = rows.owner(base);
                     if (base + lane >= rows.total) continue;
                     const int c = __ldg(a.col + st.off[o] + base + lane);
-                    const Bits<W> vc = load_bits<W>(a.vis + (size_t)c * W);
+                    const Bits<W> vc = load_bits<W>(a.vis + (size_t)(tn + c) * W);
                     bool any = false;
 #pragma unroll
                     for (int q = 0; q < W; ++q) {
@@ -661,30 +694,30 @@ __global__ void __launch_bounds__(kThreads, min_ctas<W, EDGE>()) k_batch(BArgs a
                         any |= m != 0;
                         if (m) atomicOr(Fn + (size_t)c * W + q, m);
                     }
-                    if (any && __ldcg(a.qmark + c) != d + 1 && atomicExch(a.qmark + c, d + 1) != d + 1) {
+                    if (any && __ldcg(a.qmark + tn + c) != d + 1 && atomicExch(a.qmark + tn + c, d + 1) != d + 1) {
                         cg::coalesced_group g = cg::coalesced_threads();
                         int pos = 0;
-                        if (g.thread_rank() == 0) pos = atomicAdd(a.qcnt + d + 1, (int)g.size());
+                        if (g.thread_rank() == 0) pos = atomicAdd(a.qcnt + lv0 + d + 1, (int)g.size());
                         pos = g.shfl(pos, 0) + (int)g.thread_rank();
-                        if (qtail + pos < a.qcap) a.queue[qtail + pos] = c;
+                        if (lv.qtail + pos < a.qcap) queue_of(a)[lv.qtail + pos] = c;
                     }
                 }
             });
-            if (!dev::grid_barrier(a.ctrl, a.limit_ns)) return;
-            trace_mark(a, ti, d, PH_TD_A);
-            nq1 = __ldcg(a.qcnt + d + 1);
-            queued = qtail + nq1 <= a.qcap;
+            if (!dev::grid_barrier(a.status(), a.limit_ns)) return;
+            trace_mark(a, lv.ti, d, PH_TD_A);
+            nq1 = __ldcg(a.qcnt + lv0 + d + 1);
+            queued = lv.qtail + nq1 <= a.qcap;
         }
         // ---- pull sigma from level d: bottom-up every vertex with unvisited sources, for all of
         //      them; top-down (b) every new vertex for its new bits.  Chunks of heavy vertices
         //      store partial sums.
-        const Level pull = use_bu ? Level{-1, a.n} : Level{queued ? (int)qtail : -1, nq1};
-        for_work(a, pull, wq + (use_bu ? WQ_BU : WQ_PULL), wq + (use_bu ? WQ_BU_C : WQ_PULL_C), st.until,
+        const Level pull = use_bu ? Level{nullptr, a.n} : Level{queued ? queue_of(a) + lv.qtail : nullptr, nq1};
+        for_work(a, pull, wq + (use_bu ? WQ_BU : WQ_PULL), st.hand,
                  [&](bool on, int v, int beg, int dg, int chunk) {
             Bits<W> t;
             if (on) {
-                t = load_bits<W>((use_bu ? (const unsigned long long *)a.vis : Fn) + (size_t)v * W);
-                if (use_bu) t = andnot<W>(act, t);
+                t = load_bits<W>(use_bu ? a.vis + (size_t)(tn + v) * W : Fn + (size_t)v * W);
+                if (use_bu) t = andnot<W>(active(), t);
                 on = any_bits<W>(t);
             }
             if (!__any_sync(FULL, on)) return;
@@ -694,7 +727,7 @@ __global__ void __launch_bounds__(kThreads, min_ctas<W, EDGE>()) k_batch(BArgs a
             for (int k = 0; k < 2 * W; ++k) acc[k] = 0;
             int pos;
             const unsigned done = gather<W, false, false, S32>(
-                a, on, v, beg, dg, t, Fd, st, acc, facc, facc, ovf, pos, [](int) {},
+                a, on, v, beg, dg, t, Fd, st, acc, facc, facc, pos, [](int) {},
                 [&](int o) {
                     if (chunk >= 0) return;  // stored below
                     unsigned nib = 0;
@@ -716,65 +749,62 @@ __global__ void __launch_bounds__(kThreads, min_ctas<W, EDGE>()) k_batch(BArgs a
             if (pos >= 0 && ((done >> pos) & 1u))
 #pragma unroll
                 for (int q = 0; q < W; ++q) nb.w[q] = st.t[pos][q];
-            join_level<W>(a, any_bits<W>(nb), v, dg, nb, act, Fn, &bc);
+            join_level<W>(a, any_bits<W>(nb), v, dg, nb, active(), Fn, &bc);
         });
-        if (a.H > 0 && !dev::grid_barrier(a.ctrl, a.limit_ns)) return;
-        trace_mark(a, ti, d, use_bu ? PH_BU_A : PH_TD_B);
+        if (a.H > 0 && !dev::grid_barrier(a.status(), a.limit_ns)) return;
+        trace_mark(a, lv.ti, d, use_bu ? PH_BU_A : PH_TD_B);
         // ---- heavy vertices sum their chunks in chunk order
         for_heavy(a, [&](int i, int h, int c0, int c1) {
-            const Bits<W> t = use_bu ? andnot<W>(act, load_bits<W>(a.vis + (size_t)h * W)) : load_bits<W>(Fn + (size_t)h * W);
+            const Bits<W> t = use_bu ? andnot<W>(active(), load_bits<W>(a.vis + (size_t)(tn + h) * W)) : load_bits<W>(Fn + (size_t)h * W);
             if (!any_bits<W>(t)) return;
             unsigned long long acc[2 * W];
 #pragma unroll
             for (int k = 0; k < 2 * W; ++k) acc[k] = 0;
+            bool ovf = false;
             sum_parts<W>(a, c0, c1, [&](int k, unsigned long long x) {
                 const unsigned long long y = acc[k] + x;
                 ovf |= y < x;
                 acc[k] = y;
             });
+            if (ovf) atomicOr(&a.status()->ovf, 1);
             unsigned nib = 0;
 #pragma unroll
             for (int k = 0; k < 2 * W; ++k) nib |= (acc[k] != 0ull ? 1u : 0u) << k;
-            store_sigma<W, S32>(a, h, nib, lane, acc);
+            store_sigma<W, S32>(a, tn + h, nib, lane, acc);
             __syncwarp();
             store_lane_bits<W>(st.t[0], nib, lane);
             __syncwarp();
             Bits<W> nb;
 #pragma unroll
             for (int q = 0; q < W; ++q) nb.w[q] = st.t[0][q];
-            join_level<W>(a, lane == 0 && any_bits<W>(nb), h, deg_of(a.rp, h), nb, act, Fn, &bc);
+            join_level<W>(a, lane == 0 && any_bits<W>(nb), h, deg_of(a.rp, h), nb, active(), Fn, &bc);
         });
         flush_counts(d + 1);
-        if (tid == 0) a.qoff[d + 1] = queued ? (int)qtail : -1;
-        if (!dev::grid_barrier(a.ctrl, a.limit_ns)) return;
-        trace_mark(a, ti, d, use_bu ? PH_BU_B : PH_TD_C);
-        const int c = __ldcg(a.vcnt + d + 1);
-        if (use_bu) {
-            ++bu;
-            qo = -1;
-            nq = c;
-        } else {
-            ++td;
-            qo = queued ? (int)qtail : -1;
-            nq = queued ? nq1 : c;
-            if (queued) qtail += nq1;
+        if (tid == 0) a.qoff[lv0 + d + 1] = queued ? (int)lv.qtail : -1;
+        if (!dev::grid_barrier(a.status(), a.limit_ns)) return;
+        trace_mark(a, lv.ti, d, use_bu ? PH_BU_B : PH_TD_C);
+        const int c = __ldcg(a.vcnt + lv0 + d + 1);
+        if (threadIdx.x == 0) {
+            use_bu ? ++lv.bu : ++lv.td;
+            lv.qo = queued ? (int)lv.qtail : -1;
+            lv.nq = queued ? nq1 : c;
+            if (queued) lv.qtail += nq1;
+            lv.mu -= (long long)__ldcg(a.dmu + lv0 + d + 1);
+            lv.mf = (long long)__ldcg(a.mfv + lv0 + d + 1);
         }
-        mu -= (long long)__ldcg(a.dmu + d + 1);
-        mf = (long long)__ldcg(a.mfv + d + 1);
         ++d;
         if (c == 0) break;
         if (d + 1 > a.lcap) {
-            if (tid == 0) atomicCAS(&a.ctrl->err, 0, kErrDepth);
+            if (tid == 0) atomicCAS(&a.status()->err, 0, kErrDepth);
             return;
         }
     }
     const int D = d - 1;
     if (tid == 0) {
-        a.ctrl->depth = D;
-        a.ctrl->td_levels = td;
-        a.ctrl->bu_levels = bu;
+        a.status()->depth = D;
+        a.status()->td_levels = lv.td;
+        a.status()->bu_levels = lv.bu;
     }
-    if (ovf) atomicOr(&a.ctrl->ovf, 1);
     if (a.rk_t) {
         // error-bounded estimate: one warp per source slot b walks one shortest path back
         // from its target, choosing each predecessor z of w with probability
@@ -784,24 +814,24 @@ __global__ void __launch_bounds__(kThreads, min_ctas<W, EDGE>()) k_batch(BArgs a
         // The slabs and sigma rows are complete: the last level ended with a grid barrier.
         const long long wid = tid >> 5, nw = nthr >> 5;
         for (long long b = wid; b < nsrc; b += nw) {
-            const int v = __ldg(a.rk_t + b);
+            const int v = __ldg(a.rk_t + (size_t)bi * B + b);
             const int q = (int)(b >> 6);
             const unsigned long long bit = 1ull << (b & 63);
             int L = -1;
             for (int l0 = 1; l0 <= D && L < 0; l0 += 32) {
                 const int l = l0 + lane;
-                const bool hit = l <= D && (__ldcg(a.F + (size_t)l * slab + (size_t)v * W + q) & bit) != 0;
+                const bool hit = l <= D && (__ldcg(level_bits(a, l, slab) + (size_t)v * W + q) & bit) != 0;
                 const unsigned m = __ballot_sync(FULL, hit);
                 if (m) L = l0 + __ffs(m) - 1;
             }
             if (L < 0) continue;  // the target is not reachable from the source
-            const unsigned long long key = __ldg(a.rk_key + b);
+            const unsigned long long key = __ldg(a.rk_key + (size_t)bi * B + b);
             int w = v;
             for (int l = L, step = 0; l > 1; --l, ++step) {
-                const unsigned long long sw = S32 ? (unsigned long long)__ldcg(a.sp32 + (size_t)w * B + b)
-                                                  : __ldcg(a.sp + (size_t)w * B + b);
+                const unsigned long long sw = S32 ? (unsigned long long)__ldcg(a.sp32 + (size_t)(tn + w) * B + b)
+                                                  : __ldcg(a.sp + (size_t)(tn + w) * B + b);
                 const unsigned long long t = dev::below(dev::stream_at(key, (uint64_t)step), sw);
-                const unsigned long long *Fp = a.F + (size_t)(l - 1) * slab;
+                const unsigned long long *Fp = level_bits(a, l - 1, slab);
                 const int end = __ldg(a.rp + w + 1);
                 unsigned long long run = 0;
                 int z = -1;
@@ -812,7 +842,7 @@ __global__ void __launch_bounds__(kThreads, min_ctas<W, EDGE>()) k_batch(BArgs a
                     if (j < end) {
                         c = __ldg(a.col + j);
                         if (__ldcg(Fp + (size_t)c * W + q) & bit)
-                            x = S32 ? (unsigned long long)__ldcg(a.sp32 + (size_t)c * B + b) : __ldcg(a.sp + (size_t)c * B + b);
+                            x = S32 ? (unsigned long long)__ldcg(a.sp32 + (size_t)(tn + c) * B + b) : __ldcg(a.sp + (size_t)(tn + c) * B + b);
                     }
                     unsigned long long incl = x;  // inclusive prefix over the lanes
 #pragma unroll
@@ -835,17 +865,17 @@ __global__ void __launch_bounds__(kThreads, min_ctas<W, EDGE>()) k_batch(BArgs a
     // ---- backward sweep, deepest level first (edge betweenness also needs level 0: the
     //      arcs from the sources carry shares, although the sources get no score)
     for (int l = D; l >= (EDGE ? 0 : 1); --l) {
-        const unsigned long long *Fl = a.F + (size_t)l * slab;
-        const unsigned long long *Fs = a.F + (size_t)(l + 1) * slab;
-        const int ql = __ldcg(a.qoff + l);
-        const int nl = ql >= 0 ? __ldcg(a.qcnt + l) : __ldcg(a.vcnt + l);
+        const unsigned long long *Fl = level_bits(a, l, slab);
+        const unsigned long long *Fs = level_bits(a, l + 1, slab);
+        const int ql = __ldcg(a.qoff + lv0 + l);
+        const int nl = ql >= 0 ? __ldcg(a.qcnt + lv0 + l) : __ldcg(a.vcnt + lv0 + l);
         // delta/psi/score of vertex v from its successor sums facc (whole warp; the lane's slots
         // nib, its path counts sg): psi_v = 1/sigma_v + acc and delta_v = sigma_v * acc (Brandes'
         // recurrence with sigma_v factored out), in double-single; the vertex's delta summed over
         // its source slots goes to the FP64 score once per vertex and level.  One warp adds to a
         // vertex's score per level, so the atomic addition, which returns nothing and is not
         // waited for, keeps the order of the additions.
-        auto finish = [&](int v, unsigned nib, const RowPart<W, S32> &sg, const dev::ff (&facc)[2 * W]) {
+        auto finish = [&](unsigned v, unsigned nib, const RowPart<W, S32> &sg, const dev::ff (&facc)[2 * W]) {
             dev::ff part = dev::ff_zero();
             unsigned long long *row = a.sp + (size_t)v * B;
 #pragma unroll
@@ -857,9 +887,9 @@ __global__ void __launch_bounds__(kThreads, min_ctas<W, EDGE>()) k_batch(BArgs a
                 }
             }
             part = dev::group_sum_ff<32>(part);
-            if (lane == 0 && part.hi != 0.0f && l > 0) atomicAdd(a.scores + v, dev::ff_to_double(part));
+            if (!EDGE && lane == 0 && part.hi != 0.0f) atomicAdd(a.scores + v, dev::ff_to_double(part));
         };
-        for_work(a, {ql, nl}, a.wq + (size_t)l * 8 + WQ_BACK, a.wq + (size_t)l * 8 + WQ_BACK_C, st.until,
+        for_work(a, {ql >= 0 ? queue_of(a) + ql : nullptr, nl}, a.wq + (lv0 + l) * 8 + WQ_BACK, st.hand,
                  [&](bool on, int v, int beg, int dg, int chunk) {
             Bits<W> t;
             if (on) {
@@ -873,10 +903,9 @@ __global__ void __launch_bounds__(kThreads, min_ctas<W, EDGE>()) k_batch(BArgs a
             RowPart<W, S32> sg;
 #pragma unroll
             for (int k = 0; k < 2 * W; ++k) facc[k] = dev::ff_zero();
-            bool dummy = false;
             int pos;
             const unsigned done = gather<W, true, EDGE, false>(
-                a, on, v, beg, dg, t, Fs, st, acc, facc, sv, dummy, pos,
+                a, on, v, beg, dg, t, Fs, st, acc, facc, sv, pos,
                 [&](int o) {
                     if (!EDGE && chunk >= 0) return;
                     const unsigned nib = lane_bits<W>(st.t[o], lane);
@@ -911,22 +940,22 @@ __global__ void __launch_bounds__(kThreads, min_ctas<W, EDGE>()) k_batch(BArgs a
                     if ((nib >> k) & 1u) row[slot_off<W>(k, lane)] = dev::ff_pack(dev::ff_rcp(sg.count(k)));
             }
         });
-        if (a.H > 0 && !dev::grid_barrier(a.ctrl, a.limit_ns)) return;
-        trace_mark(a, ti, l, PH_BK_A);
+        if (a.H > 0 && !dev::grid_barrier(a.status(), a.limit_ns)) return;
+        trace_mark(a, lv.ti, l, PH_BK_A);
         for_heavy(a, [&](int i, int h, int c0, int c1) {
             const Bits<W> mv = load_bits<W>(Fl + (size_t)h * W);
             if (!any_bits<W>(mv)) return;
             const unsigned nib = (unsigned)(lane_word<W>(mv, lane) >> ((2 * W * lane) & 63)) & ((1u << (2 * W)) - 1u);
             RowPart<W, S32> sg;
-            sg.load(a, h, lane, nib);
+            sg.load(a, tn + h, lane, nib);
             dev::ff facc[2 * W];
 #pragma unroll
             for (int k = 0; k < 2 * W; ++k) facc[k] = dev::ff_zero();
             sum_parts<W>(a, c0, c1, [&](int k, unsigned long long x) { facc[k] = dev::ff_add(facc[k], dev::ff_unpack(x)); });
-            finish(h, nib, sg, facc);
+            finish(tn + h, nib, sg, facc);
         });
-        if (!dev::grid_barrier(a.ctrl, a.limit_ns)) return;
-        trace_mark(a, ti, l, PH_BK_B);
+        if (!dev::grid_barrier(a.status(), a.limit_ns)) return;
+        trace_mark(a, lv.ti, l, PH_BK_B);
     }
 }
 
@@ -966,14 +995,16 @@ int64_t chunk_count(const nk_graph *g, int chunk)
     return g->A / chunk + (g->max_deg > chunk ? g->n : 0);
 }
 
-Layout layout(const nk_graph *g, int B, int lcap, int chunk = 0)
+// The workspace of `teams` teams, array by array (so that a team's rows are an offset of the row
+// number and not of a pointer).
+Layout layout(const nk_graph *g, int B, int lcap, int chunk = 0, int teams = 1)
 {
     Layout L;
     L.B = B;
     L.W = B / 64;
     L.lcap = lcap;
-    L.qcap = 2 * (int64_t)g->n + 64;
-    const size_t n = (size_t)g->n;
+    L.qcap = 2 * (int64_t)g->n + B;  // level 0 may hold a vertex several times (drawn pairs)
+    const size_t n = (size_t)g->n * teams;
     size_t o = 0;
     L.off_F = o;
     o = align_up(o + (size_t)(lcap + 2) * n * L.W * 8);
@@ -986,11 +1017,11 @@ Layout layout(const nk_graph *g, int B, int lcap, int chunk = 0)
     L.off_qmark = o;
     o = align_up(o + n * 4);
     L.off_queue = o;
-    o = align_up(o + (size_t)L.qcap * 4);
+    o = align_up(o + (size_t)L.qcap * 4 * teams);
     L.off_cnt = o;
-    o = align_up(o + (size_t)(lcap + 3) * (3 * 4 + 2 * 8 + 8 * 4));
+    o = align_up(o + (size_t)(lcap + 3) * (3 * 4 + 2 * 8 + 8 * 4) * teams);
     L.off_part = o;
-    o = align_up(o + (size_t)chunk_count(g, chunk) * B * 8);
+    o = align_up(o + (size_t)chunk_count(g, chunk) * B * 8 * teams);
     L.total = o;
     return L;
 }
@@ -1011,6 +1042,102 @@ int choose_lcap(const nk_graph *g, int B, const DevBuf *ws, int chunk = 0)
 }
 
 enum { WS_BATCH = 5, WS_BCTRL = 6 };
+
+constexpr int kMaxTeams = 64;
+constexpr size_t kTeamRows = 3300u << 20;  // bytes of sigma and psi rows that teams share
+constexpr int kTeamCtas = 128, kTeamVertices = 64;
+
+// Batches run side by side, each by a team of blocks with its own state: one batch of a small graph
+// cannot use the GPU, and on the others teams fill the tails of each other's phases.  As many as
+// there are batches while their rows stay within kTeamRows together, beyond which they only take
+// memory and cache from each other.  1, 2, 4, 8 and all batches at once, 128 sources each: ER 2000
+// exact 3.3, 1.7, 0.87, 0.60, 0.46 ms; R-MAT 14 3.7, 2.3, 1.25, 0.98; R-MAT 18 (6) 13.2, 10.6,
+// 10.0, -, 9.8; BA 10^6 (4) 31.5, 29.9, 30.0; R-MAT 20 36.2, 34.4, 35.8, 40.3; R-MAT 22 133, 132,
+// 136, 146; R-MAT 24 320, 320.  The number of teams per launch is evened out; the batches stay full and
+// the last one short (made equal, R-MAT 18 takes 12.9 instead of 11.3 ms: a row read serves fewer).  Callers with their
+// own workspace or grid (servers, captured graphs) run one batch at a time.
+int choose_teams(const nk_graph *g, int B, size_t state, int nb, int grid, const RunCfg &cfg, const DevBuf *ws, int64_t outs)
+{
+    if (cfg.ws || cfg.grid_ctas > 0 || nb < 2) return 1;
+    const size_t rows = (size_t)g->n * B * 12;
+    int want = (int)std::min<size_t>(std::min(nb, std::min(kMaxTeams, grid)), (kTeamRows + rows - 1) / rows);
+    size_t free_b = 0, total_b = 0;
+    cudaMemGetInfo(&free_b, &total_b);
+    const size_t per = state + sizeof(double) * (size_t)outs;
+    while (want > 1 && per * want > (free_b + ws[WS_BATCH].bytes) / 4) --want;
+    while (want > 1 && (int64_t)g->n * want > INT32_MAX) --want;  // rows are numbered in 32 bits
+    const int rounds = (nb + want - 1) / want;
+    return (nb + rounds - 1) / rounds;
+}
+
+// Blocks of a team: its share of the grid, but no more than a small graph can use, whose barriers get
+// dearer with every block (ER 2000, one batch of 64: 128 blocks 0.185 ms, 608 0.209; R-MAT 14:
+// 256 0.459, 608 0.509; ER 50000: 256 0.650, 608 0.596).
+int team_ctas(const nk_graph *g, int grid, int teams) { return std::min(grid / teams, std::max(kTeamCtas, g->n / kTeamVertices)); }
+
+// Sources per batch where neither the caller nor the autotuner chose: 128 if there are more than 128
+// and their state fits, else 64 (64 against 128, ms: ER 200003 k = 300 4.53 / 4.30, R-MAT 16 3.54 /
+// 3.44, R-MAT 18 11.1 / 9.8, BA 20000 1.68 / 1.58, R-MAT 20 40.3 / 34.4: the 128-source kernel
+// gathers 64 % of the rows; but up to 128 sources two batches of 64 side by side are better than
+// one: R-MAT 18 from its edge list with k = 128 7.3 / 8.0).
+int default_width(const nk_graph *g, int32_t k, const RunCfg &cfg)
+{
+    return k > 128 && choose_lcap(g, 128, scratch(cfg, const_cast<nk_graph *>(g)), cfg.chunk) >= std::min(kStartLevels, std::max(g->n, 4)) ? 128 : 64;
+}
+
+// The arguments that do not depend on the batch: graph, workspace at `base`, options.
+BArgs make_args(const nk_graph *g, const Layout &L, int teams, const HeavyView &hw, char *base, double *d_scores,
+                const RunCfg &cfg)
+{
+    BArgs a{};
+    a.n = g->n;
+    a.A = g->A;
+    a.rp = g->rp.as<int32_t>();
+    a.col = g->col.as<int32_t>();
+    a.lcap = L.lcap;
+    a.F = reinterpret_cast<unsigned long long *>(base + L.off_F);
+    a.vis = reinterpret_cast<unsigned long long *>(base + L.off_vis);
+    a.sp = reinterpret_cast<unsigned long long *>(base + L.off_sp);
+    a.sp32 = reinterpret_cast<unsigned *>(base + L.off_sp32);
+    a.qmark = reinterpret_cast<int32_t *>(base + L.off_qmark);
+    a.queue = reinterpret_cast<int32_t *>(base + L.off_queue);
+    a.qcap = L.qcap;
+    const size_t lv = ((size_t)L.lcap + 3) * teams;
+    char *cb = base + L.off_cnt;
+    a.mfv = reinterpret_cast<unsigned long long *>(cb);
+    a.dmu = a.mfv + lv;
+    a.vcnt = reinterpret_cast<int32_t *>(a.dmu + lv);
+    a.qcnt = a.vcnt + lv;
+    a.qoff = a.qcnt + lv;
+    a.wq = a.qoff + lv;
+    a.scores = d_scores;
+    a.hv = hw.hv;
+    a.hfirst = hw.hfirst;
+    a.chunk_h = hw.chunk_h;
+    a.H = hw.H;
+    a.C = hw.C;
+    a.chunk = hw.chunk;
+    a.part = reinterpret_cast<unsigned long long *>(base + L.off_part);
+    a.backward = cfg.backward ? 1 : 0;
+    a.edge = cfg.edge && cfg.backward ? cfg.edge : nullptr;
+    a.rk_t = cfg.rk_t;
+    a.rk_key = cfg.rk_key;
+    a.rk_count = cfg.rk_count;
+    a.limit_ns = cfg.limit_ns ? cfg.limit_ns : wait_limit_ns();
+    a.alpha = cfg.alpha > 0 ? cfg.alpha : 1.0;
+    a.dir = cfg.direction;
+    return a;
+}
+
+// out[i] += the teams' sums, in their order
+__global__ void k_add_teams(const double *t, int32_t teams, int64_t count, double *out)
+{
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
+        double x = out[i];
+        for (int32_t j = 0; j < teams; ++j) x += t[(size_t)j * count + i];
+        out[i] = x;
+    }
+}
 
 template <int W>
 int launch_batches(nk_graph *g, const int32_t *d_src, int32_t k, double *d_scores,
@@ -1077,7 +1204,9 @@ int launch_batches(nk_graph *g, const int32_t *d_src, int32_t k, double *d_score
     Ctrl *ctrls = ws[WS_BCTRL].as<Ctrl>();
     std::vector<int> todo(nb);
     for (int bi = 0; bi < nb; ++bi) todo[bi] = bi;
-    double alpha_used = cfg.alpha > 0 ? cfg.alpha : 1.0;
+    const double alpha_used = cfg.alpha > 0 ? cfg.alpha : 1.0;
+    // entries of the sums that the batches add to: per-arc shares, scores, or none
+    const int64_t a_out = edge ? g->A : cfg.backward ? g->n : 0;
     static const bool trace_on = std::getenv("NK_TRACE") != nullptr;
     Tmp trace_buf;
     if (trace_on) {
@@ -1085,45 +1214,20 @@ int launch_batches(nk_graph *g, const int32_t *d_src, int32_t k, double *d_score
         NK_CUDA(cudaMemsetAsync(trace_buf.p, 0, sizeof(unsigned long long) * 2 * kTraceCap, s));
     }
     for (int lcap = lstart;;) {
-        const Layout L = layout(g, B, lcap, hw.chunk);
+        // reruns of some of the batches go one by one
+        const int teams = (int)todo.size() == nb ? choose_teams(g, B, layout(g, B, lcap, hw.chunk).total, nb, grid, cfg, ws, a_out) : 1;
+        const Layout L = layout(g, B, lcap, hw.chunk, teams);
         NK_TRY(ws[WS_BATCH].ensure(L.total));
-        char *base = ws[WS_BATCH].as<char>();
-        BArgs a{};
-        a.n = g->n;
-        a.A = g->A;
-        a.rp = g->rp.as<int32_t>();
-        a.col = g->col.as<int32_t>();
-        a.lcap = lcap;
-        a.F = reinterpret_cast<unsigned long long *>(base + L.off_F);
-        a.vis = reinterpret_cast<unsigned long long *>(base + L.off_vis);
-        a.sp = reinterpret_cast<unsigned long long *>(base + L.off_sp);
-        a.sp32 = reinterpret_cast<unsigned *>(base + L.off_sp32);
-        a.qmark = reinterpret_cast<int32_t *>(base + L.off_qmark);
-        a.queue = reinterpret_cast<int32_t *>(base + L.off_queue);
-        a.qcap = L.qcap;
-        const size_t lv = (size_t)lcap + 3;
-        char *cb = base + L.off_cnt;
-        a.mfv = reinterpret_cast<unsigned long long *>(cb);
-        a.dmu = a.mfv + lv;
-        a.vcnt = reinterpret_cast<int32_t *>(a.dmu + lv);
-        a.qcnt = a.vcnt + lv;
-        a.qoff = a.qcnt + lv;
-        a.wq = a.qoff + lv;
-        a.scores = d_scores;
-        a.hv = hw.hv;
-        a.hfirst = hw.hfirst;
-        a.chunk_h = hw.chunk_h;
-        a.H = hw.H;
-        a.C = hw.C;
-        a.chunk = hw.chunk;
-        a.part = reinterpret_cast<unsigned long long *>(base + L.off_part);
-        a.trace = nullptr;
-        a.backward = cfg.backward ? 1 : 0;
-        a.edge = edge ? cfg.edge : nullptr;
-        a.rk_count = cfg.rk_count;
-        a.limit_ns = cfg.limit_ns ? cfg.limit_ns : wait_limit_ns();
-        a.alpha = alpha_used;
-        a.dir = cfg.direction;
+        BArgs a = make_args(g, L, teams, hw, ws[WS_BATCH].as<char>(), d_scores, cfg);
+        a.src = d_src;
+        a.nsrc = k;
+        a.ctrl = ctrls;
+        Tmp outs;
+        if (teams > 1 && a_out > 0) {
+            NK_TRY(outs.alloc(sizeof(double) * (size_t)a_out * teams, s));
+            NK_CUDA(cudaMemsetAsync(outs.p, 0, sizeof(double) * (size_t)a_out * teams, s));
+            (edge ? a.edge : a.scores) = outs.as<double>();
+        }
         NK_CUDA(cudaMemsetAsync(ctrls, 0, sizeof(Ctrl) * nb, s));
         cudaEvent_t e0 = nullptr, e1 = nullptr;
         if (cfg.time_kernels) {
@@ -1131,18 +1235,19 @@ int launch_batches(nk_graph *g, const int32_t *d_src, int32_t k, double *d_score
             NK_CUDA(cudaEventCreate(&e1));
             NK_CUDA(cudaEventRecord(e0, s));
         }
-        a.ksrc = nullptr;
-        a.boff = 0;
-        for (int bi : todo) {
-            a.src = d_src + (size_t)bi * B;
-            a.nsrc = std::min(B, k - bi * B);
-            a.ctrl = ctrls + bi;
-            a.rk_t = cfg.rk_t ? cfg.rk_t + (size_t)bi * B : nullptr;
-            a.rk_key = cfg.rk_key ? cfg.rk_key + (size_t)bi * B : nullptr;
-            a.trace = (trace_on && bi == todo.front()) ? trace_buf.as<unsigned long long>() : nullptr;
+        for (size_t t = 0; t < todo.size(); t += teams) {
+            a.b0 = todo[t];
+            a.trace = (trace_on && t == 0) ? trace_buf.as<unsigned long long>() : nullptr;
+            const int now = std::min<int>(teams, (int)(todo.size() - t));  // the last launch's teams are larger
             void *args[] = {&a};
-            NK_CUDA(cudaLaunchCooperativeKernel(kfn, dim3(grid), dim3(kThreads), args, edge ? smem_bytes<W, true>() : smem_bytes<W, false>(), s));
+            NK_CUDA(cudaLaunchCooperativeKernel(kfn, dim3(team_ctas(g, grid, now), now), dim3(kThreads), args, edge ? smem_bytes<W, true>() : smem_bytes<W, false>(), s));
             ::nk::count_launch();
+        }
+        if (outs.p) {
+            const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((a_out + 255) / 256, 8LL * num_sms()));
+            k_add_teams<<<blocks, 256, 0, s>>>(outs.as<double>(), teams, a_out, edge ? cfg.edge : d_scores);
+            ::nk::count_launch();
+            NK_CUDA(cudaGetLastError());
         }
         if (cfg.time_kernels) NK_CUDA(cudaEventRecord(e1, s));
         std::vector<Ctrl> h(nb);
@@ -1264,45 +1369,8 @@ int enqueue_batches(nk_graph *g, const int32_t *d_src, int32_t k, double *d_scor
     if (bps < 1) return set_error(NK_ERR_CUDA, "batched kernel cannot be resident");
     int grid = std::max(1, bps * num_sms() / std::max(1, cfg.grid_div));
     if (cfg.grid_ctas > 0) grid = std::min(grid, cfg.grid_ctas);
-    char *base = ws[WS_BATCH].as<char>();
-    BArgs a{};
-    a.n = g->n;
-    a.A = g->A;
-    a.rp = g->rp.as<int32_t>();
-    a.col = g->col.as<int32_t>();
-    a.lcap = lcap;
-    a.F = reinterpret_cast<unsigned long long *>(base + L.off_F);
-    a.vis = reinterpret_cast<unsigned long long *>(base + L.off_vis);
-    a.sp = reinterpret_cast<unsigned long long *>(base + L.off_sp);
-    a.sp32 = reinterpret_cast<unsigned *>(base + L.off_sp32);
-    a.qmark = reinterpret_cast<int32_t *>(base + L.off_qmark);
-    a.queue = reinterpret_cast<int32_t *>(base + L.off_queue);
-    a.qcap = L.qcap;
-    const size_t lv = (size_t)lcap + 3;
-    char *cb = base + L.off_cnt;
-    a.mfv = reinterpret_cast<unsigned long long *>(cb);
-    a.dmu = a.mfv + lv;
-    a.vcnt = reinterpret_cast<int32_t *>(a.dmu + lv);
-    a.qcnt = a.vcnt + lv;
-    a.qoff = a.qcnt + lv;
-    a.wq = a.qoff + lv;
-    a.scores = d_scores;
-    a.hv = hw.hv;
-    a.hfirst = hw.hfirst;
-    a.chunk_h = hw.chunk_h;
-    a.H = hw.H;
-    a.C = hw.C;
-    a.chunk = hw.chunk;
-    a.part = reinterpret_cast<unsigned long long *>(base + L.off_part);
-    a.trace = nullptr;
-    a.backward = cfg.backward ? 1 : 0;
+    BArgs a = make_args(g, L, 1, hw, ws[WS_BATCH].as<char>(), d_scores, cfg);
     a.edge = nullptr;  // the captured form serves vertex scores only
-    a.rk_t = nullptr;
-    a.rk_key = nullptr;
-    a.rk_count = nullptr;
-    a.limit_ns = cfg.limit_ns ? cfg.limit_ns : wait_limit_ns();
-    a.alpha = cfg.alpha > 0 ? cfg.alpha : 1.0;
-    a.dir = cfg.direction;
     Ctrl *ctrls = ws[WS_BCTRL].as<Ctrl>();
     int32_t *csrc = reinterpret_cast<int32_t *>(ws[WS_BCTRL].as<char>() + ctrl_bytes);
     int32_t *ccnt = reinterpret_cast<int32_t *>(ws[WS_BCTRL].as<char>() + ctrl_bytes + src_bytes);
@@ -1315,7 +1383,10 @@ int enqueue_batches(nk_graph *g, const int32_t *d_src, int32_t k, double *d_scor
         NK_TRY(order_sources(g, csrc, k, ccnt, reinterpret_cast<unsigned long long *>(ob + src_bytes), osrc, s));
         csrc = osrc;
     }
+    a.src = csrc;
+    a.nsrc = k;
     a.ksrc = ccnt;
+    a.ctrl = ctrls;
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeCooperative;
     attr.val.cooperative = 1;
@@ -1327,10 +1398,7 @@ int enqueue_batches(nk_graph *g, const int32_t *d_src, int32_t k, double *d_scor
     lc.attrs = &attr;
     lc.numAttrs = 1;
     for (int bi = 0; bi < nb; ++bi) {
-        a.src = csrc + (size_t)bi * B;
-        a.nsrc = std::min(B, k - bi * B);
-        a.boff = bi * B;
-        a.ctrl = ctrls + bi;
+        a.b0 = bi;
         void *args[] = {&a};
         NK_CUDA(cudaLaunchKernelExC(&lc, (const void *)k_batch<W, false, true>, args));
         ::nk::count_launch();
@@ -1350,7 +1418,7 @@ int run_batched(nk_graph *g, const int32_t *d_src, int32_t k, double *d_scores,
                 const RunCfg &cfg, RunStats *st, cudaStream_t s)
 {
     int B = cfg.batch;
-    if (B == 0) B = g->tuned.valid ? g->tuned.batch : 64;
+    if (B == 0) B = g->tuned.valid ? g->tuned.batch : default_width(g, k, cfg);
     switch (B) {
     case 64: return launch_batches<1>(g, d_src, k, d_scores, cfg, st, s);
     case 128: return launch_batches<2>(g, d_src, k, d_scores, cfg, st, s);

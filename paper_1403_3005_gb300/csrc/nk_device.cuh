@@ -177,7 +177,7 @@ __device__ __forceinline__ ff ff_from_u64(unsigned long long x)
 __device__ __forceinline__ ff ff_from_u32(unsigned x)
 {
     const float hi = __uint2float_rz(x);
-    return {hi, __uint2float_rn(x - __float2uint_rz(hi))};  // exact: the remainder has at most 8 bits
+    return ff_fast2sum(hi, __uint2float_rn(x - __float2uint_rz(hi)));  // exact: the remainder has at most 8 bits
 }
 
 __device__ __forceinline__ double ff_to_double(ff a) { return (double)a.hi + (double)a.lo; }

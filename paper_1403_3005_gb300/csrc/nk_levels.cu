@@ -55,6 +55,8 @@ struct LArgs {
     int32_t chunk;
     const int32_t *hv, *hfirst, *chunk_h;
     int32_t H, C;
+
+    __device__ __forceinline__ Ctrl *status() const { return ctrl; }
 };
 
 // One warp's shared memory: a group's vertices.
@@ -62,7 +64,7 @@ template <int W> struct GroupBuf {
     unsigned long long t[32][W];  // bits a vertex waits for (bottom-up) or pushes (top-down)
     unsigned long long f[32][W];  // bits found so far
     int off[32];                  // first arc, less the arcs of the vertices before
-    unsigned long long until;     // deadline of the phase
+    Hand hand;
 };
 
 // Lane L's vertex w (where `on`) joins level d+1 for the sources nb.
@@ -166,7 +168,7 @@ template <int W> __global__ void __launch_bounds__(kThreads, 4) k_levels(LArgs a
         const bool use_bu = a.dir == NK_DIR_BOTTOM_UP ||
                             (a.dir == NK_DIR_AUTO && a.alpha * (double)mf > (double)mu);
         if (use_bu) {
-            for_work(a, {-1, a.n}, wq + WQ_BU, wq + WQ_BU_C, st.until, [&](bool on, int v, int beg, int dg, int chunk) {
+            for_work(a, {nullptr, a.n}, wq + WQ_BU, st.hand, [&](bool on, int v, int beg, int dg, int chunk) {
                 Bits<W> t;
                 if (on) {
                     t = andnot<W>(act, load_bits<W>(a.vis + (size_t)v * W));
@@ -249,8 +251,8 @@ template <int W> __global__ void __launch_bounds__(kThreads, 4) k_levels(LArgs a
             ++bu;
         } else {
             int32_t *qnext = a.queue + (size_t)((d + 1) & 1) * a.n;
-            const int qo = queued ? (int)(d & 1) * a.n : -1;
-            for_work(a, {qo, nq}, wq + WQ_PUSH, wq + WQ_PUSH_C, st.until, [&](bool on, int v, int beg, int dg, int) {
+            for_work(a, {queued ? a.queue + (size_t)(d & 1) * a.n : nullptr, nq}, wq + WQ_PUSH, st.hand,
+                     [&](bool on, int v, int beg, int dg, int) {
                 Bits<W> t;
                 if (on) {
                     t = load_bits<W>(Fd + (size_t)v * W);

@@ -1,8 +1,8 @@
 // Parts shared by the kernels that sweep a graph level by level for a batch of sources: bitsets
 // of W 64-bit words (one bit per source), the hand-out of a phase's work to warps, and the walk
 // over the concatenated arcs of a group of vertices.  `Args` is a kernel's argument structure;
-// the fields used here are n, A, rp, col, queue, ctrl, limit_ns and the chunk table (chunk, hv,
-// hfirst, chunk_h, H, C).
+// the members used here are n, A, rp, limit_ns, the chunk table (chunk, hv, hfirst, chunk_h, H, C)
+// and status(), the control words of the block's sweep.  The warps that share a sweep are those of gridDim.x blocks (a team, blockIdx.y).
 #pragma once
 
 #include "nk_device.cuh"
@@ -68,12 +68,11 @@ __device__ __forceinline__ int deg_of(const int32_t *rp, int v) { return __ldg(r
 
 // Records the first failed device-side check (code, where, offending value); every CTA
 // then leaves at its next grid barrier and the host reports the status.
-template <class Args>
-__device__ __forceinline__ void check_failed(const Args &a, int code, int where, int value)
+__device__ __forceinline__ void check_failed(Ctrl *ctrl, int code, int where, int value)
 {
-    if (atomicCAS(&a.ctrl->err, 0, code) == 0) {
-        a.ctrl->where = where;
-        a.ctrl->bad_id = value;
+    if (atomicCAS(&ctrl->err, 0, code) == 0) {
+        ctrl->where = where;
+        ctrl->bad_id = value;
     }
 }
 
@@ -104,46 +103,53 @@ template <class Args> __device__ __forceinline__ int grab_size(const Args &a, in
     return most >= kGrabV ? kGrabV : most <= 1 ? 1 : 1 << (31 - __clz(most));
 }
 
-// How a phase finds its vertices: entries [qo, qo + nq) of the queue, or a scan of all
-// vertices (the callee looks at their bits).  nq: the number of vertices expected.
+// How a phase finds its vertices: the nq entries of a queue, or (null) a scan of all vertices, whose
+// bits the callee looks at (nq: the number of vertices expected).
 struct Level {
-    int qo;   // -1: scan
+    const int32_t *queue;
     int nq;
+};
+
+// A warp's place in the hand-out of a phase's work, in shared memory (lane 0 writes it).
+struct Hand {
+    unsigned long long until;  // deadline of the phase
+    int c, cend;               // the grabbed chunks left
 };
 
 // Calls fn(on, v, beg, dg, chunk) with the whole warp for all work of a phase.  First the
 // chunks of the heavy vertices, whose work is largest (chunk >= 0: lane 0 holds the vertex and
 // the chunk's arcs), then groups of light vertices, one per lane (chunk = -1).  Warps take work
-// dynamically from the two zeroed counters, each grab requested while the one before is worked
+// dynamically from two zeroed counters (ctr[0] vertices, ctr[1] chunks), each grab requested while the one before is worked
 // on; scans of sparse levels (under n/32 vertices) are static.  Loops are bounded in time: lane
-// 0 checks the phase's deadline (kept in shared memory) once per item and the warp leaves together (the status is read
+// 0 checks the phase's deadline once per item and the warp leaves together (the status is read
 // at the next barrier).
 template <class Args, class Fn>
-__device__ __forceinline__ void for_work(const Args &a, Level lv, int32_t *ctr, int32_t *ctr_c,
-                                         unsigned long long &deadline, Fn fn)
+__device__ __forceinline__ void for_work(const Args &a, Level lv, int32_t *ctr, Hand &hand, Fn fn)
 {
     const int lane = threadIdx.x & 31;
     const int nw = (int)(((long long)gridDim.x * blockDim.x) >> 5);
-    if (lane == 0) deadline = dev::globaltimer() + a.limit_ns;
+    if (lane == 0) {
+        hand.until = dev::globaltimer() + a.limit_ns;
+        hand.c = hand.cend = 0;
+    }
+    __syncwarp();
     // about C / (32 warps) chunks per grab, 1..16: few chunks stay spread over many warps,
     // millions of chunks cost few atomics
-    const int gc = max(1, min(kGrabCMax, a.C / (32 * nw)));
-    const bool fixed = lv.qo < 0 && lv.nq < a.n / 32;
-    const int gv = fixed ? kGrabV : grab_size(a, lv.qo >= 0 ? lv.nq : a.n, nw);
-    const int step = fixed ? nw * kGrabV : 0;
-    const unsigned end = lv.qo >= 0 ? lv.nq : a.n;
-    int c = 0, cend = 0;
+    auto chunk_grab = [&]() { return max(1, min(kGrabCMax, a.C / (32 * nw))); };
+    const bool fixed = !lv.queue && lv.nq < a.n / 32;
+    const int gv = fixed ? kGrabV : grab_size(a, lv.queue ? lv.nq : a.n, nw);
+    const unsigned end = lv.queue ? lv.nq : a.n;
     unsigned next = 0;  // lane 0: the grab under way
     bool chunks = a.C > 0;
     auto grab = [&]() {
         if (lane == 0) {
-            if (chunks) next = (unsigned)atomicAdd(ctr_c, gc);
-            else next = step ? next + step : (unsigned)atomicAdd(ctr, gv);
+            if (chunks) next = (unsigned)atomicAdd(ctr + 1, chunk_grab());
+            else next = fixed ? next + nw * kGrabV : (unsigned)atomicAdd(ctr, gv);
         }
     };
-    auto first = [&]() {  // of the scan
-        if (lane == 0) next = step ? (unsigned)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kGrabV
-                                   : (unsigned)atomicAdd(ctr, gv);
+    auto first = [&]() {  // of the vertices
+        if (lane == 0) next = fixed ? (unsigned)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * kGrabV
+                                    : (unsigned)atomicAdd(ctr, gv);
     };
     if (chunks) grab();
     else first();
@@ -151,30 +157,35 @@ __device__ __forceinline__ void for_work(const Args &a, Level lv, int32_t *ctr, 
         bool on = false;
         int v = 0, beg = 0, dg = 0, chunk = -1;
         if (chunks) {
-            if (c >= cend) {
+            int c = hand.c;
+            if (c >= hand.cend) {
                 c = __shfl_sync(FULL, (int)next, 0);
                 if (c >= a.C) {
                     chunks = false;
                     first();
                     continue;
                 }
-                cend = min(c + gc, a.C);
+                __syncwarp();
+                if (lane == 0) hand.cend = min(c + chunk_grab(), a.C);
                 grab();
             }
+            __syncwarp();
+            if (lane == 0) hand.c = c + 1;
+            __syncwarp();
             const int i = __ldg(a.chunk_h + c);
             v = __ldg(a.hv + i);
             beg = __ldg(a.rp + v) + (c - __ldg(a.hfirst + i)) * a.chunk;
             dg = min(a.chunk, __ldg(a.rp + v + 1) - beg);
             on = lane == 0;
-            chunk = c++;
+            chunk = c;
         } else {
             const unsigned i = __shfl_sync(FULL, next, 0) + lane;
             if (i - lane >= end) break;
             grab();
             on = lane < gv && i < end;
-            if (on) v = lv.qo >= 0 ? __ldcg(a.queue + lv.qo + i) : (int)i;
+            if (on) v = lv.queue ? __ldcg(lv.queue + i) : (int)i;
             if (on && (unsigned)v >= (unsigned)a.n) {
-                check_failed(a, kErrCheck, 3, v);
+                check_failed(a.status(), kErrCheck, 3, v);
                 on = false;
             }
             if (on) {
@@ -184,8 +195,8 @@ __device__ __forceinline__ void for_work(const Args &a, Level lv, int32_t *ctr, 
             }
         }
         int late = 0;
-        if (lane == 0 && dev::globaltimer() > deadline) {
-            check_failed(a, NK_ERR_TIMEOUT, 2, lv.nq);
+        if (lane == 0 && dev::globaltimer() > hand.until) {
+            check_failed(a.status(), NK_ERR_TIMEOUT, 2, lv.nq);
             late = 1;
         }
         if (__shfl_sync(FULL, late, 0)) break;

@@ -96,3 +96,33 @@ def test_closeness_levels(nk, batch):
             far, reach = nk.closeness_sampled(g, 8, k, nk.run_opts(mode=nk.MODE_BATCHED, batch=batch, direction=direction))
             assert np.array_equal(far, np.abs(i[:, None] - src).sum(1) * (n / k))
             assert np.array_equal(reach, (i[:, None] != src).sum(1) * (n / k))
+
+
+@pytest.mark.parametrize("direction", [0, 1, 2])
+def test_more_sources_than_vertices(nk, direction):
+    """Pairs are drawn with repetitions: a batch of 256 of them on 40 vertices."""
+    n, u, v = G.path(40)
+    rp, col = oracle.csr_build(n, u, v)
+    want, r, vd = oracle.betweenness_rk(rp, col, 0.1, 0.1, 7)
+    g = nk.graph_from_edges(n, u, v)
+    for batch in (64, 256):
+        got, r1, vd1 = nk.betweenness_rk(g, 0.1, 0.1, 7, nk.run_opts(mode=nk.MODE_BATCHED, batch=batch, direction=direction))
+        assert (r1, vd1) == (r, vd) and np.array_equal(got, want)
+
+
+@pytest.mark.parametrize("k", [65, 128, 192, 300])
+def test_batches_side_by_side(nk, k):
+    """Several batches of a small graph run in one launch, by teams with their own state and sums:
+    2, 2, 3 and 5 batches of 64, the last one full or not, for vertex and edge scores, drawn pairs
+    and counts that need 64-bit rows in some of the batches."""
+    n, u, v = G.disjoint_union(G.gnp(400, 0.02, 11), G.grid(24, 24), G.star(300))
+    g = nk.graph_from_edges(n, u, v)
+    rp, col = oracle.csr_build(n, u, v)
+    o = nk.run_opts(mode=nk.MODE_BATCHED, batch=64)
+    assert np.allclose(nk.betweenness_sampled(g, 3, k, o), oracle.betweenness_sampled(rp, col, 3, k), rtol=1e-9, atol=1e-12)
+    assert np.allclose(nk.edge_betweenness_sampled(g, 3, k, o), oracle.edge_betweenness_sampled(rp, col, 3, k),
+                       rtol=1e-9, atol=1e-12)
+    assert nk.last_run_stats()["launches"] >= (k + 63) // 64
+    want, r, _ = oracle.betweenness_rk(rp, col, 0.15, 0.1, 7)
+    got, r1, _ = nk.betweenness_rk(g, 0.15, 0.1, 7, o)
+    assert r1 == r and np.array_equal(got, want)
