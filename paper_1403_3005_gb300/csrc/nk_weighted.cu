@@ -25,6 +25,7 @@
 
 #include <algorithm>
 #include <climits>
+#include <type_traits>
 #include <vector>
 
 #include "nk_device.cuh"
@@ -35,6 +36,7 @@ namespace {
 
 constexpr int kThreads = 512;
 constexpr long long kInf = LLONG_MAX;
+constexpr int kShortRow = 32;  // arcs up to which a row is walked by 8 lanes
 
 struct WArgs {
     int32_t n;
@@ -59,11 +61,6 @@ struct WArgs {
     int32_t H, C;
 };
 
-__device__ __forceinline__ bool heavy(const WArgs &a, int v)
-{
-    return a.H > 0 && __ldg(a.rp + v + 1) - __ldg(a.rp + v) > kHeavyChunk;
-}
-
 // Chunk c of a heavy vertex: its vertex h and arc range [j0, j1).
 __device__ __forceinline__ void chunk_of(const WArgs &a, long long c, int &h, int &j0, int &j1)
 {
@@ -76,6 +73,28 @@ __device__ __forceinline__ void chunk_of(const WArgs &a, long long c, int &h, in
 __device__ __forceinline__ long long ld_dist(const long long *p)
 {
     return *reinterpret_cast<const volatile long long *>(p);
+}
+
+// fn(c, h, j0, j1), with the whole warp, for every chunk of a heavy vertex at distance D; the chunks
+// wid, wid + nw, ... are the warp's.  Few heavy vertices are in one bucket, so the lanes look at the
+// vertices of 32 of the warp's chunks at once and only the chunks of the bucket are walked.  (One by
+// one, every bucket paid the chain chunk -> vertex -> distance C / nw times over, forward and
+// backward.)
+template <class Fn>
+__device__ __forceinline__ void for_bucket_chunks(const WArgs &a, long long D, long long wid, long long nw, Fn fn)
+{
+    const int lane = threadIdx.x & 31;
+    for (long long c0 = wid; c0 < a.C; c0 += 32 * nw) {
+        const long long mine = c0 + lane * nw;
+        bool in = false;
+        if (mine < a.C) in = ld_dist(a.dist + __ldg(a.hv + __ldg(a.chunk_h + mine))) == D;
+        for (unsigned m = __ballot_sync(0xffffffffu, in); m; m &= m - 1) {
+            const long long c = c0 + (__ffs(m) - 1) * nw;
+            int h, j0, j1;
+            chunk_of(a, c, h, j0, j1);
+            fn(c, h, j0, j1);
+        }
+    }
 }
 
 // Barrier over the `count` CTAs of one group, bounded like the grid barrier: after limit_ns
@@ -114,6 +133,32 @@ __device__ __forceinline__ bool group_barrier(Ctrl *ctrl, unsigned count, uint64
     }
     __syncthreads();
     return s_ok != 0;
+}
+
+// fn(v, j0, j1, l0, wide) for the light vertices of a bucket: four at a time, 8 lanes each, then, with
+// the whole warp, those of the four whose rows are longer than kShortRow (in the first pass they,
+// and places beyond the bucket's end, have an empty row and v = -1).  A row of a few arcs by a whole
+// warp left most lanes idle on a chain of dependent reads.
+template <class Fn>
+__device__ __forceinline__ void for_bucket_vertices(const WArgs &a, const int32_t *bucket, int count, long long wid,
+                                                    long long nw, Fn fn)
+{
+    const int lane = threadIdx.x & 31, part = lane >> 3;
+    for (long long i = 4 * wid; i < count; i += 4 * nw) {
+        int v = -1, j0 = 0, j1 = 0;
+        if (i + part < count) {
+            v = dev::ldcg(bucket + i + part);
+            j0 = __ldg(a.rp + v);
+            j1 = __ldg(a.rp + v + 1);
+        }
+        const bool light = v >= 0 && j1 - j0 <= kHeavyChunk, shrt = light && j1 - j0 <= kShortRow;
+        if (__any_sync(0xffffffffu, shrt)) fn(shrt ? v : -1, j0, shrt ? j1 : j0, lane & 7, std::integral_constant<int, 8>());
+        for (unsigned m = __ballot_sync(0xffffffffu, light && !shrt && (lane & 7) == 0); m; m &= m - 1) {
+            const int l = __ffs(m) - 1;
+            fn(__shfl_sync(0xffffffffu, v, l), __shfl_sync(0xffffffffu, j0, l), __shfl_sync(0xffffffffu, j1, l), lane,
+               std::integral_constant<int, 32>());
+        }
+    }
 }
 
 // One search from s by the CTAs of one group (a: this group's view); false if a barrier
@@ -172,9 +217,10 @@ __device__ bool sweep(const WArgs &a, int s, long long tid, long long nthr)
         //      vertex; heavy vertices chunk by chunk, their sigma summed with integer
         //      atomics, which are exact in any order)
         long long lmin = kInf;
-        auto settle_arcs = [&](int v, int j0, int j1) -> unsigned long long {
+        // `wide` lanes (32, or 8 of them: lane l0 of a part of the warp) go over the arcs of a row
+        auto settle_arcs = [&](int v, int j0, int j1, int l0, int wide) -> unsigned long long {
             unsigned long long sig = 0;
-            for (int j = j0 + lane; j < j1; j += 32) {
+            for (int j = j0 + l0; j < j1; j += wide) {
                 const int x = __ldg(a.col + j);
                 const long long wj = __ldg(a.w + j);
                 const long long dx = ld_dist(a.dist + x);
@@ -189,24 +235,19 @@ __device__ bool sweep(const WArgs &a, int s, long long tid, long long nthr)
                     lmin = min(lmin, nd);
                 }
             }
-            return dev::group_sum_u64<32>(sig, ovf);
+            return sig;
         };
-        for (long long i = wid; i < nb; i += nw) {
-            const int v = dev::ldcg(a.order + qtail + i);
-            if (heavy(a, v)) continue;
-            const unsigned long long sig = settle_arcs(v, __ldg(a.rp + v), __ldg(a.rp + v + 1));
-            if (v != s && lane == 0) a.sp[v] = sig;
-        }
-        for (long long c = wid; c < a.C; c += nw) {
-            int h, j0, j1;
-            chunk_of(a, c, h, j0, j1);
-            if (ld_dist(a.dist + h) != D) continue;
-            const unsigned long long sig = settle_arcs(h, j0, j1);
+        for_bucket_vertices(a, a.order + qtail, nb, wid, nw, [&](int v, int j0, int j1, int l0, auto wide) {
+            const unsigned long long sig = dev::group_sum_u64<decltype(wide)::value>(settle_arcs(v, j0, j1, l0, wide), ovf);
+            if (v >= 0 && v != s && l0 == 0) a.sp[v] = sig;
+        });
+        for_bucket_chunks(a, D, wid, nw, [&](long long, int h, int j0, int j1) {
+            const unsigned long long sig = dev::group_sum_u64<32>(settle_arcs(h, j0, j1, lane, 32), ovf);
             if (h != s && lane == 0 && sig != 0) {
                 const unsigned long long old = atomicAdd(a.sp + h, sig);
                 ovf |= old + sig < old;
             }
-        }
+        });
         atomicMin(&s_min, lmin);  // s_min still holds the scan minimum of this block
         __syncthreads();
         if (threadIdx.x == 0 && s_min < kInf) atomicMin(a.bnext + b, s_min);
@@ -222,13 +263,13 @@ __device__ bool sweep(const WArgs &a, int s, long long tid, long long nthr)
     if (ovf) atomicOr(&a.ctrl->ovf, 1);
     if (!a.scores) return true;
     // ---- backward, last bucket first; heavy vertices sum per-chunk partials in chunk order
-    auto psi_sum = [&](long long dv, int j0, int j1) {
+    auto psi_sum = [&](long long dv, int j0, int j1, int l0, int wide) {
         dev::ff acc = dev::ff_zero();
-        for (int j = j0 + lane; j < j1; j += 32) {
+        for (int j = j0 + l0; j < j1; j += wide) {
             const int x = __ldg(a.col + j);
             if (ld_dist(a.dist + x) == dv + __ldg(a.w + j)) acc = dev::ff_add(acc, dev::ff_unpack(dev::ldcg(a.sp + x)));
         }
-        return dev::group_sum_ff<32>(acc);
+        return acc;
     };
     auto finish = [&](int v, dev::ff acc) {
         const dev::ff sv = dev::ff_from_u64(dev::ldcg(a.sp + v));
@@ -239,20 +280,15 @@ __device__ bool sweep(const WArgs &a, int s, long long tid, long long nthr)
     for (int bb = nbk - 1; bb >= 0; --bb) {
         const int off = dev::ldcg(a.boff + bb), cnt = dev::ldcg(a.bcnt + bb);
         const long long Db = dev::ldcg(a.bdist + bb);
-        for (long long i = wid; i < cnt; i += nw) {
-            const int v = dev::ldcg(a.order + off + i);
-            if (heavy(a, v)) continue;
-            const dev::ff acc = psi_sum(Db, __ldg(a.rp + v), __ldg(a.rp + v + 1));
-            if (lane == 0) finish(v, acc);
-        }
+        for_bucket_vertices(a, a.order + off, cnt, wid, nw, [&](int v, int j0, int j1, int l0, auto wide) {
+            const dev::ff acc = dev::group_sum_ff<decltype(wide)::value>(psi_sum(Db, j0, j1, l0, wide));
+            if (v >= 0 && l0 == 0) finish(v, acc);
+        });
         if (a.H > 0) {
-            for (long long c = wid; c < a.C; c += nw) {
-                int h, j0, j1;
-                chunk_of(a, c, h, j0, j1);
-                if (ld_dist(a.dist + h) != Db) continue;
-                const dev::ff acc = psi_sum(Db, j0, j1);
+            for_bucket_chunks(a, Db, wid, nw, [&](long long c, int, int j0, int j1) {
+                const dev::ff acc = dev::group_sum_ff<32>(psi_sum(Db, j0, j1, lane, 32));
                 if (lane == 0) a.part[c] = dev::ff_pack(acc);
-            }
+            });
             if (!group_barrier(a.ctrl, cpg, a.limit_ns)) return false;
             for (long long i = tid; i < a.H; i += nthr) {
                 const int h = __ldg(a.hv + i);
@@ -390,12 +426,33 @@ int run_weighted(nk_graph *g, const int32_t *d_src, int32_t k, double *d_scores,
     }
     if (bps < 1) return set_error(NK_ERR_CUDA, "weighted kernel cannot be resident");
     const int total = std::max(1, bps * num_sms() / std::max(1, cfg.grid_div));
-    // CTAs per search: about one per 2^18 arcs (measured best on R-MAT 18 and BA 10^6 with
-    // weights 1..16; a few CTAs at least, the whole grid for the largest graphs), or
-    // grid_ctas when given; as many groups as fit, k at most, and their state within a
-    // quarter of the free memory
-    int cpg = cfg.grid_ctas > 0 ? cfg.grid_ctas
-                                : (int)std::max<int64_t>(bps, std::min<int64_t>(total, (g->A + (1 << 18) - 1) >> 18));
+    // sources without arcs add nothing and would leave their group idle
+    Tmp csrc, ccnt;
+    if (d_scores && !dist_out && !sigma_out) {
+        NK_TRY(csrc.alloc(sizeof(int32_t) * (size_t)k, s));
+        NK_TRY(ccnt.alloc(sizeof(int32_t), s));
+        NK_TRY(compact_sources(g, d_src, k, csrc.as<int32_t>(), ccnt.as<int32_t>(), s));
+        int32_t kk = 0;
+        NK_CUDA(cudaMemcpyAsync(&kk, ccnt.p, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+        NK_CUDA(cudaStreamSynchronize(s));
+        if (kk < 0 || kk > k) return set_error(NK_ERR_CUDA, "source compaction returned %d of %d", kk, k);
+        d_src = csrc.as<int32_t>();
+        k = kk;
+    }
+    // CTAs per search: the sources in as few equal rounds as leave each search a CTA per 2^20 arcs (3
+    // at least), and no more CTAs than a search can use, one per 2^17 arcs (57 at least).  R-MAT 18, 64
+    // listed sources, groups x CTAs: 64 x 6 10.4 ms, 32 x 14 9.4, 15 x 30 10.4, 8 x 57 12.0; 8 listed: 8 x
+    // 30 2.26, 8 x 57 1.68, 4 x 114 2.66; ER 100003, 64: 64 x 4 4.35, 64 x 6 3.56, 32 x 14 3.66, 15 x 30 6.0; 8: 8 x
+    // 4 3.75, 8 x 57 1.09; R-MAT 20, 64: 32 x 14 39.5, 8 x 57 32.3, 3 x 120 40.0.  grid_ctas overrides it.
+    // As many groups as fit, k at most, and their state within a quarter of the free memory.
+    int cpg = cfg.grid_ctas;
+    if (cpg <= 0) {
+        const int least = (int)std::max<int64_t>(bps, std::min<int64_t>(total, g->A >> 20));
+        int rounds = 1;
+        while (total / ((std::max(k, 1) + rounds - 1) / rounds) < least && rounds < k) ++rounds;
+        const int most = (int)std::max<int64_t>(57, std::min<int64_t>(total, g->A >> 17));
+        cpg = std::max(1, std::min(most, total / ((std::max(k, 1) + rounds - 1) / rounds)));
+    }
     cpg = std::min(cpg, total);
     int groups = std::max(1, std::min(total / cpg, k));
     const size_t per_group = 16 * (size_t)n + 4 * (size_t)n + 24 * lv + 8 * (C + 1) + (d_scores ? 8 * (size_t)n : 0) + sizeof(Ctrl);

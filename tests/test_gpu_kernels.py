@@ -126,3 +126,17 @@ def test_batches_side_by_side(nk, k):
     want, r, _ = oracle.betweenness_rk(rp, col, 0.15, 0.1, 7)
     got, r1, _ = nk.betweenness_rk(g, 0.15, 0.1, 7, o)
     assert r1 == r and np.array_equal(got, want)
+
+
+@pytest.mark.parametrize("k", [1, 5, 40])
+def test_weighted_rows(nk, k):
+    """Weighted sweeps over rows of 1 to 600 arcs (8 lanes up to 32 arcs, a warp, chunks of 256) and
+    isolated vertices, by many and by few blocks per search, against the oracle."""
+    n, u, v = GROUPS["rows"]
+    g = nk.graph_from_edges(n, u, v)
+    rp, col = oracle.csr_build(n, u, v)
+    nk.random_weights(g, 4, 5)
+    ref = oracle.betweenness_weighted_sampled(rp, col, oracle.edge_weights(rp, col, 4, 5), 9, k)
+    for ctas in (0, 1, 7):
+        got = nk.betweenness_weighted_sampled(g, 9, k, nk.run_opts(grid_ctas=ctas))
+        assert np.allclose(got, ref, rtol=1e-9, atol=1e-12)
