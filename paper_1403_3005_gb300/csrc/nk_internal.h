@@ -272,6 +272,10 @@ int run_batched(nk_graph *g, const int32_t *d_src, int32_t k, double *d_scores,
 // reach counts of the k device sources, in batches of cfg.batch sources (0: by k).
 int run_levels(nk_graph *g, const int32_t *d_src, int32_t k, const RunCfg &cfg, RunStats *st, cudaStream_t s);
 
+// Betweenness of a handful of device sources in batches of 8 (nk_thin.cu): scores += dependencies.
+int run_thin(nk_graph *g, const int32_t *d_src, int32_t k, double *d_scores, const RunCfg &cfg, RunStats *st,
+             cudaStream_t s);
+
 // Capturable pieces of the batched form: prepare_only sizes and allocates the scratch
 // (outside any stream capture); otherwise the status reset and the launches are enqueued
 // without host synchronisation, and *ctrls / *nb give the per-batch status words.

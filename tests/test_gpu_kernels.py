@@ -140,3 +140,25 @@ def test_weighted_rows(nk, k):
     for ctas in (0, 1, 7):
         got = nk.betweenness_weighted_sampled(g, 9, k, nk.run_opts(grid_ctas=ctas))
         assert np.allclose(got, ref, rtol=1e-9, atol=1e-12)
+
+
+@pytest.mark.parametrize("name", ["rows", "tiny", "many", "path", "grid"])
+@pytest.mark.parametrize("k", [1, 4, 8, 9, 15])
+def test_few_sources(nk, name, k):
+    """Below 16 sources: batches of 8, rows of up to 32 arcs by parts of a warp, longer ones and
+    chunks by all of it, searches deeper than the first attempt's level slabs."""
+    n, u, v = {"path": G.path(300), "grid": G.grid(30, 31)}.get(name) or GROUPS[name]
+    g = nk.graph_from_edges(n, u, v)
+    rp, col = oracle.csr_build(n, u, v)
+    src = oracle.sample_sources(n, 5, k)
+    ref = oracle.betweenness_sources(rp, col, src, 2.0)
+    for kw in (dict(), dict(direction=1), dict(direction=2), dict(chunk=32, alpha=4.0)):
+        got = nk.betweenness_sources(g, src, 2.0, nk.run_opts(**kw))
+        assert np.allclose(got, ref, rtol=1e-9, atol=1e-12)
+
+
+def test_few_sources_overflow(nk):
+    g = nk.graph_from_edges(*G.grid(36, 36))
+    with pytest.raises(nk.NkError) as e:
+        nk.betweenness_sources(g, np.array([0, 1, 2, 3, 4], np.int32), 1.0)
+    assert e.value.rc == nk.ERR_OVERFLOW
