@@ -237,6 +237,15 @@ struct LbStage {
     unsigned long long val[32];
 };
 
+// Vertices of a group for a level of `count` queue entries: 32, or the warp's share of a short level,
+// so that its vertices spread over all warps (groups of 32 kept 10 to 60 warps of a small graph's
+// level busy and the others waiting: one search with its results on the host, ER 2000 220 -> 136 us,
+// ER 200003 620 -> 254, R-MAT 18 372 -> 296, R-MAT 20 582 -> 550).
+__device__ __forceinline__ int lb_group(int count, long long nwarps)
+{
+    return (int)max(1LL, min(32LL, (count + nwarps - 1) / nwarps));
+}
+
 // Stages the group (v = -1 or deg = 0 for no vertex) and returns its arc count.
 __device__ __forceinline__ int lb_stage(LbStage &st, int v, int deg, unsigned long long val, const int32_t *rp)
 {
@@ -304,7 +313,7 @@ __device__ __forceinline__ void lb_seg_add(LbStage &st, int k, bool valid, unsig
 }
 
 // ------------------------------------------------------------------ top-down level d
-// Light frontier vertices: groups of 32 queue entries, lanes over their arcs.
+// Light frontier vertices: groups of up to 32 queue entries, lanes over their arcs.
 
 __device__ void td_level(const SrcArgs &a, int d, int qo, int nf, int qnext, unsigned long long *s_mf,
                          bool &ovf, LbStage *stages)
@@ -313,9 +322,10 @@ __device__ void td_level(const SrcArgs &a, int d, int qo, int nf, int qnext, uns
     LbStage &st = stages[threadIdx.x >> 5];
     const long long wid = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-    for (long long base = wid * 32; base < nf; base += nwarps * 32) {
+    const int gs = lb_group(nf, nwarps);
+    for (long long base = wid * gs; base < nf; base += nwarps * gs) {
         int v = -1, deg = 0;
-        if (base + lane < nf) {
+        if (lane < gs && base + lane < nf) {
             v = __ldcg(a.queue + qo + base + lane);
             if ((unsigned)v < (unsigned)a.n && !heavy(a, v)) deg = degree(a.rp, v);
             else v = -1;
@@ -370,15 +380,19 @@ __device__ void bu_level(const SrcArgs &a, int d, int qnext, unsigned long long 
     const unsigned *cur = lvl_bits(a, d);
     // a warp takes the 32 vertices of one word of the visited bitmap: its words are
     // wid + i * nwarps, read 32 at a time (a lane each), and the words with an unvisited
-    // vertex are walked in turn
-    for (long long i0 = 0; wid + i0 * nwarps < a.nw; i0 += 32) {
-        const long long wl = wid + (i0 + lane) * nwarps;
-        const unsigned vl = wl < a.nw ? __ldcg(vis_bits(a) + wl) : FULL;
+    // vertex are walked in turn.  With fewer words than warps, `share` warps (a power of two)
+    // take equal parts of a word.
+    const int share = a.nw >= nwarps ? 1 : min(32, 1 << (31 - __clz((int)(nwarps / a.nw))));
+    const unsigned part = share == 1 ? FULL : ((1u << (32 / share)) - 1u) << ((wid % share) * (32 / share));
+    const long long w0 = wid / share, wstep = nwarps / share;
+    for (long long i0 = 0; w0 < wstep && w0 + i0 * wstep < a.nw; i0 += 32) {
+        const long long wl = w0 + (i0 + lane) * wstep;
+        const unsigned vl = wl < a.nw ? __ldcg(vis_bits(a) + wl) | ~part : FULL;
         unsigned open = __ballot_sync(FULL, vl != FULL);
       while (open) {
         const int b = __ffs(open) - 1;
         open &= open - 1;
-        const long long wd = wid + (i0 + b) * nwarps;
+        const long long wd = w0 + (i0 + b) * wstep;
         const unsigned visw = __shfl_sync(FULL, vl, b);
         const long long w = wd * 32 + lane;
         const bool act = w < a.n && !((visw >> lane) & 1u) && !heavy(a, (int)w);
@@ -463,9 +477,10 @@ __device__ void back_level(const SrcArgs &a, int d, int qo, int nd, LbStage *sta
     const long long wid = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
     const unsigned *succ = lvl_bits(a, 0);
-    for (long long base = wid * 32; light && base < nd; base += nwarps * 32) {
+    const int gs = lb_group(nd, nwarps);
+    for (long long base = wid * gs; light && base < nd; base += nwarps * gs) {
         int v = -1, deg = 0;
-        if (base + lane < nd) {
+        if (lane < gs && base + lane < nd) {
             v = __ldcg(a.queue + qo + base + lane);
             if ((unsigned)v < (unsigned)a.n && !heavy(a, v)) deg = degree(a.rp, v);
             else v = -1;
@@ -565,10 +580,11 @@ __device__ void back_push(const SrcArgs &a, int d, int qo1, int n1, LbStage *sta
     const long long wid = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
     const unsigned *tgt = lvl_bits(a, 1);
-    // light vertices of level d+1: groups of 32 queue entries, lanes over their arcs
-    for (long long base = wid * 32; base < n1; base += nwarps * 32) {
+    // light vertices of level d+1: groups of up to 32 queue entries, lanes over their arcs
+    const int gs = lb_group(n1, nwarps);
+    for (long long base = wid * gs; base < n1; base += nwarps * gs) {
         int w = -1, deg = 0;
-        if (base + lane < n1) {
+        if (lane < gs && base + lane < n1) {
             w = __ldcg(a.queue + qo1 + base + lane);
             if ((unsigned)w < (unsigned)a.n && !heavy(a, w)) deg = degree(a.rp, w);
             else w = -1;
@@ -840,6 +856,9 @@ __global__ void k_add_distances(const int32_t *dist, int32_t n, unsigned long lo
     }
 }
 
+// CTAs of a sweep: no more than a small graph can use (32, 64, 128 and 256 at least measured alike).
+int sweep_grid(int grid, int32_t n) { return std::max(1, std::min(grid, std::max(128, n / 64))); }
+
 // ------------------------------------------------------------------ host side
 struct Launch {
     const void *fn;
@@ -947,7 +966,7 @@ int run(nk_graph *g, const int32_t *d_src, int32_t k, double *d_scores, const Ru
         a.src = d_src + i;
         a.trace = (trace_on && i == 0) ? trace_buf.as<unsigned long long>() : nullptr;
         void *args[] = {&a};
-        int grid = std::max(1, L.grid / std::max(1, cfg.grid_div));
+        int grid = sweep_grid(L.grid / std::max(1, cfg.grid_div), n);
         if (cfg.grid_ctas > 0) grid = std::min(grid, cfg.grid_ctas);
         NK_CUDA(cudaLaunchCooperativeKernel(L.fn, dim3(grid), dim3(kThreads), args, 0, s));
         ::nk::count_launch();
@@ -1117,7 +1136,7 @@ extern "C" int nk_sssp_noalloc(int32_t n, const int32_t *row_ptr, const int32_t 
     NK_CUDA(cudaMemsetAsync(a.ctrl, 0, sizeof(Ctrl), st));
     NK_CUDA(cudaMemcpyAsync(scr + kNaSrc, &s, sizeof(int32_t), cudaMemcpyHostToDevice, st));
     void *args[] = {&a};
-    NK_CUDA(cudaLaunchCooperativeKernel(L.fn, dim3(L.grid), dim3(kThreads), args, 0, st));
+    NK_CUDA(cudaLaunchCooperativeKernel(L.fn, dim3(sweep_grid(L.grid, n)), dim3(kThreads), args, 0, st));
     ::nk::count_launch();
     Ctrl h;
     NK_CUDA(cudaMemcpyAsync(&h, a.ctrl, sizeof(Ctrl), cudaMemcpyDeviceToHost, st));

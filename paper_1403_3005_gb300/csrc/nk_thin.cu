@@ -467,12 +467,15 @@ int run_thin(nk_graph *g, const int32_t *d_src, int32_t k, double *d_scores, con
     if (k == 0) return NK_OK;
     HeavyView hw;
     NK_TRY(heavy_view(g, cfg.chunk, s, &hw));
-    // one to three sources on a graph most of whose arcs are hubs' go one by one: a hub's chunk then is
-    // a warp's for one source, without the parts.  Per-source against 8 at once, ms: R-MAT 20 with 1, 2,
-    // 3, 4, 8 sources 0.99 / 2.36, 2.0 / 2.6, 3.2 / 3.0, 4.1 / 3.0, 7.8 / 3.4; R-MAT 22 3.2 / 7.4, 5.6 / 8.0, 9.4
-    // / 9.5, 12.7 / 9.6, 23.9 / 12.1; but BA 10^6 2.0 / 1.4, 3.6 / 1.8, 5.6 / 2.1, 7.6 / 2.1, 15.0 / 2.3; ER 200003
-    // 0.84 / 0.58, 1.6 / 0.63, ..., 6.4 / 0.81
-    if (k < 4 && (int64_t)hw.C * hw.chunk > g->A / 4) return run_per_source(g, d_src, k, d_scores, cfg, st, s);
+    // a single source, and two or three on large graphs most of whose arcs are hubs', go one by one: a
+    // hub's chunk then is a warp's for one source, without the parts.  Per-source against 8 at once, ms,
+    // for 1, 2, 3, 4, 8 sources: ER 200003 0.41 / 0.57, 0.74 / 0.64, 1.0 / 0.70, ..., 2.7 / 0.82; BA 10^6 1.1 /
+    // 1.4, 2.1 / 1.8, ..., 8.2 / 2.3; R-MAT 16 0.38 / 0.61, 0.71 / 0.64, 1.0 / 0.64; R-MAT 18 0.53 / 0.91, 1.1 / 1.1,
+    // 1.6 / 1.2; R-MAT 20 1.0 / 2.4, 2.0 / 2.6, 3.3 / 3.0, 4.4 / 3.0, 7.8 / 3.4; R-MAT 22 3.0 / 7.4, 5.1 / 8.0, 8.5 / 9.5,
+    // 11.6 / 9.7, 21.7 / 12.2
+    const bool hubs = (int64_t)hw.C * hw.chunk > g->A / 4;
+    if (k == 1 || (hubs && ((k == 2 && g->A >= (4 << 20)) || (k == 3 && g->A >= (64 << 20)))))
+        return run_per_source(g, d_src, k, d_scores, cfg, st, s);
     DevBuf *ws = scratch(cfg, g);
     const int nb = (k + kT - 1) / kT;
     NK_TRY(ws[WS_BCTRL].ensure(sizeof(Ctrl) * nb));
