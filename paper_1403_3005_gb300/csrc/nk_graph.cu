@@ -10,7 +10,7 @@
 //   2. exclusive scan of the degrees -> bucket offsets;
 //   3. scatter of both arcs into their row buckets (atomic cursors; order arbitrary);
 //   4. per-row sort + duplicate removal into a second buffer: a warp bitonic network
-//      for rows of <= 32 arcs, a shared-memory bitonic sort for rows of <= 4096, and a
+//      for rows of <= 256 arcs, a shared-memory bitonic sort for rows of <= 4096, and a
 //      windowed shared-memory bitmap for longer rows (ids are < n, so marking bits of a
 //      window of the id range and reading them back in order sorts and dedupes at once);
 //   5. scan of the unique counts -> row_ptr, and a warp-per-row copy into col.
@@ -28,6 +28,7 @@ namespace {
 
 int finish_graph(nk_graph *g, cudaStream_t st, int *d_maxdeg);
 
+constexpr int kWarpRow = 256;           // rows up to this length: a warp's registers
 constexpr int kMidMax = 4096;           // rows up to this length: shared-memory bitonic
 constexpr int kWinBits = 1 << 18;       // bitmap window for long rows (32 KiB)
 constexpr int kWinWords = kWinBits / 32;
@@ -69,58 +70,117 @@ __global__ void k_scatter(const int32_t *u, const int32_t *v, int64_t m,
     }
 }
 
-// rows of length <= 32: one warp, bitonic network on shuffles
-__global__ void k_sort_small(const int64_t *off, const int32_t *buf, int32_t *out,
-                             int64_t *ucnt, int32_t n)
+// Sorted distinct values of src[0..len), len <= 32 E, into dst; returns their number.  A bitonic
+// network over the warp's registers: element e*32 + lane is x[e] of the lane, so that distances of 32
+// and more exchange registers and smaller ones shuffle.
+template <int E> __device__ __forceinline__ int warp_sort_unique(const int32_t *src, int len, int32_t *dst)
+{
+    const int lane = threadIdx.x & 31;
+    int x[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) x[e] = e * 32 + lane < len ? src[e * 32 + lane] : INT_MAX;
+#pragma unroll
+    for (int k = 2; k <= 32 * E; k <<= 1) {
+#pragma unroll
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            if (j >= 32) {
+#pragma unroll
+                for (int e = 0; e < E; ++e)
+                    if ((e & (j / 32)) == 0) {
+                        int &p = x[e], &q = x[(e | (j / 32)) % E];  // % E: only for the compiler
+                        const int lo = min(p, q), hi = max(p, q);
+                        const bool up = ((e * 32) & k) == 0;
+                        p = up ? lo : hi;
+                        q = up ? hi : lo;
+                    }
+            } else {
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    const int y = __shfl_xor_sync(0xffffffffu, x[e], j);
+                    const bool up = ((e * 32 + lane) & k) == 0, lower = (lane & j) == 0;
+                    x[e] = lower == up ? min(x[e], y) : max(x[e], y);
+                }
+            }
+        }
+    }
+    int count = 0, last = INT_MAX;  // last: the largest value of the registers before
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        int prev = __shfl_up_sync(0xffffffffu, x[e], 1);
+        if (lane == 0) prev = last;
+        const bool keep = x[e] != INT_MAX && ((e == 0 && lane == 0) || prev != x[e]);
+        const unsigned bal = __ballot_sync(0xffffffffu, keep);
+        if (keep) dst[count + __popc(bal & dev::lanemask_lt())] = x[e];
+        count += __popc(bal);
+        last = __shfl_sync(0xffffffffu, x[e], 31);
+    }
+    return count;
+}
+
+// rows of length <= kWarpRow: one warp per row, in registers.  A block of 512 threads with a barrier
+// per step took the rows from 33 on before: R-MAT 18 (8.4M arcs) 2.24 ms for those up to 4096.
+__global__ void __launch_bounds__(256)
+k_sort_small(const int64_t *off, const int32_t *buf, int32_t *out, int64_t *ucnt, int32_t n)
 {
     const int lane = threadIdx.x & 31;
     const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t r = warp; r < n; r += nwarps) {
-        const int64_t b = off[r], len = off[r + 1] - b;
-        if (len > 32) continue;  // warp-uniform
-        int x = lane < len ? buf[b + lane] : INT_MAX;
-        for (int k = 2; k <= 32; k <<= 1) {
-            for (int j = k >> 1; j > 0; j >>= 1) {
-                int y = __shfl_xor_sync(0xffffffffu, x, j);
-                bool up = (lane & k) == 0;
-                bool lower = (lane & j) == 0;
-                x = (lower == up) ? min(x, y) : max(x, y);
-            }
-        }
-        int prev = __shfl_up_sync(0xffffffffu, x, 1);
-        bool keep = x != INT_MAX && (lane == 0 || prev != x);
-        unsigned bal = __ballot_sync(0xffffffffu, keep);
-        if (keep) out[b + __popc(bal & dev::lanemask_lt())] = x;
-        if (lane == 0) ucnt[r] = __popc(bal);
+        const int64_t b = off[r], l64 = off[r + 1] - b;
+        if (l64 > kWarpRow) continue;  // warp-uniform
+        const int len = (int)l64;
+        const int c = len <= 32    ? warp_sort_unique<1>(buf + b, len, out + b)
+                      : len <= 64  ? warp_sort_unique<2>(buf + b, len, out + b)
+                      : len <= 128 ? warp_sort_unique<4>(buf + b, len, out + b)
+                                   : warp_sort_unique<8>(buf + b, len, out + b);
+        if (lane == 0) ucnt[r] = c;
     }
 }
 
-// rows of length in (32, 4096]: one block of 512 threads, bitonic sort in shared memory
+// Calls fn(r) with the whole block for the block's rows blockIdx.x + i * gridDim.x whose length is in
+// (lo, hi]: its 512 threads look at 512 rows at a time and list them (row by row, the block waited
+// for the offsets of every short row).
+template <class Fn>
+__device__ __forceinline__ void for_long_rows(const int64_t *off, int32_t n, int64_t lo, int64_t hi, Fn fn)
+{
+    __shared__ int list[512];
+    __shared__ int count;
+    for (int64_t r0 = blockIdx.x; r0 < n; r0 += 512ll * gridDim.x) {  // block-uniform
+        if (threadIdx.x == 0) count = 0;
+        __syncthreads();
+        const int64_t r = r0 + (int64_t)threadIdx.x * gridDim.x;
+        if (r < n) {
+            const int64_t len = off[r + 1] - off[r];
+            if (len > lo && len <= hi) list[atomicAdd(&count, 1)] = (int)r;
+        }
+        __syncthreads();
+        const int found = count;
+        for (int i = 0; i < found; ++i) fn((int64_t)list[i]);
+        __syncthreads();
+    }
+}
+
+// rows of length in (kWarpRow, 4096]: one block of 512 threads, bitonic sort in shared memory
 __global__ void __launch_bounds__(512)
 k_sort_mid(const int64_t *off, const int32_t *buf, int32_t *out, int64_t *ucnt, int32_t n)
 {
     __shared__ int s[kMidMax];
     __shared__ int warp_cnt[16];
-    for (int64_t r = blockIdx.x; r < n; r += gridDim.x) {
+    for_long_rows(off, n, kWarpRow, kMidMax, [&](int64_t r) {
         const int64_t b = off[r];
         const int len = (int)(off[r + 1] - b);
-        if (len <= 32 || len > kMidMax) continue;  // block-uniform
-        int N = 64;
+        int N = 512;
         while (N < len) N <<= 1;
         for (int i = threadIdx.x; i < N; i += blockDim.x) s[i] = i < len ? buf[b + i] : INT_MAX;
         __syncthreads();
         for (int k = 2; k <= N; k <<= 1) {
             for (int j = k >> 1; j > 0; j >>= 1) {
-                for (int i = threadIdx.x; i < N; i += blockDim.x) {
-                    int p = i ^ j;
-                    if (p > i) {
-                        int a = s[i], c = s[p];
-                        bool up = (i & k) == 0;
-                        if ((a > c) == up) {
-                            s[i] = c;
-                            s[p] = a;
-                        }
+                for (int t = threadIdx.x; t < N / 2; t += blockDim.x) {
+                    const int i = ((t & ~(j - 1)) << 1) | (t & (j - 1)), p = i | j;
+                    const int a = s[i], c = s[p];
+                    if ((a > c) == ((i & k) == 0)) {
+                        s[i] = c;
+                        s[p] = a;
                     }
                 }
                 __syncthreads();
@@ -146,7 +206,7 @@ k_sort_mid(const int64_t *off, const int32_t *buf, int32_t *out, int64_t *ucnt, 
         }
         if (threadIdx.x == 0) ucnt[r] = base;
         __syncthreads();
-    }
+    });
 }
 
 // rows longer than 4096: windowed bitmap over the id range
@@ -156,10 +216,9 @@ k_sort_big(const int64_t *off, const int32_t *buf, int32_t *out, int64_t *ucnt, 
     __shared__ unsigned bits[kWinWords];
     __shared__ int warp_cnt[16];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int64_t r = blockIdx.x; r < n; r += gridDim.x) {
+    for_long_rows(off, n, kMidMax, LLONG_MAX, [&](int64_t r) {
         const int64_t b = off[r];
         const int64_t len = off[r + 1] - b;
-        if (len <= kMidMax) continue;  // block-uniform
         int64_t written = 0;
         for (int64_t lo = 0; lo < n; lo += kWinBits) {
             for (int i = threadIdx.x; i < kWinWords; i += blockDim.x) bits[i] = 0u;
@@ -199,9 +258,10 @@ k_sort_big(const int64_t *off, const int32_t *buf, int32_t *out, int64_t *ucnt, 
         }
         if (threadIdx.x == 0) ucnt[r] = written;
         __syncthreads();
-    }
+    });
 }
 
+// A warp per row, eight loads in flight (one at a time, the longest hub's row took 0.5 ms alone).
 __global__ void k_compact_rows(const int64_t *off, const int64_t *rp64, const int32_t *src,
                                int32_t *rp, int32_t *col, int32_t n, int *max_deg)
 {
@@ -215,7 +275,15 @@ __global__ void k_compact_rows(const int64_t *off, const int64_t *rp64, const in
         if (r == n) continue;
         const int64_t len = rp64[r + 1] - dst;
         const int64_t b = off[r];
-        for (int64_t i = lane; i < len; i += 32) col[dst + i] = src[b + i];
+        int64_t i = lane;
+        for (; i + 7 * 32 < len; i += 8 * 32) {
+            int32_t x[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) x[q] = __ldg(src + b + i + 32 * q);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) col[dst + i + 32 * q] = x[q];
+        }
+        for (; i < len; i += 32) col[dst + i] = __ldg(src + b + i);
         local_max = max(local_max, (int)len);
     }
     if (lane == 0) atomicMax(max_deg, local_max);

@@ -162,3 +162,19 @@ def test_few_sources_overflow(nk):
     with pytest.raises(nk.NkError) as e:
         nk.betweenness_sources(g, np.array([0, 1, 2, 3, 4], np.int32), 1.0)
     assert e.value.rc == nk.ERR_OVERFLOW
+
+
+def test_csr_rows_at_the_sort_sizes(nk):
+    """Raw rows (with duplicates and loops) around the sizes where the sort changes: 32, 64, 128 and
+    256 (registers), 512 and 4096 (shared memory), and above (bitmap)."""
+    sizes = [1, 31, 32, 33, 63, 64, 65, 127, 128, 129, 255, 256, 257, 511, 512, 513, 4095, 4096, 4097, 9000]
+    rng = np.random.default_rng(3)
+    n = len(sizes) + 12000
+    u = np.concatenate([np.full(s, i) for i, s in enumerate(sizes)] + [[5, 7000]]).astype(np.int32)
+    v = np.concatenate([rng.integers(len(sizes), n, s) for s in sizes] + [[5, 7000]]).astype(np.int32)
+    v[rng.random(len(v)) < 0.1] = n - 1  # duplicates
+    order = rng.permutation(len(u))
+    g = nk.graph_from_edges(n, u[order], v[order])
+    rp, col = oracle.csr_build(n, u, v)
+    a, b = g.export_csr()
+    assert np.array_equal(a, rp) and np.array_equal(b, col)
