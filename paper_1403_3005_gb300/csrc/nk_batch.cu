@@ -1186,14 +1186,14 @@ int launch_batches(nk_graph *g, const int32_t *d_src, int32_t k, double *d_score
     NK_TRY(ws[WS_BCTRL].ensure(sizeof(Ctrl) * nb));
     const bool edge = cfg.edge && cfg.backward;
     // sigma in 32-bit rows unless a batch's counts do not fit (then that batch is rerun with
-    // 64-bit rows); the edge variant keeps 64-bit rows
-    bool s32 = !edge;
+    // 64-bit rows)
+    bool s32 = true;
     auto pick = [&](const void *&kfn, int &grid) -> int {
-        const int bps = edge ? blocks_per_sm<W, true, false>() : s32 ? blocks_per_sm<W, false, true>()
-                                                                     : blocks_per_sm<W, false, false>();
+        const int bps = edge ? (s32 ? blocks_per_sm<W, true, true>() : blocks_per_sm<W, true, false>())
+                             : (s32 ? blocks_per_sm<W, false, true>() : blocks_per_sm<W, false, false>());
         if (bps < 1) return set_error(NK_ERR_CUDA, "batched kernel cannot be resident");
-        kfn = edge ? (const void *)k_batch<W, true, false>
-                   : s32 ? (const void *)k_batch<W, false, true> : (const void *)k_batch<W, false, false>;
+        kfn = edge ? (s32 ? (const void *)k_batch<W, true, true> : (const void *)k_batch<W, true, false>)
+                   : (s32 ? (const void *)k_batch<W, false, true> : (const void *)k_batch<W, false, false>);
         grid = std::max(1, bps * num_sms() / std::max(1, cfg.grid_div));
         if (cfg.grid_ctas > 0) grid = std::min(grid, cfg.grid_ctas);
         return NK_OK;
