@@ -1055,12 +1055,13 @@ constexpr int kTeamCtas = 128, kTeamVertices = 64;
 // 10.0, -, 9.8; BA 10^6 (4) 31.5, 29.9, 30.0; R-MAT 20 36.2, 34.4, 35.8, 40.3; R-MAT 22 133, 132,
 // 136, 146; R-MAT 24 320, 320.  The number of teams per launch is evened out; the batches stay full and
 // the last one short (made equal, R-MAT 18 takes 12.9 instead of 11.3 ms: a row read serves fewer).  Callers with their
-// own workspace or grid (servers, captured graphs) run one batch at a time.
+// own workspace or grid (captured graphs) run one batch at a time unless they say how many (servers).
 int choose_teams(const nk_graph *g, int B, size_t state, int nb, int grid, const RunCfg &cfg, const DevBuf *ws, int64_t outs)
 {
-    if (cfg.ws || cfg.grid_ctas > 0 || nb < 2) return 1;
+    if (nb < 2 || (cfg.teams <= 0 && (cfg.ws || cfg.grid_ctas > 0))) return 1;
     const size_t rows = (size_t)g->n * B * 12;
-    int want = (int)std::min<size_t>(std::min(nb, std::min(kMaxTeams, grid)), (kTeamRows + rows - 1) / rows);
+    int want = std::min(nb, std::min(kMaxTeams, grid));
+    want = cfg.teams > 0 ? std::min(want, cfg.teams) : (int)std::min<size_t>(want, (kTeamRows + rows - 1) / rows);
     size_t free_b = 0, total_b = 0;
     cudaMemGetInfo(&free_b, &total_b);
     const size_t per = state + sizeof(double) * (size_t)outs;

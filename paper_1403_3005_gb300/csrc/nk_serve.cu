@@ -7,11 +7,12 @@
 // own non-blocking CUDA stream; its request's state (sampled sources, per-batch bitset
 // levels, sigma/psi rows, scores) is allocated stream-ordered on that stream and freed
 // when the request ends, so the work of different requests - on different graphs or on
-// the same one - overlaps on the device.  A request's persistent grid is sized by its
-// graph (about one CTA per 8192 arcs, at least 128, at most half of the co-resident
-// CTAs): small requests stay cheap to synchronise and many run side by side, large ones
-// get up to half of the GPU, so that a large request never holds the small ones back.  CSR arrays
-// stay resident in the graph objects the caller owns.
+// the same one - overlaps on the device.  A job gets its share of the GPU's CTAs by its work
+// (arcs x sources) among all jobs running or waiting, at least 128 and one per 8192 arcs, at
+// most half of them, and its batches run side by side within them: a small sweep is the cheaper
+// the fewer CTAs wait at its barriers, so many narrow sweeps do more per second than a few wide
+// ones, and a job alone still gets half of the GPU.  CSR arrays stay resident in the graph
+// objects the caller owns.
 //
 // Latency is measured from submit to the moment the scores are in the caller's buffer.
 #include <algorithm>
@@ -46,6 +47,9 @@ struct Request {
 };
 
 constexpr int kServeLcap = 64;
+constexpr int kShareMin = 128;         // CTAs of a job at least, and
+constexpr int64_t kShareArcs = 8192;   // one per that many arcs
+constexpr int kTeamMin = 16;           // CTAs of a batch at least
 
 }  // namespace
 }  // namespace nk
@@ -70,6 +74,7 @@ struct nk_server {
     int64_t peak_inflight = 0;
     int64_t launches_jobs = 0, packed = 0;  // jobs started; requests that ran in packs
     double busy_s = 0, exs = 0;
+    double work_running = 0;                // arcs x sources of the running jobs
     nk::clk::time_point busy_since;
     std::vector<double> lat_ms, wait_ms, run_ms;
 };
@@ -95,7 +100,31 @@ size_t request_bytes(const nk_graph *g, int B, int32_t k)
            sizeof(int32_t) * (size_t)k + sizeof(double) * (size_t)g->n + 4096;
 }
 
-int run_request(nk_server *S, Request *r, cudaStream_t st, double **h_buf, size_t *h_cap)
+// A job's part of the GPU: CTAs of its launches, and batches that run side by side in them.
+struct Share {
+    int ctas = 0, teams = 1;
+};
+
+double work_of(const Request *r) { return (double)r->g->A * (double)r->k + 1.0; }
+
+// `work` of `all` the work at hand, on `arcs` arcs in `nb` batches; `bytes`: device bytes of one
+// batch's state, `room`: what may be used for more of them.  (128 sources a launch use 4 CTAs per
+// SM.)  CTAs by the graph alone and one batch at a time, against this: one request of 500 sources on ER
+// 100000 10.7 / 5.4 ms, of 1000 on R-MAT 16 7.4 / 4.5; 16 mixed requests 17.4 / 14.4, 64 79 / 75.  By the
+// share alone, without the lower bound, the 64 took 119 ms; with the bound but one batch at a time the
+// 16 took 18.5.
+Share share_of(double work, double all, int64_t arcs, int nb, size_t bytes, size_t room)
+{
+    Share s;
+    const int sms = num_sms();
+    const double least = (double)std::max<int64_t>(kShareMin, arcs / kShareArcs);
+    s.ctas = (int)std::min(2.0 * sms, std::max(least, 4.0 * sms * work / all));
+    s.teams = std::max(1, std::min(nb, s.ctas / kTeamMin));
+    while (s.teams > 1 && bytes * (size_t)(s.teams - 1) > room) --s.teams;
+    return s;
+}
+
+int run_request(nk_server *S, Request *r, const Share &share, cudaStream_t st, double **h_buf, size_t *h_cap)
 {
     nk_graph *g = r->g;
     const int32_t n = g->n;
@@ -113,10 +142,10 @@ int run_request(nk_server *S, Request *r, cudaStream_t st, double **h_buf, size_
     cfg.mode = NK_MODE_BATCHED;
     cfg.batch = request_batch(S, g, r->k);
     cfg.ws = ws;
-    // persistent grid sized by the graph: about one CTA per 8192 arcs, at least 128, at
-    // most half of the co-resident CTAs (co-residency is guaranteed per launch; launches
-    // that do not fit beside the running ones wait for their CTAs to free up)
-    cfg.grid_ctas = (int)std::min<int64_t>(std::max<int64_t>(g->A / 8192, 128), 1 << 20);
+    // co-residency is guaranteed per launch; launches that do not fit beside the running ones
+    // wait for their CTAs to free up
+    cfg.grid_ctas = share.ctas;
+    cfg.teams = share.teams;
     cfg.grid_div = 2;  // no request takes more than half of the co-resident CTAs
     cfg.lcap = std::min(kServeLcap, std::max(n, 4));
     cfg.limit_ns = S->limit_ns;
@@ -175,7 +204,7 @@ __global__ void k_set_last(int32_t *rp_u, int32_t n_u, int32_t A_u) { rp_u[n_u] 
 
 int blocks_for(int64_t items) { return (int)std::max<int64_t>(1, std::min<int64_t>((items + 255) / 256, 4 * num_sms())); }
 
-int run_pack(nk_server *S, const std::vector<Request *> &rs, cudaStream_t st, double **h_buf,
+int run_pack(nk_server *S, const std::vector<Request *> &rs, const Share &share, cudaStream_t st, double **h_buf,
              size_t *h_cap)
 {
     // offsets of each member in the union: vertices, arcs, sources, heavy rows, chunks
@@ -256,7 +285,8 @@ int run_pack(nk_server *S, const std::vector<Request *> &rs, cudaStream_t st, do
     cfg.batch = k_u > 64 ? kPackWidth : 64;
     cfg.keep_order = true;  // the members' sources stay together: a batch of several graphs shares no rows
     cfg.ws = ws;
-    cfg.grid_ctas = (int)std::min<int64_t>(std::max<int64_t>(A_u / 8192, 128), 1 << 20);
+    cfg.grid_ctas = share.ctas;
+    cfg.teams = share.teams;
     cfg.grid_div = 2;
     cfg.lcap = std::min<int64_t>(kServeLcap, std::max<int64_t>(n_u, 4));
     cfg.limit_ns = S->limit_ns;
@@ -289,6 +319,8 @@ void worker(nk_server *S)
     for (;;) {
         std::vector<Request *> job;
         size_t need = 0;
+        double work = 0;
+        Share share;
         {
             std::unique_lock<std::mutex> lk(S->mu);
             S->cv_work.wait(lk, [&] {
@@ -322,6 +354,20 @@ void worker(nk_server *S)
                 }
                 if (job.size() > 1) need = pneed;
             }
+            // the job's share, and the state of the batches that run beside its first one
+            int64_t kj = 0, arcs = 0;
+            double all = S->work_running;
+            for (const Request *r : job) {
+                kj += r->k;
+                arcs += r->g->A;
+                work += work_of(r);
+            }
+            all += work;
+            for (const Request *r : S->queue) all += work_of(r);
+            const int width = job.size() > 1 ? kPackWidth : request_batch(S, job[0]->g, job[0]->k);
+            share = share_of(work, all, arcs, (int)((kj + width - 1) / width), need, (S->budget - S->used - need) / 2);
+            need *= (size_t)share.teams;
+            S->work_running += work;
             S->used += need;
             S->peak_bytes = std::max(S->peak_bytes, S->used);
             const auto now = clk::now();
@@ -334,13 +380,14 @@ void worker(nk_server *S)
             ++S->launches_jobs;
             if (job.size() > 1) S->packed += (int64_t)job.size();
         }
-        const int rc = job.size() == 1 ? run_request(S, job[0], st, &h_buf, &h_cap)
-                                       : run_pack(S, job, st, &h_buf, &h_cap);
+        const int rc = job.size() == 1 ? run_request(S, job[0], share, st, &h_buf, &h_cap)
+                                       : run_pack(S, job, share, st, &h_buf, &h_cap);
         const std::string msg = rc == NK_OK ? std::string() : std::string(nk_last_error());
         {
             std::lock_guard<std::mutex> lk(S->mu);
             const auto done = clk::now();
             S->used -= need;
+            S->work_running -= work;
             if (--S->running == 0) S->busy_s += std::chrono::duration<double>(done - S->busy_since).count();
             for (Request *r : job) {
                 r->t_done = done;
