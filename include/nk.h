@@ -140,12 +140,14 @@ int nk_sssp_noalloc(int32_t n, const int32_t *row_ptr, const int32_t *col, int64
                     int32_t s, int32_t *dist, uint64_t *sigma, void *stream);
 
 /* ---------------------------------------------------------------- betweenness */
-#define NK_MODE_AUTO 0       /* batched where it fits, per-source otherwise */
+#define NK_MODE_AUTO 0       /* batched where it fits (below 16 sources in batches of 8),
+                                per-source otherwise and for a single source */
 #define NK_MODE_PER_SOURCE 1 /* plain per-source kernel (one BFS tree at a time); backward levels
                                 whose successors carry few arcs add psi with FP64 atomics, so the
                                 last bits of its scores may differ from run to run (distances and
                                 path counts never do) */
-#define NK_MODE_BATCHED 2    /* bitset multi-source kernel, `batch` sources per launch */
+#define NK_MODE_BATCHED 2    /* bitset multi-source kernel, `batch` sources per batch, several
+                                batches per launch */
 
 #define NK_DIR_AUTO 0        /* direction-optimising: switch by alpha */
 #define NK_DIR_TOP_DOWN 1    /* every level top-down (push from the frontier) */
@@ -165,7 +167,7 @@ int nk_sssp_noalloc(int32_t n, const int32_t *row_ptr, const int32_t *col, int64
 
 typedef struct nk_run_opts {
     int32_t mode;      /* NK_MODE_* */
-    int32_t batch;     /* batched mode: sources per batch, 64/128/256; 0 = autotuned */
+    int32_t batch;     /* batched mode: sources per batch, 64/128/256; 0 = autotuned, or by k */
     int32_t tpv;       /* accepted for compatibility (0 or a power of 2 <= 32) and ignored: the
                           per-source sweep runs lanes over the arcs of groups of vertices */
     int32_t direction; /* NK_DIR_* */
@@ -296,7 +298,8 @@ int nk_edge_betweenness_sampled(const nk_graph *g, uint64_t seed, int32_t k, dou
  * so that closeness(v) = reach[v] / far[v] ((n-1) / sum_u d(u, v) on a connected graph).
  * Exact: S = V, scale 1 (the sums are exact integers).  Sampled: S from
  * nk_sample_sources(n, seed, k), scale n/k.  far and reach hold n doubles each (device
- * pointers with NK_RUN_DEVICE_PTRS).  The batched form runs its forward sweep only. */
+ * pointers with NK_RUN_DEVICE_PTRS).  The batched form sweeps level bitsets
+ * without path counts. */
 int nk_closeness_exact(const nk_graph *g, double *far, double *reach);
 int nk_closeness_sampled(const nk_graph *g, uint64_t seed, int32_t k, double *far, double *reach,
                          const nk_run_opts *opts);

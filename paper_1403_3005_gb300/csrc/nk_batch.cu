@@ -1,5 +1,5 @@
-// Batched multi-source betweenness: B = 64*W sources share one persistent cooperative
-// launch.  The paper parallelises Brandes' algorithm over sources with one dependency
+// Batched multi-source betweenness: B = 64*W sources share one sweep, and several such batches
+// one persistent cooperative launch, a row of the grid each.  The paper parallelises Brandes' algorithm over sources with one dependency
 // array per thread, summed at the end (Section 3.2); on the GPU the sources of a batch
 // instead share every pass over the CSR, so the adjacency of a level is read once for
 // all B shortest-path trees.
@@ -15,10 +15,10 @@
 //               iterated by scanning F_d)
 // Forward level d, either
 //   bottom-up  every vertex w with unvisited sources u = act & ~vis[w] gathers F_d of
-//              its neighbours (one warp per vertex, lanes over neighbours); for every
-//              neighbour c with F_d[c] & u != 0 the lanes switch to one lane per source
-//              bit and add sigma_b(c) (the sigma row of c is contiguous, so the gather
-//              reads only the sectors of the sources that need it);
+//              its neighbours (a warp per group of vertices, lanes over their arcs); for
+//              every neighbour c with F_d[c] & u != 0 the lanes switch to the source slots
+//              and add sigma_b(c) (the sigma row of c is contiguous, so the gather reads
+//              only the sectors of the sources that need it);
 //              F_{d+1}[w] = the bits whose sum is non-zero;  or
 //   top-down   (a) every frontier vertex v pushes m = F_d[v] & ~vis[c] into F_{d+1}[c]
 //              (atomicOr) and queues c once per level; (b) every queued vertex w pulls

@@ -856,7 +856,8 @@ __global__ void k_add_distances(const int32_t *dist, int32_t n, unsigned long lo
     }
 }
 
-// CTAs of a sweep: no more than a small graph can use (32, 64, 128 and 256 at least measured alike).
+// CTAs of a sweep: no more than a small graph can use, whose barriers get dearer with every one (the
+// same bound as the batched sweep's).
 int sweep_grid(int grid, int32_t n) { return std::max(1, std::min(grid, std::max(128, n / 64))); }
 
 // ------------------------------------------------------------------ host side

@@ -48,14 +48,6 @@ template <int W> __device__ __forceinline__ bool any_bits(const Bits<W> &b)
     return o != 0;
 }
 
-template <int W> __device__ __forceinline__ Bits<W> shfl_bits(const Bits<W> &b, int src)
-{
-    Bits<W> r;
-#pragma unroll
-    for (int q = 0; q < W; ++q) r.w[q] = __shfl_sync(FULL, b.w[q], src);
-    return r;
-}
-
 template <int W> __device__ __forceinline__ Bits<W> andnot(const Bits<W> &x, const Bits<W> &y)
 {
     Bits<W> r;
