@@ -146,10 +146,13 @@ int run_captured(nk_graph *g, uint64_t seed, int32_t k, double scale, double *d_
     if (cfg.relabel && build_relabeled(g, s) != NK_OK) cfg.relabel = false;
     // with relabelling the sweep runs on the copy: sources mapped in, scores gathered back
     nk_graph *gr = cfg.relabel ? g->relab.get() : g;
+    // the kernel nodes hold what the arguments alone do not fix: the pointers of the chunk table, which
+    // a call with another chunk size frees and rebuilds, and the bound on device-side waits
+    const uint64_t limit = cfg.limit_ns ? cfg.limit_ns : wait_limit_ns();
     const bool hit = e.valid && e.seed == seed && e.k == k && e.batch == cfg.batch &&
                      e.alpha == cfg.alpha && e.dir == cfg.direction && e.scores == d_scores &&
                      e.scale == scale && e.grid_ctas == cfg.grid_ctas && e.chunk == cfg.chunk &&
-                     e.relabel == cfg.relabel;
+                     e.relabel == cfg.relabel && e.table == table_build(gr, cfg.chunk) && e.limit_ns == limit;
     if (!hit) {
         e.reset();
         NK_TRY(e.src.ensure(sizeof(int32_t) * k));
@@ -210,6 +213,8 @@ int run_captured(nk_graph *g, uint64_t seed, int32_t k, double scale, double *d_
         e.grid_ctas = cfg.grid_ctas;
         e.chunk = cfg.chunk;
         e.relabel = cfg.relabel;
+        e.table = table_build(gr, cfg.chunk);
+        e.limit_ns = limit;
         e.nb = nb;
         e.launches = captured;
     }

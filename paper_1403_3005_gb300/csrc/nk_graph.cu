@@ -590,6 +590,7 @@ int heavy_view(nk_graph *g, int chunk, cudaStream_t s, HeavyView *out)
     if (g->heavy_alt_H < 0 || g->heavy_alt_chunk != chunk) {
         int32_t H = -1, C = 0;
         g->heavy_alt_H = -1;
+        ++g->heavy_alt_build;
         NK_TRY(build_table(g, chunk, g->heavy_alt, H, C, nullptr, nullptr, s));
         g->heavy_alt_H = H;
         g->heavy_alt_C = C;
@@ -598,6 +599,11 @@ int heavy_view(nk_graph *g, int chunk, cudaStream_t s, HeavyView *out)
     *out = {g->heavy_alt[0].as<int32_t>(), g->heavy_alt[1].as<int32_t>(), g->heavy_alt[2].as<int32_t>(),
             g->heavy_alt_H, g->heavy_alt_C, chunk};
     return NK_OK;
+}
+
+uint64_t table_build(const nk_graph *g, int chunk)
+{
+    return chunk <= 0 || chunk == kHeavyChunk ? 0 : g->heavy_alt_build;
 }
 
 __global__ void k_relabel_perm(int32_t n, int32_t *perm)

@@ -103,6 +103,9 @@ struct CapturedRun {
     bool relabel = false;
     double alpha = 0, scale = 0;
     double *scores = nullptr;
+    // recorded in the kernel nodes too: which build of the swept graph's second chunk table
+    // (0: the run reads the graph's own table, which is never rebuilt), and the wait bound
+    uint64_t table = 0, limit_ns = 0;
     DevBuf ws[8];
     DevBuf src, msrc, iscores;  // sources; relabelled sources and scores (relabel only)
     Ctrl *h_status = nullptr;  // pinned copy of the per-batch status words
@@ -154,6 +157,7 @@ struct nk_graph {
     // a second chunk table with another chunk size, for the batched sweep only (built on demand)
     nk::DevBuf heavy_alt[3];
     int32_t heavy_alt_H = -1, heavy_alt_C = 0, heavy_alt_chunk = 0;
+    uint64_t heavy_alt_build = 0;         // counts its builds; each may free the table before
     nk::DevBuf wt;                        // int32[A] arc weights (nk_weighted.cu), when weighted
     bool weighted = false;
     // relabelled copy for the batched sweep (vertex v of this graph is vertex relab_perm[v] of
@@ -199,6 +203,9 @@ struct HeavyView {
     int32_t H, C, chunk;
 };
 int heavy_view(nk_graph *g, int chunk, cudaStream_t s, HeavyView *out);
+// What tells one chunk table from another at the same addresses: 0 for the graph's own table, else
+// the number of the second table's present build.
+uint64_t table_build(const nk_graph *g, int chunk);
 // Relabelling for the batched sweep: vertex v becomes (v * kRelabelMul) mod n, a bijection
 // (kRelabelMul is a prime above 2^31, so it has no factor in common with n).  Vertex ids of
 // power-law generators cluster the hubs at small ids; scattered ids spread them over the

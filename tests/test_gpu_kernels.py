@@ -178,3 +178,45 @@ def test_csr_rows_at_the_sort_sizes(nk):
     rp, col = oracle.csr_build(n, u, v)
     a, b = g.export_csr()
     assert np.array_equal(a, rp) and np.array_equal(b, col)
+
+
+@pytest.mark.parametrize("flag", ["RUN_NO_RELABEL", "RUN_RELABEL"])
+def test_captured_run_after_another_chunk_size(nk, flag):
+    """A captured run reads the chunk table that its kernel nodes point to.  A call with another chunk
+    size in between rebuilds that table (with chunks of 32 arcs a larger one, elsewhere in memory)."""
+    import torch
+    n, u, v = GROUPS["rows"]
+    g = nk.graph_from_edges(n, u, v)
+    rp, col = oracle.csr_build(n, u, v)
+    ref = oracle.betweenness_sampled(rp, col, 3, 150)
+    out, other = (torch.empty(n, dtype=torch.float64, device="cuda") for _ in range(2))
+    flags = getattr(nk, flag)
+    captured = nk.run_opts(mode=nk.MODE_BATCHED, batch=64, chunk=128, flags=flags | nk.RUN_CUDA_GRAPH)
+    for chunk in (0, 32, 96, 128):
+        if chunk:
+            nk.betweenness_sampled(g, 3, 150, nk.run_opts(mode=nk.MODE_BATCHED, batch=64, chunk=chunk, flags=flags), out=other)
+            assert np.allclose(other.cpu().numpy(), ref, rtol=1e-9, atol=1e-12)
+        for _ in range(2):
+            out.fill_(-1.0)
+            nk.betweenness_sampled(g, 3, 150, captured, out=out)
+            assert np.allclose(out.cpu().numpy(), ref, rtol=1e-9, atol=1e-12)
+
+
+def test_captured_run_follows_the_wait_limit(nk):
+    """The bound on device-side waits is part of a captured run: a later nk_set_wait_limit_ns holds for
+    the same call too (a bound of 1 ns runs out at once, the default one does not)."""
+    import torch
+    g = nk.graph_generate("er", 3000, 4, avg_deg=8.0)
+    out = torch.empty(3000, dtype=torch.float64, device="cuda")
+    o = nk.run_opts(mode=nk.MODE_BATCHED, batch=64, flags=nk.RUN_CUDA_GRAPH)
+    nk.betweenness_sampled(g, 3, 100, o, out=out)
+    want = out.cpu().numpy().copy()
+    try:
+        nk.set_wait_limit_ns(1)
+        with pytest.raises(nk.NkError) as e:
+            nk.betweenness_sampled(g, 3, 100, o, out=out)
+        assert e.value.rc == nk.ERR_TIMEOUT
+    finally:
+        nk.set_wait_limit_ns(10_000_000_000)  # the default
+    nk.betweenness_sampled(g, 3, 100, o, out=out)
+    assert np.array_equal(out.cpu().numpy(), want)
