@@ -10,7 +10,11 @@
 // (1 + delta) / sigma of its successors; psi replaces sigma in the row.  Path counts are 64-bit
 // throughout (an overflow is reported).  Rows longer than the hub chunk are summed from per-chunk
 // partials in chunk order, so results do not depend on timing.  Several batches run side by side,
-// one per row of the grid.
+// one per row of the grid.  Sums of psi, and of a vertex's dependencies over its sources, are rounded once
+// (ff_sum): added step by step in double-single, scores of 2 to 15 sources were up to twice as far
+// from FP64 as the per-source form's (ER 112063, degree 22, 13 sources, 2-norm: 3.5e-15 against 1.5e-15,
+// now 5e-16).  It costs 2 to 3 % (R-MAT 20, 8 sources, 3.37 -> 3.44 ms); FP64 sums are as exact and cost
+// 10 to 17 %.
 //
 // What bounds it: the latency of the dependent reads column id -> level byte -> row entry (48
 // registers for 40 warps an SM: 5 blocks 3.4 ms on R-MAT 20 with 8 sources, 4 3.6, 6 3.4, R-MAT 22
@@ -55,7 +59,7 @@ struct TArgs {
     int32_t *vcnt, *qcnt;        // [teams][lcap+3]
     unsigned long long *mfv, *dmu;  // [teams][lcap+3]
     int32_t *wq;                 // [teams][lcap+3][8]
-    unsigned long long *part;    // [teams][C][8]
+    unsigned long long *part;    // [teams][C][8] a hub chunk's path counts, or its psi (double)
     double *scores;              // [teams][n]
     Ctrl *ctrl;
     uint64_t limit_ns;
@@ -83,7 +87,7 @@ struct ThinBuf {
 // it; a part without work has dg = 0.
 template <bool PSI>
 __device__ __forceinline__ void thin_gather(const TArgs &a, int beg, int dg, unsigned t, const unsigned char *Fsel,
-                                            int parts, unsigned long long &acc, dev::ff &facc, bool &ovf)
+                                            int parts, unsigned long long &acc, dev::ff_sum &facc, bool &ovf)
 {
     const int lane = threadIdx.x & 31, slot = lane & 7;
     const unsigned long long *rows = a.sp + (size_t)blockIdx.y * a.n * kT + slot;
@@ -112,7 +116,7 @@ __device__ __forceinline__ void thin_gather(const TArgs &a, int beg, int dg, uns
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
                 if constexpr (PSI) {
-                    facc = dev::ff_add(facc, dev::ff_unpack(x[r]));
+                    if (r < left) facc.add(dev::ff_unpack(x[r]));  // uniform
                 } else {
                     acc += x[r];
                     ovf |= acc < x[r];
@@ -124,10 +128,7 @@ __device__ __forceinline__ void thin_gather(const TArgs &a, int beg, int dg, uns
 #pragma unroll
         for (int o = 8; o < 32; o <<= 1) {
             if constexpr (PSI) {
-                dev::ff y;
-                y.hi = __shfl_xor_sync(FULL, facc.hi, o);
-                y.lo = __shfl_xor_sync(FULL, facc.lo, o);
-                facc = dev::ff_add(facc, y);
+                facc.join(o);
             } else {
                 const unsigned long long y = __shfl_xor_sync(FULL, acc, o);
                 acc += y;
@@ -306,7 +307,7 @@ __global__ void __launch_bounds__(kThreads, 5) k_thin(TArgs a)
             if (!__any_sync(FULL, on)) return;
             if (chunk >= 0) {
                 unsigned long long acc = 0;
-                dev::ff facc;
+                dev::ff_sum facc;
                 thin_gather<false>(a, beg, dg, __shfl_sync(FULL, t, 0), Fd, 4, acc, facc, ovf);
                 if (part == 0) a.part[((size_t)blockIdx.y * a.C + chunk) * kT + slot] = acc;
                 return;
@@ -314,7 +315,7 @@ __global__ void __launch_bounds__(kThreads, 5) k_thin(TArgs a)
             unsigned done = 0;
             each_row(on, v, beg, dg, t, [&](int o, int w, int b, int g, unsigned tw, int parts) {
                 unsigned long long acc = 0;
-                dev::ff facc;
+                dev::ff_sum facc;
                 thin_gather<false>(a, b, g, tw, Fd, parts, acc, facc, ovf);
                 const bool mine = o >= 0 && (parts == 1 || part == 0) && acc != 0;
                 if (mine) rows[(size_t)w * kT + slot] = acc;
@@ -380,15 +381,16 @@ __global__ void __launch_bounds__(kThreads, 5) k_thin(TArgs a)
 
     // backward: psi and delta of vertex v from its successor sums (the lane's slot), delta summed
     // over the part's 8 lanes into the score; one warp adds to a vertex's score per level
-    auto finish = [&](bool in, int v, dev::ff acc) {
-        dev::ff delta = dev::ff_zero();
+    auto finish = [&](bool in, int v, const dev::ff_sum &acc) {
+        dev::ff_sum delta;
         if (in) {
             const dev::ff s = dev::ff_from_u64(__ldcg(rows + (size_t)v * kT + slot));
-            rows[(size_t)v * kT + slot] = dev::ff_pack(dev::ff_add(dev::ff_rcp(s), acc));
-            delta = dev::ff_mul(s, acc);
+            rows[(size_t)v * kT + slot] = dev::ff_pack(dev::ff_add(dev::ff_rcp(s), acc.value()));
+            delta = acc.times(s);
         }
-        delta = dev::group_sum_ff<8>(delta);
-        if (slot == 0 && delta.hi != 0.0f) atomicAdd(a.scores + tn + v, dev::ff_to_double(delta));
+#pragma unroll
+        for (int o = 1; o < kT; o <<= 1) delta.join(o);
+        if (slot == 0 && delta.s != 0.0f) atomicAdd(a.scores + tn + v, delta.to_double());
     };
     for (int l = D; l >= 1; --l) {
         const unsigned char *Fl = a.level(l), *Fs = a.level(l + 1);
@@ -402,13 +404,13 @@ __global__ void __launch_bounds__(kThreads, 5) k_thin(TArgs a)
             unsigned long long acc = 0;
             bool dummy = false;
             if (chunk >= 0) {
-                dev::ff facc = dev::ff_zero();
+                dev::ff_sum facc;
                 thin_gather<true>(a, beg, dg, __shfl_sync(FULL, t, 0), Fs, 4, acc, facc, dummy);
-                if (part == 0) a.part[((size_t)blockIdx.y * a.C + chunk) * kT + slot] = dev::ff_pack(facc);
+                if (part == 0) a.part[((size_t)blockIdx.y * a.C + chunk) * kT + slot] = (unsigned long long)__double_as_longlong(facc.to_double());
                 return;
             }
             each_row(on, v, beg, dg, t, [&](int o, int w, int b, int g, unsigned tw, int parts) {
-                dev::ff facc = dev::ff_zero();
+                dev::ff_sum facc;
                 thin_gather<true>(a, b, g, tw, Fs, parts, acc, facc, dummy);
                 finish(o >= 0 && (parts == 1 || part == 0) && ((tw >> slot) & 1u), w, facc);
             });
@@ -418,17 +420,12 @@ __global__ void __launch_bounds__(kThreads, 5) k_thin(TArgs a)
             for_heavy(a, [&](int, int h, int c0, int c1) {
                 const unsigned t = __ldcg(Fl + h);
                 if (!t) return;
-                dev::ff facc = dev::ff_zero();
+                double facc = 0.0;
                 for (int c = c0 + part; c < c1; c += 4)
-                    facc = dev::ff_add(facc, dev::ff_unpack(__ldcg(a.part + ((size_t)blockIdx.y * a.C + c) * kT + slot)));
+                    facc += __longlong_as_double((long long)__ldcg(a.part + ((size_t)blockIdx.y * a.C + c) * kT + slot));
 #pragma unroll
-                for (int o = 8; o < 32; o <<= 1) {
-                    dev::ff y;
-                    y.hi = __shfl_xor_sync(FULL, facc.hi, o);
-                    y.lo = __shfl_xor_sync(FULL, facc.lo, o);
-                    facc = dev::ff_add(facc, y);
-                }
-                finish(part == 0 && ((t >> slot) & 1u), h, facc);
+                for (int o = 8; o < 32; o <<= 1) facc += __shfl_xor_sync(FULL, facc, o);
+                finish(part == 0 && ((t >> slot) & 1u), h, dev::ff_sum(facc));
             });
         }
         if (!dev::grid_barrier(a.status(), a.limit_ns)) return;

@@ -220,3 +220,17 @@ def test_captured_run_follows_the_wait_limit(nk):
         nk.set_wait_limit_ns(10_000_000_000)  # the default
     nk.betweenness_sampled(g, 3, 100, o, out=out)
     assert np.array_equal(out.cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("avg_deg", [15.0, 22.0])
+@pytest.mark.parametrize("k", [4, 6, 13])
+def test_few_sources_are_as_exact_as_one_by_one(nk, avg_deg, k):
+    """Scores of a few sources swept together are no further from the oracle's FP64 than those of the
+    per-source form, a quarter allowed for the oracle's own rounding and the order of the sums."""
+    g = nk.graph_generate("er", 5000, 3, avg_deg=avg_deg)
+    n, rp, col = oracle.generate("er", 5000, 3, avg_deg=avg_deg)
+    src = oracle.sample_sources(n, 5, k)
+    ref = oracle.betweenness_sources(rp, col, src, 1.0)
+    off = [np.linalg.norm(nk.betweenness_sources(g, src, 1.0, nk.run_opts(mode=m)) - ref) / np.linalg.norm(ref)
+           for m in (nk.MODE_AUTO, nk.MODE_PER_SOURCE)]
+    assert off[0] <= 1.25 * off[1], off
