@@ -188,7 +188,9 @@ typedef struct nk_run_stats {
     int32_t batch;           /* sources per batch used (1 for per-source) */
     int32_t tpv;
     int32_t max_depth;       /* deepest BFS level seen */
-    int64_t launches;        /* sweep-kernel launches */
+    int64_t launches;        /* sweeps: batches of sources (reruns too), or sources one by one; one for
+                                a weighted call.  A launch may hold several batches:
+                                nk_last_run_launches counts launches */
     double kernel_ms;        /* sum of sweep-kernel durations (CUDA events), if timed */
     int64_t td_levels;       /* levels run top-down / bottom-up */
     int64_t bu_levels;
@@ -214,6 +216,11 @@ int nk_betweenness_sources(const nk_graph *g, const int32_t *src, int32_t k, dou
 /* Stats of the calling thread's last betweenness call (no counterpart in the paper:
  * launch width, levels run top-down and bottom-up, kernel time). */
 int nk_last_run_stats(nk_run_stats *out);
+
+/* Launches of the sweep kernel in that call: at most stats.launches, fewer where batches ran side by
+ * side.  Divide kernel_ms by it for the average duration of a launch, by stats.launches for that of a
+ * sweep. */
+int nk_last_run_launches(int64_t *launches);
 
 /* Autotuner (no counterpart in the paper; it tunes the batched GPU sweep, which is this
  * library's own design): on up to 256 of the run's own sources (seed, k), times the

@@ -1259,6 +1259,7 @@ int launch_batches(nk_graph *g, const int32_t *d_src, int32_t k, double *d_score
             st->batch = B;
             st->tpv = 32;
             st->launches += (int64_t)todo.size();
+            st->kernel_launches += ((int64_t)todo.size() + teams - 1) / teams;
             st->alpha = alpha_used;
             for (int bi : todo) {
                 st->max_depth = std::max(st->max_depth, h[bi].depth);

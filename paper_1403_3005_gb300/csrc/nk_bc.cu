@@ -232,7 +232,7 @@ int run_captured(nk_graph *g, uint64_t seed, int32_t k, double scale, double *d_
     t_stats.mode = NK_MODE_BATCHED;
     t_stats.batch = e.batch;
     t_stats.tpv = 32;
-    t_stats.launches = e.nb;
+    t_stats.launches = t_stats.kernel_launches = e.nb;
     t_stats.alpha = e.alpha;
     if (cfg.time_kernels) {
         float ms = 0;
@@ -769,6 +769,13 @@ int nk_last_run_stats(nk_run_stats *out)
     out->td_levels = t_stats.td_levels;
     out->bu_levels = t_stats.bu_levels;
     out->alpha = t_stats.alpha;
+    return NK_OK;
+}
+
+int nk_last_run_launches(int64_t *launches)
+{
+    if (!launches) return set_error(NK_ERR_ARG, "launches is null");
+    *launches = t_stats.kernel_launches;
     return NK_OK;
 }
 

@@ -254,7 +254,9 @@ inline DevBuf *scratch(const RunCfg &c, nk_graph *g);
 
 struct RunStats {
     int mode = 0, batch = 0, tpv = 0, max_depth = 0;
-    int64_t launches = 0, td_levels = 0, bu_levels = 0;
+    int64_t launches = 0;         // sweeps: batches, or sources one by one
+    int64_t kernel_launches = 0;  // launches of the sweep kernel, which may hold several batches
+    int64_t td_levels = 0, bu_levels = 0;
     double kernel_ms = 0.0, alpha = 0.0;
 };
 

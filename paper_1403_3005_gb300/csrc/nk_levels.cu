@@ -418,6 +418,7 @@ int run_levels_w(nk_graph *g, const int32_t *d_src, int32_t k, const RunCfg &cfg
     NK_TRY(rc);
     st->tpv = 32;
     st->launches += nb;
+    st->kernel_launches += nb;
     st->alpha = a.alpha;
     for (const Ctrl &c : h) {
         if (c.err == NK_ERR_TIMEOUT)

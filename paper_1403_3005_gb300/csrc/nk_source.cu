@@ -998,6 +998,7 @@ int run(nk_graph *g, const int32_t *d_src, int32_t k, double *d_scores, const Ru
         st->tpv = L.tpv;
         st->max_depth = std::max(st->max_depth, h.depth);
         st->launches += k;
+        st->kernel_launches += k;
         st->td_levels += h.td_levels;
         st->bu_levels += h.bu_levels;
         st->alpha = a.alpha;

@@ -574,6 +574,7 @@ int run_thin(nk_graph *g, const int32_t *d_src, int32_t k, double *d_scores, con
         NK_TRY(rc);
         st->tpv = 8;
         st->launches += (int64_t)todo.size();
+        st->kernel_launches += ((int64_t)todo.size() + side - 1) / side;
         st->alpha = a.alpha;
         std::vector<int> deep;
         bool ovf = false;

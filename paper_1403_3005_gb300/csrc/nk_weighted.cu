@@ -532,6 +532,7 @@ int run_weighted(nk_graph *g, const int32_t *d_src, int32_t k, double *d_scores,
         st->batch = groups;  // searches running side by side
         st->tpv = cpg;       // CTAs per search
         st->launches += k > 0 ? 1 : 0;
+        st->kernel_launches += k > 0 ? 1 : 0;
         st->max_depth = std::max(st->max_depth, depth);
         if (cfg.time_kernels) {
             float ms = 0;

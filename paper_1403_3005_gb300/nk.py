@@ -107,6 +107,7 @@ SIGNATURES = {
     "nk_closeness_exact": (_INT, [_P, _P, _P]),
     "nk_closeness_sampled": (_INT, [_P, _U64, _I32, _P, _P, _P]),
     "nk_last_run_stats": (_INT, [_P]),
+    "nk_last_run_launches": (_INT, [_P]),
     "nk_autotune": (_INT, [_P, _U64, _I32, _P]),
     "nk_server_create": (_INT, [_P, _P]),
     "nk_server_destroy": (None, [_P]),
@@ -541,7 +542,9 @@ def closeness_sampled(g: Graph, seed: int, k: int, opts: RunOpts | None = None, 
 def last_run_stats() -> dict:
     st = RunStats()
     _check(lib().nk_last_run_stats(ctypes.byref(st)))
-    return st.as_dict()
+    launches = ctypes.c_int64()
+    _check(lib().nk_last_run_launches(ctypes.byref(launches)))
+    return dict(st.as_dict(), kernel_launches=launches.value)
 
 
 def autotune(g: Graph, seed: int, k: int) -> RunOpts:

@@ -234,3 +234,28 @@ def test_few_sources_are_as_exact_as_one_by_one(nk, avg_deg, k):
     off = [np.linalg.norm(nk.betweenness_sources(g, src, 1.0, nk.run_opts(mode=m)) - ref) / np.linalg.norm(ref)
            for m in (nk.MODE_AUTO, nk.MODE_PER_SOURCE)]
     assert off[0] <= 1.25 * off[1], off
+
+
+def test_launches_and_sweeps_are_told_apart(nk):
+    """Stats: batches, sources or searches swept, and the launches that held them."""
+    g = nk.graph_generate("er", 1500, 4, avg_deg=8.0)
+    n, rp, col = oracle.generate("er", 1500, 4, avg_deg=8.0)
+    with_arcs = lambda k: int((np.diff(rp)[oracle.sample_sources(n, 2, k)] > 0).sum())  # noqa: E731
+    stats = lambda: tuple(nk.last_run_stats()[x] for x in ("launches", "kernel_launches"))  # noqa: E731
+    for k in (300, 64):
+        batches = (with_arcs(k) + 63) // 64
+        for call in (nk.betweenness_sampled, nk.edge_betweenness_sampled):
+            call(g, 2, k, nk.run_opts(mode=nk.MODE_BATCHED, batch=64))
+            assert stats() == (batches, 1)  # one launch, side by side
+        nk.closeness_sampled(g, 2, k, nk.run_opts(mode=nk.MODE_BATCHED, batch=64))
+        assert stats() == (batches, batches)
+        # a grid given by the caller holds one batch at a time
+        nk.betweenness_sampled(g, 2, k, nk.run_opts(mode=nk.MODE_BATCHED, batch=64, grid_ctas=200))
+        assert stats() == (batches, batches)
+    nk.betweenness_sampled(g, 2, 15)
+    assert stats() == ((with_arcs(15) + 7) // 8, 1)
+    nk.betweenness_sampled(g, 2, 5, nk.run_opts(mode=nk.MODE_PER_SOURCE))
+    assert stats() == (with_arcs(5), with_arcs(5))
+    nk.random_weights(g, 1, 4)
+    nk.betweenness_weighted_sampled(g, 2, 5)
+    assert stats() == (1, 1)
