@@ -1055,20 +1055,33 @@ constexpr int kTeamCtas = 128, kTeamVertices = 64;
 // 10.0, -, 9.8; BA 10^6 (4) 31.5, 29.9, 30.0; R-MAT 20 36.2, 34.4, 35.8, 40.3; R-MAT 22 133, 132,
 // 136, 146; R-MAT 24 320, 320.  The number of teams per launch is evened out; the batches stay full and
 // the last one short (made equal, R-MAT 18 takes 12.9 instead of 11.3 ms: a row read serves fewer).  Callers with their
-// own workspace or grid (captured graphs) run one batch at a time unless they say how many (servers).
-int choose_teams(const nk_graph *g, int B, size_t state, int nb, int grid, const RunCfg &cfg, const DevBuf *ws, int64_t outs)
+// own workspace or grid (captured graphs) run one batch at a time unless they say how many at most (servers).
+//
+// The sums are kept apart from how many run at once: batch i of a call adds to vector i mod P, in the
+// order of the batches, and the P vectors are added up in their order, where P is the number of teams
+// that the graph and the batches ask for.  Free memory, or a server's load, may make the teams fewer
+// without changing a bit of the scores.
+int choose_partials(const nk_graph *g, int B, int nb, const RunCfg &cfg)
 {
     if (nb < 2 || (cfg.teams <= 0 && (cfg.ws || cfg.grid_ctas > 0))) return 1;
     const size_t rows = (size_t)g->n * B * 12;
-    int want = std::min(nb, std::min(kMaxTeams, grid));
-    want = cfg.teams > 0 ? std::min(want, cfg.teams) : (int)std::min<size_t>(want, (kTeamRows + rows - 1) / rows);
-    size_t free_b = 0, total_b = 0;
-    cudaMemGetInfo(&free_b, &total_b);
-    const size_t per = state + sizeof(double) * (size_t)outs;
-    while (want > 1 && per * want > (free_b + ws[WS_BATCH].bytes) / 4) --want;
+    int want = (int)std::min<size_t>(std::min(nb, kMaxTeams), (kTeamRows + rows - 1) / rows);
     while (want > 1 && (int64_t)g->n * want > INT32_MAX) --want;  // rows are numbered in 32 bits
     const int rounds = (nb + want - 1) / want;
     return (nb + rounds - 1) / rounds;
+}
+
+// Teams of a launch: `partials` of them if a quarter of the memory holds their state beside the vectors
+// (`outs` sums each), and no more than the caller asks for.
+int choose_teams(size_t state, int partials, int grid, const RunCfg &cfg, const DevBuf *ws, int64_t outs)
+{
+    int want = std::min(partials, grid);
+    if (cfg.teams > 0) want = std::min(want, cfg.teams);
+    size_t free_b = 0, total_b = 0;
+    cudaMemGetInfo(&free_b, &total_b);
+    const size_t sums = sizeof(double) * (size_t)outs * partials;
+    while (want > 1 && state * want + sums > (free_b + ws[WS_BATCH].bytes) / 4) --want;
+    return want;
 }
 
 // Blocks of a team: its share of the grid, but no more than a small graph can use, whose barriers get
@@ -1128,16 +1141,6 @@ BArgs make_args(const nk_graph *g, const Layout &L, int teams, const HeavyView &
     a.alpha = cfg.alpha > 0 ? cfg.alpha : 1.0;
     a.dir = cfg.direction;
     return a;
-}
-
-// out[i] += the teams' sums, in their order
-__global__ void k_add_teams(const double *t, int32_t teams, int64_t count, double *out)
-{
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
-        double x = out[i];
-        for (int32_t j = 0; j < teams; ++j) x += t[(size_t)j * count + i];
-        out[i] = x;
-    }
 }
 
 template <int W>
@@ -1216,19 +1219,19 @@ int launch_batches(nk_graph *g, const int32_t *d_src, int32_t k, double *d_score
     }
     for (int lcap = lstart;;) {
         // reruns of some of the batches go one by one
-        const int teams = (int)todo.size() == nb ? choose_teams(g, B, layout(g, B, lcap, hw.chunk).total, nb, grid, cfg, ws, a_out) : 1;
+        int partials = (int)todo.size() == nb ? choose_partials(g, B, nb, cfg) : 1;
+        Tmp outs;
+        if (partials > 1 && a_out > 0 && outs.alloc(sizeof(double) * (size_t)a_out * partials, s) != NK_OK)
+            partials = 1;  // no room for the vectors: batch after batch into one
+        const int teams = choose_teams(layout(g, B, lcap, hw.chunk).total, partials, grid, cfg, ws, a_out);
         const Layout L = layout(g, B, lcap, hw.chunk, teams);
         NK_TRY(ws[WS_BATCH].ensure(L.total));
         BArgs a = make_args(g, L, teams, hw, ws[WS_BATCH].as<char>(), d_scores, cfg);
         a.src = d_src;
         a.nsrc = k;
         a.ctrl = ctrls;
-        Tmp outs;
-        if (teams > 1 && a_out > 0) {
-            NK_TRY(outs.alloc(sizeof(double) * (size_t)a_out * teams, s));
-            NK_CUDA(cudaMemsetAsync(outs.p, 0, sizeof(double) * (size_t)a_out * teams, s));
-            (edge ? a.edge : a.scores) = outs.as<double>();
-        }
+        if (outs.p) NK_CUDA(cudaMemsetAsync(outs.p, 0, sizeof(double) * (size_t)a_out * partials, s));
+        int64_t sweep_launches = 0;
         NK_CUDA(cudaMemsetAsync(ctrls, 0, sizeof(Ctrl) * nb, s));
         cudaEvent_t e0 = nullptr, e1 = nullptr;
         if (cfg.time_kernels) {
@@ -1236,20 +1239,20 @@ int launch_batches(nk_graph *g, const int32_t *d_src, int32_t k, double *d_score
             NK_CUDA(cudaEventCreate(&e1));
             NK_CUDA(cudaEventRecord(e0, s));
         }
-        for (size_t t = 0; t < todo.size(); t += teams) {
+        for (size_t t = 0; t < todo.size();) {
             a.b0 = todo[t];
             a.trace = (trace_on && t == 0) ? trace_buf.as<unsigned long long>() : nullptr;
-            const int now = std::min<int>(teams, (int)(todo.size() - t));  // the last launch's teams are larger
+            // the last launch's teams are larger; a launch's batches add to vectors in a row
+            const int at = a.b0 % partials;
+            const int now = std::min<int>(std::min(teams, partials - at), (int)(todo.size() - t));
+            if (outs.p) (edge ? a.edge : a.scores) = outs.as<double>() + (size_t)at * a_out;
             void *args[] = {&a};
             NK_CUDA(cudaLaunchCooperativeKernel(kfn, dim3(team_ctas(g, grid, now), now), dim3(kThreads), args, edge ? smem_bytes<W, true>() : smem_bytes<W, false>(), s));
             ::nk::count_launch();
+            ++sweep_launches;
+            t += now;
         }
-        if (outs.p) {
-            const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((a_out + 255) / 256, 8LL * num_sms()));
-            k_add_teams<<<blocks, 256, 0, s>>>(outs.as<double>(), teams, a_out, edge ? cfg.edge : d_scores);
-            ::nk::count_launch();
-            NK_CUDA(cudaGetLastError());
-        }
+        if (outs.p) NK_TRY(add_vectors(outs.as<double>(), partials, a_out, edge ? cfg.edge : d_scores, s));
         if (cfg.time_kernels) NK_CUDA(cudaEventRecord(e1, s));
         std::vector<Ctrl> h(nb);
         NK_CUDA(cudaMemcpyAsync(h.data(), ctrls, sizeof(Ctrl) * nb, cudaMemcpyDeviceToHost, s));
@@ -1259,7 +1262,7 @@ int launch_batches(nk_graph *g, const int32_t *d_src, int32_t k, double *d_score
             st->batch = B;
             st->tpv = 32;
             st->launches += (int64_t)todo.size();
-            st->kernel_launches += ((int64_t)todo.size() + teams - 1) / teams;
+            st->kernel_launches += sweep_launches;
             st->alpha = alpha_used;
             for (int bi : todo) {
                 st->max_depth = std::max(st->max_depth, h[bi].depth);

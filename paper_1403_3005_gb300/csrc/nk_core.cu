@@ -370,6 +370,27 @@ int order_sources(const nk_graph *g, const int32_t *d_src, int32_t k, const int3
     return NK_OK;
 }
 
+// ---------------------------------------------------------------- sums of vectors
+namespace {
+__global__ void k_add_vectors(const double *v, int32_t vectors, int64_t count, double *out)
+{
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
+        double x = out[i];
+        for (int32_t j = 0; j < vectors; ++j) x += v[(size_t)j * count + i];
+        out[i] = x;
+    }
+}
+}  // namespace
+
+int add_vectors(const double *v, int32_t vectors, int64_t count, double *out, cudaStream_t s)
+{
+    const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>((count + 255) / 256, 8LL * num_sms()));
+    k_add_vectors<<<blocks, 256, 0, s>>>(v, vectors, count, out);
+    ::nk::count_launch();
+    NK_CUDA(cudaGetLastError());
+    return NK_OK;
+}
+
 // ---------------------------------------------------------------- vector scale
 namespace {
 __global__ void k_scale(double *d, int32_t n, double s)

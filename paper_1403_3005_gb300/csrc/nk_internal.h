@@ -315,6 +315,9 @@ int compact_sources(const nk_graph *g, const int32_t *d_src, int32_t k, int32_t 
 int order_sources(const nk_graph *g, const int32_t *d_src, int32_t k, const int32_t *d_count,
                   unsigned long long *d_key, int32_t *d_out, cudaStream_t s);
 
+// out[i] += the sum of the `vectors` device vectors of `count` entries at v, in their order.
+int add_vectors(const double *v, int32_t vectors, int64_t count, double *out, cudaStream_t s);
+
 // Scale a device vector in place.
 int scale_vector(double *d, int32_t n, double scale, cudaStream_t s);
 

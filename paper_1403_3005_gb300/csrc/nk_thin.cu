@@ -432,16 +432,6 @@ __global__ void __launch_bounds__(kThreads, 5) k_thin(TArgs a)
     }
 }
 
-// out[i] += the teams' sums, in their order
-__global__ void k_add_teams(const double *t, int32_t teams, int64_t count, double *out)
-{
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
-        double x = out[i];
-        for (int32_t j = 0; j < teams; ++j) x += t[(size_t)j * count + i];
-        out[i] = x;
-    }
-}
-
 enum { WS_BATCH = 5, WS_BCTRL = 6 };
 
 }  // namespace
@@ -555,11 +545,7 @@ int run_thin(nk_graph *g, const int32_t *d_src, int32_t k, double *d_scores, con
             NK_CUDA(cudaLaunchCooperativeKernel((const void *)k_thin, dim3(ctas, now), dim3(kThreads), args, 0, s));
             ::nk::count_launch();
         }
-        if (side > 1) {
-            k_add_teams<<<(unsigned)std::max<size_t>(1, std::min<size_t>((n + 255) / 256, 8 * (size_t)num_sms())), 256, 0, s>>>(
-                outs.as<double>(), side, (int64_t)n, d_scores);
-            ::nk::count_launch();
-        }
+        if (side > 1) NK_TRY(add_vectors(outs.as<double>(), side, (int64_t)n, d_scores, s));
         if (cfg.time_kernels) NK_CUDA(cudaEventRecord(e1, s));
         std::vector<Ctrl> h(nb);
         NK_CUDA(cudaMemcpyAsync(h.data(), ctrls, sizeof(Ctrl) * nb, cudaMemcpyDeviceToHost, s));

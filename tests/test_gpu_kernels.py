@@ -259,3 +259,23 @@ def test_launches_and_sweeps_are_told_apart(nk):
     nk.random_weights(g, 1, 4)
     nk.betweenness_weighted_sampled(g, 2, 5)
     assert stats() == (1, 1)
+
+
+@pytest.mark.parametrize("kind,n,params,k", [("er", 3000, dict(avg_deg=8.0), 2900), ("ba", 4000, dict(m0=6), 700)])
+def test_scores_do_not_depend_on_how_many_batches_run_at_once(nk, kind, n, params, k):
+    """The same request with room for many batches side by side and with room for one at a time, and
+    the same call without a server: the sums are added in one order, so the scores are equal."""
+    g = nk.graph_generate(kind, n, 6, **params)
+    probe = nk.Server(max_inflight=1, pack=False)
+    assert probe.wait(probe.submit(g, 1, 100)[0], 300.0) == nk.OK
+    need = probe.stats()["peak_bytes"]
+    got = []
+    for budget in (0, 1.3 * need):
+        srv = nk.Server(mem_budget_bytes=budget, max_inflight=1, pack=False, batch=128)
+        rid, out = srv.submit(g, 1, k)
+        assert srv.wait(rid, 300.0) == nk.OK
+        got.append(out.copy())
+        srv.close()
+    probe.close()
+    got.append(nk.betweenness_sampled(g, 1, k, nk.run_opts(mode=nk.MODE_BATCHED, batch=128)))
+    assert np.array_equal(got[0], got[1]) and np.array_equal(got[0], got[2])
