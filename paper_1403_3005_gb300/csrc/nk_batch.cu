@@ -1064,11 +1064,7 @@ constexpr int kTeamCtas = 128, kTeamVertices = 64;
 int choose_partials(const nk_graph *g, int B, int nb, const RunCfg &cfg)
 {
     if (nb < 2 || (cfg.teams <= 0 && (cfg.ws || cfg.grid_ctas > 0))) return 1;
-    const size_t rows = (size_t)g->n * B * 12;
-    int want = (int)std::min<size_t>(std::min(nb, kMaxTeams), (kTeamRows + rows - 1) / rows);
-    while (want > 1 && (int64_t)g->n * want > INT32_MAX) --want;  // rows are numbered in 32 bits
-    const int rounds = (nb + want - 1) / want;
-    return (nb + rounds - 1) / rounds;
+    return batch_partials(g->n, B, nb);
 }
 
 // Teams of a launch: `partials` of them if a quarter of the memory holds their state beside the vectors
@@ -1077,8 +1073,7 @@ int choose_teams(size_t state, int partials, int grid, const RunCfg &cfg, const 
 {
     int want = std::min(partials, grid);
     if (cfg.teams > 0) want = std::min(want, cfg.teams);
-    size_t free_b = 0, total_b = 0;
-    cudaMemGetInfo(&free_b, &total_b);
+    const size_t free_b = free_bytes(ws[WS_BATCH].stream_ordered);
     const size_t sums = sizeof(double) * (size_t)outs * partials;
     while (want > 1 && state * want + sums > (free_b + ws[WS_BATCH].bytes) / 4) --want;
     return want;
@@ -1414,6 +1409,15 @@ int enqueue_batches(nk_graph *g, const int32_t *d_src, int32_t k, double *d_scor
 }
 
 }  // namespace
+
+int batch_partials(int32_t n, int B, int nb)
+{
+    const size_t rows = (size_t)n * B * 12;
+    int want = (int)std::min<size_t>(std::min(nb, kMaxTeams), (kTeamRows + rows - 1) / rows);
+    while (want > 1 && (int64_t)n * want > INT32_MAX) --want;  // rows are numbered in 32 bits
+    const int rounds = (nb + want - 1) / want;
+    return (nb + rounds - 1) / rounds;
+}
 
 size_t batched_bytes(const nk_graph *g, int B) { return layout(g, B, 16).total; }
 

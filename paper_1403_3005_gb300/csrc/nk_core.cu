@@ -74,6 +74,20 @@ static void keep_pool_memory()
     done.fetch_or(bit);
 }
 
+size_t free_bytes(bool pool)
+{
+    size_t free_b = 0, total_b = 0;
+    if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) return 0;
+    int dev = 0;
+    cudaMemPool_t p;
+    uint64_t held = 0, used = 0;
+    if (pool && cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetDefaultMemPool(&p, dev) == cudaSuccess &&
+        cudaMemPoolGetAttribute(p, cudaMemPoolAttrReservedMemCurrent, &held) == cudaSuccess &&
+        cudaMemPoolGetAttribute(p, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess && held > used)
+        free_b += (size_t)(held - used);
+    return free_b;
+}
+
 int DevBuf::ensure(size_t b)
 {
     if (b <= bytes && p) return NK_OK;

@@ -69,6 +69,10 @@ struct DevBuf {
     DevBuf &operator=(const DevBuf &) = delete;
 };
 
+// Free device memory; with `pool`, what the device's default memory pool holds without using it
+// counts as free (to a stream-ordered allocation it is).
+size_t free_bytes(bool pool);
+
 // Stream-ordered temporary (cudaMallocAsync / cudaFreeAsync on the library stream).
 struct Tmp {
     void *p = nullptr;
@@ -233,7 +237,7 @@ struct RunCfg {
     DevBuf *ws = nullptr;  // scratch slots (8); null = the graph's cached workspace
     int grid_div = 1;      // persistent grids use 1/grid_div of the co-resident CTAs
     int grid_ctas = 0;     // if > 0: persistent grids use at most this many CTAs
-    int teams = 0;         // batched sweep, if > 0: batches side by side (0: chosen by the graph's size)
+    int teams = 0;         // batched sweep, if > 0: most batches side by side (0: by the graph's size alone)
     int lcap = 0;          // batched level slabs; 0 = sized from free memory
     uint64_t limit_ns = 0; // bound on device-side waits; 0 = the process-wide bound
     bool backward = true;  // false: forward sweep only
@@ -296,6 +300,9 @@ int enqueue_batched(nk_graph *g, const int32_t *d_src, int32_t k, double *d_scor
 size_t batched_bytes(const nk_graph *g, int B);
 
 inline DevBuf *scratch(const RunCfg &c, nk_graph *g) { return c.ws ? c.ws : g->ws; }
+
+// Batches of B sources that run side by side at most, of the nb of a call on n vertices.
+int batch_partials(int32_t n, int B, int nb);
 
 // Device bytes of a batched run with B sources per batch and lcap level slabs.
 size_t batched_bytes_lcap(const nk_graph *g, int B, int lcap);

@@ -107,19 +107,19 @@ struct Share {
 
 double work_of(const Request *r) { return (double)r->g->A * (double)r->k + 1.0; }
 
-// `work` of `all` the work at hand, on `arcs` arcs in `nb` batches; `bytes`: device bytes of one
-// batch's state, `room`: what may be used for more of them.  (128 sources a launch use 4 CTAs per
+// `work` of `all` the work at hand, on `arcs` arcs, whose batches could run `most` at a time; `bytes`:
+// device bytes of one batch's state, `room`: what may be used for more of them.  (128 sources a launch use 4 CTAs per
 // SM.)  CTAs by the graph alone and one batch at a time, against this: one request of 500 sources on ER
 // 100000 10.7 / 5.4 ms, of 1000 on R-MAT 16 7.4 / 4.5; 16 mixed requests 17.4 / 14.4, 64 79 / 75.  By the
 // share alone, without the lower bound, the 64 took 119 ms; with the bound but one batch at a time the
 // 16 took 18.5.
-Share share_of(double work, double all, int64_t arcs, int nb, size_t bytes, size_t room)
+Share share_of(double work, double all, int64_t arcs, int most, size_t bytes, size_t room)
 {
     Share s;
     const int sms = num_sms();
     const double least = (double)std::max<int64_t>(kShareMin, arcs / kShareArcs);
     s.ctas = (int)std::min(2.0 * sms, std::max(least, 4.0 * sms * work / all));
-    s.teams = std::max(1, std::min(nb, s.ctas / kTeamMin));
+    s.teams = std::max(1, std::min(most, s.ctas / kTeamMin));
     while (s.teams > 1 && bytes * (size_t)(s.teams - 1) > room) --s.teams;
     return s;
 }
@@ -355,17 +355,22 @@ void worker(nk_server *S)
                 if (job.size() > 1) need = pneed;
             }
             // the job's share, and the state of the batches that run beside its first one
-            int64_t kj = 0, arcs = 0;
+            int64_t kj = 0, arcs = 0, verts = 0;
             double all = S->work_running;
             for (const Request *r : job) {
                 kj += r->k;
                 arcs += r->g->A;
+                verts += r->g->n;
                 work += work_of(r);
             }
             all += work;
             for (const Request *r : S->queue) all += work_of(r);
             const int width = job.size() > 1 ? kPackWidth : request_batch(S, job[0]->g, job[0]->k);
-            share = share_of(work, all, arcs, (int)((kj + width - 1) / width), need, (S->budget - S->used - need) / 2);
+            // memory for them: up to the slot's part of the budget and half of what is left of it, so that
+            // the requests of the other slots find theirs
+            const size_t left = S->budget - S->used - need, part = S->budget / (size_t)S->slots;
+            const size_t room = std::min(left / 2, part > need ? part - need : 0);
+            share = share_of(work, all, arcs, batch_partials((int32_t)verts, width, (int)((kj + width - 1) / width)), need, room);
             need *= (size_t)share.teams;
             S->work_running += work;
             S->used += need;

@@ -279,3 +279,21 @@ def test_scores_do_not_depend_on_how_many_batches_run_at_once(nk, kind, n, param
     probe.close()
     got.append(nk.betweenness_sampled(g, 1, k, nk.run_opts(mode=nk.MODE_BATCHED, batch=128)))
     assert np.array_equal(got[0], got[1]) and np.array_equal(got[0], got[2])
+
+
+def test_served_batches_side_by_side_within_a_slots_memory(nk):
+    """Batches beside a request's first one take memory within the slot's part of the budget, and no
+    more of them are counted than the sweep runs side by side on a graph of that size."""
+    def peak(g, k, **kw):
+        srv = nk.Server(pack=False, batch=128, **kw)
+        assert srv.wait(srv.submit(g, 1, k)[0], 300.0) == nk.OK
+        bytes_ = srv.stats()["peak_bytes"]
+        srv.close()
+        return bytes_
+
+    g = nk.graph_generate("er", 3000, 6, avg_deg=8.0)
+    one = peak(g, 100, max_inflight=1)
+    assert peak(g, 1000, max_inflight=4, mem_budget_bytes=4.4 * one) < 1.1 * one
+    assert 3.9 * one < peak(g, 1000, max_inflight=4, mem_budget_bytes=18 * one) <= 4.5 * one
+    g = nk.graph_generate("er", 1 << 20, 6, avg_deg=4.0)
+    assert peak(g, 1024, max_inflight=1) < 3.1 * peak(g, 100, max_inflight=1)
