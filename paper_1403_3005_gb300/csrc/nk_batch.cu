@@ -1044,16 +1044,19 @@ int choose_lcap(const nk_graph *g, int B, const DevBuf *ws, int chunk = 0)
 enum { WS_BATCH = 5, WS_BCTRL = 6 };
 
 constexpr int kMaxTeams = 64;
-constexpr size_t kTeamRows = 3300u << 20;  // bytes of sigma and psi rows that teams share
+constexpr size_t kTeamRows = 3300u << 20;  // bytes of sigma and psi rows from which on no team is added
 constexpr int kTeamCtas = 128, kTeamVertices = 64;
 
 // Batches run side by side, each by a team of blocks with its own state: one batch of a small graph
 // cannot use the GPU, and on the others teams fill the tails of each other's phases.  As many as
-// there are batches while their rows stay within kTeamRows together, beyond which they only take
-// memory and cache from each other.  1, 2, 4, 8 and all batches at once, 128 sources each: ER 2000
+// there are batches until their rows reach kTeamRows together (the last team may go beyond it, to at
+// most twice that), from where on they only take memory and cache from each other.  1, 2, 4, 8 and all batches at once, 128 sources each: ER 2000
 // exact 3.3, 1.7, 0.87, 0.60, 0.46 ms; R-MAT 14 3.7, 2.3, 1.25, 0.98; R-MAT 18 (6) 13.2, 10.6,
 // 10.0, -, 9.8; BA 10^6 (4) 31.5, 29.9, 30.0; R-MAT 20 36.2, 34.4, 35.8, 40.3; R-MAT 22 133, 132,
-// 136, 146; R-MAT 24 320, 320.  The number of teams per launch is evened out; the batches stay full and
+// 136, 146; R-MAT 24 320, 320.  Stopping short of kTeamRows, with 2 instead of 3 teams on 2^20 vertices
+// (k = 600, 1000): R-MAT 20 of 31M arcs 24.0 against 26.3 ms and 36.6 / 37.5, of 16M arcs 15.7 / 14.2 and 23.4 / 21.2;
+// ER 900000 39.6 / 39.8 and 64.9 / 65.3; on 2^21, 1 against 2, R-MAT 21 of 32M arcs 28.9 / 28.0 and 38.8 / 38.2.
+// The number of teams per launch is evened out; the batches stay full and
 // the last one short (made equal, R-MAT 18 takes 12.9 instead of 11.3 ms: a row read serves fewer).  Callers with their
 // own workspace or grid (captured graphs) run one batch at a time unless they say how many at most (servers).
 //

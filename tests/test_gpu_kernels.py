@@ -297,3 +297,13 @@ def test_served_batches_side_by_side_within_a_slots_memory(nk):
     assert 3.9 * one < peak(g, 1000, max_inflight=4, mem_budget_bytes=18 * one) <= 4.5 * one
     g = nk.graph_generate("er", 1 << 20, 6, avg_deg=4.0)
     assert peak(g, 1024, max_inflight=1) < 3.1 * peak(g, 100, max_inflight=1)
+
+
+def test_rows_side_by_side(nk):
+    """Path-count and psi rows of the batches that share a launch: 12 bytes a source and vertex, batches
+    until they reach 3300 MB together.  2^20 vertices, 128 sources (1536 MB each): three batches."""
+    g = nk.graph_generate("er", 1 << 20, 6, avg_deg=4.0)
+    for k, batches, launches in ((700, 6, 2), (300, 3, 1)):
+        nk.betweenness_sampled(g, 1, k, nk.run_opts(mode=nk.MODE_BATCHED, batch=128))
+        st = nk.last_run_stats()
+        assert (st["launches"], st["kernel_launches"]) == (batches, launches)
