@@ -1329,6 +1329,7 @@ int launch_batches(nk_graph *g, const int32_t *d_src, int32_t k, double *d_score
         for (int bi : deep) {
             RunCfg pc = cfg;
             pc.tpv = 0;
+            pc.compacted = true;
             if (pc.rk_t) {
                 pc.rk_t += (size_t)bi * B;
                 pc.rk_key += (size_t)bi * B;

@@ -247,6 +247,7 @@ struct RunCfg {
     int chunk = 0;                        // batched sweep: arcs per hub chunk (0: kHeavyChunk)
     bool relabel = false;                 // betweenness entry: use the relabelled copy
     bool keep_order = false;              // batched sweep: batches in the order the sources are given
+    bool compacted = false;               // per-source form: every source is known to have arcs
     // error-bounded estimate: per source index i, the target of its random shortest path,
     // the key of the walk's random stream, and the per-vertex counts of interior vertices
     const int32_t *rk_t = nullptr;

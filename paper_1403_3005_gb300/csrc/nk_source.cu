@@ -952,7 +952,7 @@ int run(nk_graph *g, const int32_t *d_src, int32_t k, double *d_scores, const Ru
     // others are swept (not for a single-source sweep, whose outputs the caller reads, nor
     // for the error-bounded estimate, whose sources are tied to their targets)
     Tmp csrc, ccnt;
-    if (!d_dist_out && !cfg.rk_t && k > 0) {
+    if (!d_dist_out && !cfg.rk_t && !cfg.compacted && k > 0) {
         NK_TRY(csrc.alloc(sizeof(int32_t) * (size_t)k, s));
         NK_TRY(ccnt.alloc(sizeof(int32_t), s));
         NK_TRY(compact_sources(g, d_src, k, csrc.as<int32_t>(), ccnt.as<int32_t>(), s));

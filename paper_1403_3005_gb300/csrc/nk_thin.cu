@@ -461,8 +461,10 @@ int run_thin(nk_graph *g, const int32_t *d_src, int32_t k, double *d_scores, con
     // 1.6 / 1.2; R-MAT 20 1.0 / 2.4, 2.0 / 2.6, 3.3 / 3.0, 4.4 / 3.0, 7.8 / 3.4; R-MAT 22 3.0 / 7.4, 5.1 / 8.0, 8.5 / 9.5,
     // 11.6 / 9.7, 21.7 / 12.2
     const bool hubs = (int64_t)hw.C * hw.chunk > g->A / 4;
+    RunCfg pc = cfg;  // of the per-source form
+    pc.compacted = true;
     if (k == 1 || (hubs && ((k == 2 && g->A >= (4 << 20)) || (k == 3 && g->A >= (64 << 20)))))
-        return run_per_source(g, d_src, k, d_scores, cfg, st, s);
+        return run_per_source(g, d_src, k, d_scores, pc, st, s);
     DevBuf *ws = scratch(cfg, g);
     const int nb = (k + kT - 1) / kT;
     NK_TRY(ws[WS_BCTRL].ensure(sizeof(Ctrl) * nb));
@@ -583,7 +585,7 @@ int run_thin(nk_graph *g, const int32_t *d_src, int32_t k, double *d_scores, con
         }
         // deeper than any level cap: the per-source form takes these sources
         for (int bi : deep)
-            NK_TRY(run_per_source(g, d_src + (size_t)bi * kT, std::min(kT, k - bi * kT), d_scores, cfg, st, s));
+            NK_TRY(run_per_source(g, d_src + (size_t)bi * kT, std::min(kT, k - bi * kT), d_scores, pc, st, s));
         return NK_OK;
     }
 }

@@ -307,3 +307,19 @@ def test_rows_side_by_side(nk):
         nk.betweenness_sampled(g, 1, k, nk.run_opts(mode=nk.MODE_BATCHED, batch=128))
         st = nk.last_run_stats()
         assert (st["launches"], st["kernel_launches"]) == (batches, launches)
+
+
+@pytest.mark.parametrize("kind,n,params,k", [("er", 2000, dict(avg_deg=8.0), 1), ("rmat", 18, dict(edge_factor=16), 2)])
+def test_sources_swept_one_by_one_are_compacted_once(nk, kind, n, params, k):
+    """A single source, and two on a large hub graph, take the per-source form from the library's own
+    choice with the launches that the form takes when it is asked for."""
+    g = nk.graph_generate(kind, n, 4, **params)
+    src = np.argsort(-np.diff(g.export_csr()[0]))[5:5 + k].astype(np.int32)  # vertices with arcs
+    launches, scores = [], []
+    for mode in (nk.MODE_AUTO, nk.MODE_PER_SOURCE):
+        before = nk.launch_count()
+        scores.append(nk.betweenness_sources(g, src, 1.0, nk.run_opts(mode=mode)))
+        launches.append(nk.launch_count() - before)
+        assert nk.last_run_stats()["mode"] == nk.MODE_PER_SOURCE
+    assert launches[0] == launches[1]
+    assert np.allclose(scores[0], scores[1], rtol=1e-9, atol=1e-12)
