@@ -1141,40 +1141,21 @@ BArgs make_args(const nk_graph *g, const Layout &L, int teams, const HeavyView &
     return a;
 }
 
+// d_count: the number of sources on the device, if they may be put in another order (all have arcs)
 template <int W>
-int launch_batches(nk_graph *g, const int32_t *d_src, int32_t k, double *d_scores,
+int launch_batches(nk_graph *g, const int32_t *d_src, int32_t k, const int32_t *d_count, double *d_scores,
                    const RunCfg &cfg, RunStats *st, cudaStream_t s)
 {
     constexpr int B = 64 * W;
-    // sources without arcs add nothing: the batches take the others (the error-bounded
-    // estimate keeps its slots, which are tied to their targets)
-    Tmp csrc, ccnt, osrc, okey;
-    if (!cfg.rk_t) {
-        NK_TRY(csrc.alloc(sizeof(int32_t) * (size_t)k, s));
-        NK_TRY(ccnt.alloc(sizeof(int32_t), s));
-        NK_TRY(compact_sources(g, d_src, k, csrc.as<int32_t>(), ccnt.as<int32_t>(), s));
-        int32_t kk = 0;
-        NK_CUDA(cudaMemcpyAsync(&kk, ccnt.p, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-        NK_CUDA(cudaStreamSynchronize(s));
-        if (kk < 0 || kk > k) return set_error(NK_ERR_CUDA, "source compaction returned %d of %d", kk, k);
-        d_src = csrc.as<int32_t>();
-        k = kk;
-        if (k == 0) {
-            if (st) {
-                st->mode = NK_MODE_BATCHED;
-                st->batch = B;
-            }
-            return NK_OK;
-        }
-        // more than one batch: similar sources share one.  R-MAT 18, 670 sources by 128: 65.2M
-        // rows gathered in the order of the ids, 42.8M in this order, 18.3 -> 13.4 ms; R-MAT 24,
-        // 271 sources: 493 -> 348 ms; BA 10^6, 512 sources: 40.2 -> 36.9 ms; ER (no hubs) equal
-        if (k > B && !cfg.keep_order) {
-            NK_TRY(osrc.alloc(sizeof(int32_t) * (size_t)k, s));
-            NK_TRY(okey.alloc(sizeof(unsigned long long) * (size_t)k, s));
-            NK_TRY(order_sources(g, d_src, k, ccnt.as<int32_t>(), okey.as<unsigned long long>(), osrc.as<int32_t>(), s));
-            d_src = osrc.as<int32_t>();
-        }
+    // more than one batch: similar sources share one.  R-MAT 18, 670 sources by 128: 65.2M
+    // rows gathered in the order of the ids, 42.8M in this order, 18.3 -> 13.4 ms; R-MAT 24,
+    // 271 sources: 493 -> 348 ms; BA 10^6, 512 sources: 40.2 -> 36.9 ms; ER (no hubs) equal
+    Tmp osrc, okey;
+    if (d_count && k > B && !cfg.keep_order) {
+        NK_TRY(osrc.alloc(sizeof(int32_t) * (size_t)k, s));
+        NK_TRY(okey.alloc(sizeof(unsigned long long) * (size_t)k, s));
+        NK_TRY(order_sources(g, d_src, k, d_count, okey.as<unsigned long long>(), osrc.as<int32_t>(), s));
+        d_src = osrc.as<int32_t>();
     }
     HeavyView hw;
     NK_TRY(heavy_view(g, cfg.chunk, s, &hw));
@@ -1430,12 +1411,23 @@ size_t batched_bytes_lcap(const nk_graph *g, int B, int lcap) { return layout(g,
 int run_batched(nk_graph *g, const int32_t *d_src, int32_t k, double *d_scores,
                 const RunCfg &cfg, RunStats *st, cudaStream_t s)
 {
+    // sources without arcs add nothing: the batches, and the choice of their width, take the others
+    // (the error-bounded estimate keeps its slots, which are tied to their targets)
+    Tmp list, count;
+    if (!cfg.rk_t) NK_TRY(compact_list(g, &d_src, &k, list, count, s));
     int B = cfg.batch;
     if (B == 0) B = g->tuned.valid ? g->tuned.batch : default_width(g, k, cfg);
+    if (k == 0) {
+        if (st) {
+            st->mode = NK_MODE_BATCHED;
+            st->batch = B;
+        }
+        return NK_OK;
+    }
     switch (B) {
-    case 64: return launch_batches<1>(g, d_src, k, d_scores, cfg, st, s);
-    case 128: return launch_batches<2>(g, d_src, k, d_scores, cfg, st, s);
-    case 256: return launch_batches<4>(g, d_src, k, d_scores, cfg, st, s);
+    case 64: return launch_batches<1>(g, d_src, k, count.as<int32_t>(), d_scores, cfg, st, s);
+    case 128: return launch_batches<2>(g, d_src, k, count.as<int32_t>(), d_scores, cfg, st, s);
+    case 256: return launch_batches<4>(g, d_src, k, count.as<int32_t>(), d_scores, cfg, st, s);
     default: return set_error(NK_ERR_ARG, "batch must be 64, 128 or 256 (got %d)", B);
     }
 }

@@ -325,6 +325,20 @@ int compact_sources(const nk_graph *g, const int32_t *d_src, int32_t k, int32_t 
     return NK_OK;
 }
 
+int compact_list(const nk_graph *g, const int32_t **d_src, int32_t *k, Tmp &list, Tmp &count, cudaStream_t s)
+{
+    NK_TRY(list.alloc(sizeof(int32_t) * (size_t)*k, s));
+    NK_TRY(count.alloc(sizeof(int32_t), s));
+    NK_TRY(compact_sources(g, *d_src, *k, list.as<int32_t>(), count.as<int32_t>(), s));
+    int32_t kk = 0;
+    NK_CUDA(cudaMemcpyAsync(&kk, count.p, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
+    NK_CUDA(cudaStreamSynchronize(s));
+    if (kk < 0 || kk > *k) return set_error(NK_ERR_CUDA, "source compaction returned %d of %d", kk, *k);
+    *d_src = list.as<int32_t>();
+    *k = kk;
+    return NK_OK;
+}
+
 // ---------------------------------------------------------------- similar sources together
 namespace {
 constexpr int kKeyArcs = 2048;      // arcs of a source that its key looks at

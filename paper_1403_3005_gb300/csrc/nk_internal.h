@@ -315,6 +315,10 @@ size_t batched_bytes_lcap(const nk_graph *g, int B, int lcap);
 int compact_sources(const nk_graph *g, const int32_t *d_src, int32_t k, int32_t *d_out, int32_t *d_count,
                     cudaStream_t s);
 
+// The same with the count on the host: *d_src and *k become the compacted list's, which `list` holds
+// (its count on the device: `count`).  Waits for s.
+int compact_list(const nk_graph *g, const int32_t **d_src, int32_t *k, Tmp &list, Tmp &count, cudaStream_t s);
+
 // Orders the sources d_src[0..*d_count) (device; k is an upper bound of the count) so that
 // consecutive ones have similar BFS trees: by the number of two-step walks from them, largest
 // first.  A batch of the multi-source sweep reads a neighbour's row once for all sources that

@@ -323,26 +323,14 @@ template <int W> __global__ void __launch_bounds__(kThreads, 4) k_levels(LArgs a
 enum { WS_BATCH = 5, WS_BCTRL = 6 };
 
 template <int W>
-int run_levels_w(nk_graph *g, const int32_t *d_src, int32_t k, const RunCfg &cfg, RunStats *st, cudaStream_t s)
+int run_levels_w(nk_graph *g, const int32_t *d_src, int32_t k, const int32_t *d_count, const RunCfg &cfg, RunStats *st, cudaStream_t s)
 {
     constexpr int B = 64 * W;
-    Tmp csrc, ccnt, osrc, okey;
-    NK_TRY(csrc.alloc(sizeof(int32_t) * (size_t)k, s));
-    NK_TRY(ccnt.alloc(sizeof(int32_t), s));
-    NK_TRY(compact_sources(g, d_src, k, csrc.as<int32_t>(), ccnt.as<int32_t>(), s));
-    int32_t kk = 0;
-    NK_CUDA(cudaMemcpyAsync(&kk, ccnt.p, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-    NK_CUDA(cudaStreamSynchronize(s));
-    if (kk < 0 || kk > k) return set_error(NK_ERR_CUDA, "source compaction returned %d of %d", kk, k);
-    d_src = csrc.as<int32_t>();
-    k = kk;
-    st->mode = NK_MODE_BATCHED;
-    st->batch = B;
-    if (k == 0) return NK_OK;
+    Tmp osrc, okey;
     if (k > B) {  // similar sources share a batch and its bottom-up levels
         NK_TRY(osrc.alloc(sizeof(int32_t) * (size_t)k, s));
         NK_TRY(okey.alloc(sizeof(unsigned long long) * (size_t)k, s));
-        NK_TRY(order_sources(g, d_src, k, ccnt.as<int32_t>(), okey.as<unsigned long long>(), osrc.as<int32_t>(), s));
+        NK_TRY(order_sources(g, d_src, k, d_count, okey.as<unsigned long long>(), osrc.as<int32_t>(), s));
         d_src = osrc.as<int32_t>();
     }
     HeavyView hw;
@@ -435,12 +423,18 @@ int run_levels_w(nk_graph *g, const int32_t *d_src, int32_t k, const RunCfg &cfg
 
 int run_levels(nk_graph *g, const int32_t *d_src, int32_t k, const RunCfg &cfg, RunStats *st, cudaStream_t s)
 {
-    // without a width from the caller: the narrowest that takes all sources in one launch, up to 256
+    Tmp list, count;
+    NK_TRY(compact_list(g, &d_src, &k, list, count, s));
+    // without a width from the caller: the narrowest that takes all sources (with arcs) in one launch,
+    // up to 256
     const int B = cfg.batch ? cfg.batch : k > 128 ? 256 : k > 64 ? 128 : 64;
+    st->mode = NK_MODE_BATCHED;
+    st->batch = B;
+    if (k == 0) return NK_OK;
     switch (B) {
-    case 64: return run_levels_w<1>(g, d_src, k, cfg, st, s);
-    case 128: return run_levels_w<2>(g, d_src, k, cfg, st, s);
-    case 256: return run_levels_w<4>(g, d_src, k, cfg, st, s);
+    case 64: return run_levels_w<1>(g, d_src, k, count.as<int32_t>(), cfg, st, s);
+    case 128: return run_levels_w<2>(g, d_src, k, count.as<int32_t>(), cfg, st, s);
+    case 256: return run_levels_w<4>(g, d_src, k, count.as<int32_t>(), cfg, st, s);
     default: return set_error(NK_ERR_ARG, "batch must be 64, 128 or 256 (got %d)", B);
     }
 }

@@ -323,3 +323,20 @@ def test_sources_swept_one_by_one_are_compacted_once(nk, kind, n, params, k):
         assert nk.last_run_stats()["mode"] == nk.MODE_PER_SOURCE
     assert launches[0] == launches[1]
     assert np.allclose(scores[0], scores[1], rtol=1e-9, atol=1e-12)
+
+
+def test_width_follows_the_sources_with_arcs(nk):
+    """150 sources, 100 of them with arcs, without a width from the caller: the width of 100 sources."""
+    rng = np.random.default_rng(5)
+    n, u, v = 1500, rng.integers(0, 1000, 6000), rng.integers(0, 1000, 6000)
+    g = nk.graph_from_edges(n, u.astype(np.int32), v.astype(np.int32))
+    rp, col = oracle.csr_build(n, u.astype(np.int32), v.astype(np.int32))
+    src = np.concatenate([np.arange(1000, 1050), np.flatnonzero(np.diff(rp) > 0)[:100]]).astype(np.int32)
+    got = nk.betweenness_sources(g, src, 1.0)
+    assert nk.last_run_stats()["batch"] == 64
+    assert np.allclose(got, oracle.betweenness_sources(rp, col, src, 1.0), rtol=1e-9, atol=1e-12)
+    seed = next(s for s in range(100) if (np.diff(rp)[oracle.sample_sources(n, s, 150)] > 0).sum() <= 128)
+    far, reach = nk.closeness_sampled(g, seed, 150)
+    assert nk.last_run_stats()["batch"] == 128
+    ref = oracle.closeness_sampled(rp, col, seed, 150)
+    assert np.array_equal(far, ref[0]) and np.array_equal(reach, ref[1])
