@@ -200,17 +200,19 @@ __device__ __forceinline__ dev::ff edge_sum2(dev::ff a, dev::ff b)
 // 16- and 8-byte loads that bypass L1, zeros where `on` is zero.  Written out so that a load is
 // predicated: the compiler made it a branch, and R-MAT 18 took 13.6 instead of 12.5 ms.  (Reading
 // a dummy address instead takes 33 ms: the lanes of all warps meet in one L2 slice.)
+// "memory" keeps them in order with the plain stores to the rows that they read; with it and without
+// it every form of the kernel takes the same registers and spills.
 __device__ __forceinline__ void load16_if(unsigned on, const void *p, unsigned &x, unsigned &y, unsigned &z, unsigned &w)
 {
     x = y = z = w = 0;
     asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %4, 0;\n\t@p ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%5];\n\t}"
-                 : "+r"(x), "+r"(y), "+r"(z), "+r"(w) : "r"(on), "l"(p));
+                 : "+r"(x), "+r"(y), "+r"(z), "+r"(w) : "r"(on), "l"(p) : "memory");
 }
 __device__ __forceinline__ void load8_if(unsigned on, const void *p, unsigned &x, unsigned &y)
 {
     x = y = 0;
     asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %2, 0;\n\t@p ld.global.cg.v2.u32 {%0, %1}, [%3];\n\t}"
-                 : "+r"(x), "+r"(y) : "r"(on), "l"(p));
+                 : "+r"(x), "+r"(y) : "r"(on), "l"(p) : "memory");
 }
 
 // acc += x where on is not zero

@@ -103,6 +103,22 @@ def test_noalloc_refuses_bad_buffers_before_any_launch(libpath):
     assert nk.launch_count() == launches
 
 
+# ---------------------------------------------------------------- sources
+def test_inline_memory_accesses_are_ordered():
+    """An inline-PTX load or store names memory among what it changes: without that the compiler may
+    move it across the plain accesses to the same rows."""
+    import re
+    csrc = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1403_3005_gb300", "csrc")
+    seen = 0
+    for name in sorted(os.listdir(csrc)):
+        text = open(os.path.join(csrc, name)).read()
+        for m in re.finditer(r"\basm\b[^;]*\((?:[^()\"]|\"(?:[^\"\\]|\\.)*\"|\([^()]*\))*\);", text):
+            if re.search(r"\b(ld|st|red|atom)\.(global|shared|volatile|relaxed|acquire|release)", m.group(0)):
+                seen += 1
+                assert '"memory"' in m.group(0), (name, m.group(0))
+    assert seen >= 2
+
+
 # ---------------------------------------------------------------- multi-rank sharding
 def test_source_shard_partitions_the_set():
     from paper_1403_3005_gb300 import nk
