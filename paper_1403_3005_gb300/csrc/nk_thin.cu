@@ -481,12 +481,13 @@ int run_thin(nk_graph *g, const int32_t *d_src, int32_t k, double *d_scores, con
     Ctrl *ctrls = ws[WS_BCTRL].as<Ctrl>();
     std::vector<int> todo(nb);
     for (int i = 0; i < nb; ++i) todo[i] = i;
-    // level slabs: 48 at first; deeper searches run again with up to an eighth of the free memory
+    // level slabs: 48 at first; deeper searches run again with those that an eighth of the free memory,
+    // 8 GB at most, holds for the batches side by side together
     size_t free_b = 0, total_b = 0;
     cudaMemGetInfo(&free_b, &total_b);
-    const int lmax = (int)std::min<size_t>(std::max<size_t>(n, 4), std::max<size_t>(kStartLevels, std::min<size_t>(free_b / 8, (size_t)8 << 30) / std::max<size_t>(n, 1)));
-    for (int lcap = std::min(lmax, kStartLevels);; lcap = lmax) {
-        const int side = (int)todo.size() == nb ? teams : 1;  // reruns of some of the batches go one by one
+    const size_t slabs = std::min<size_t>(free_b / 8, (size_t)8 << 30) / std::max<size_t>(n, 1), deepest = std::max<size_t>(n, 4);
+    int lcap = (int)std::min<size_t>(deepest, kStartLevels), side = teams;
+    for (;;) {
         TArgs a{};
         a.nw8 = (int64_t)((n + 15) / 16 * 16);
         const size_t lv = (size_t)(lcap + 3) * side;
@@ -579,8 +580,11 @@ int run_thin(nk_graph *g, const int32_t *d_src, int32_t k, double *d_scores, con
         }
         if (ovf) return set_error(NK_ERR_OVERFLOW, "a shortest-path count exceeded 2^64 - 1");
         if (deep.empty()) return NK_OK;
+        side = (int)deep.size() == nb ? teams : 1;  // reruns of some of the batches go one by one
+        const int lmax = (int)std::min(deepest, slabs / side);
         if (lcap < lmax) {
             todo = deep;
+            lcap = lmax;
             continue;
         }
         // deeper than any level cap: the per-source form takes these sources

@@ -340,3 +340,32 @@ def test_width_follows_the_sources_with_arcs(nk):
     assert nk.last_run_stats()["batch"] == 128
     ref = oracle.closeness_sampled(rp, col, seed, 150)
     assert np.array_equal(far, ref[0]) and np.array_equal(reach, ref[1])
+
+
+def test_deep_searches_side_by_side_stay_within_their_memory(nk):
+    """Two batches of 8 whose searches are 1000 levels deep (a thousand paths of a thousand vertices from
+    one vertex): level slabs for both together within 8 GB, beside 84 bytes a vertex of rows and queues."""
+    import torch
+    n = 1_000_001
+    v = torch.arange(1, n, device="cuda", dtype=torch.int32)
+    g = nk.graph_from_edges(n, torch.where((v - 1) % 1000 == 0, 0, v - 1).int(), v)
+    src = np.concatenate([[0], 1000 * np.arange(14) + 1 + 37 * np.arange(14)]).astype(np.int32)
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    got = nk.betweenness_sources(g, src, 1.0)
+    assert nk.last_run_stats()["launches"] == 4  # both batches, with 48 levels and again with more
+    held = before - torch.cuda.mem_get_info()[0]
+    assert held < (8 << 30) + 2 * 84 * n + (1 << 28), held
+    # in a tree a vertex's dependency is the number of vertices that it separates from the source.  Path p
+    # has the vertices 1000 p + 1 + j, j = 0 ... 999 outwards: 999 - j beyond one; on the source's own path,
+    # between it and the root, j nearer the root, the root, and the other 999 paths
+    want = np.zeros(n)
+    j = np.arange(1000)
+    for s in src:
+        below = np.tile(999.0 - j, 1000)  # vertices further out, per path
+        if s:
+            p, i = divmod(int(s) - 1, 1000)
+            want[0] += 999 * 1000
+            below[1000 * p: 1000 * (p + 1)] = np.where(j > i, 999 - j, np.where(j < i, j + 1 + 999 * 1000, 0))
+        want[1:] += below
+    assert np.allclose(got, want, rtol=1e-9, atol=1e-12)
