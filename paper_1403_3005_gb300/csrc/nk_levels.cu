@@ -289,10 +289,14 @@ template <int W> __global__ void __launch_bounds__(kThreads, 4) k_levels(LArgs a
                 }
             });
             if (!dev::grid_barrier(a.ctrl, a.limit_ns)) return;
-            nq = __ldcg(a.qcnt + s1);
+            nq = min(__ldcg(a.qcnt + s1), a.n);
             for (long long i0 = tid - lane; i0 < nq; i0 += nthr) {
-                const bool in = i0 + lane < nq;
+                bool in = i0 + lane < nq;
                 const int w = in ? __ldcg(qnext + i0 + lane) : 0;
+                if (in && (unsigned)w >= (unsigned)a.n) {
+                    check_failed(a.status(), kErrCheck, 4, w);
+                    in = false;
+                }
                 Bits<W> nb;
                 if (in) nb = load_bits<W>(Fn + (size_t)w * W);
                 join<W>(a, in, w, d, nb, act, &bc);
