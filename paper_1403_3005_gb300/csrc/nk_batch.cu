@@ -1292,12 +1292,6 @@ int launch_batches(nk_graph *g, const int32_t *d_src, int32_t k, const int32_t *
             continue;
         }
         for (int bi : todo) {
-            if (h[bi].err == NK_ERR_TIMEOUT)
-                return set_error(NK_ERR_TIMEOUT, "batched sweep aborted: a bounded device-side wait or phase ran out (check %d, value %d)",
-                                 h[bi].where, h[bi].bad_id);
-            if (h[bi].err == kErrCheck)
-                return set_error(NK_ERR_CUDA, "batched sweep aborted: device range check %d failed (value %d)",
-                                 h[bi].where, h[bi].bad_id);
             ovf |= h[bi].ovf != 0;
             if (h[bi].err == kErrDepth) deep.push_back(bi);
         }
