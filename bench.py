@@ -355,10 +355,17 @@ def _cpu_baseline_child(config, seconds, rank_seed, q):
 
 
 # ------------------------------------------------------------------ widened rows
+def levels_bytes(n, A, B):
+    """Closeness by level bitsets, per batch: row offsets and columns once (4n + 4A), every vertex's
+    visited and level words read and written once (32nB/64), the two uint64 sums read and written
+    (32n)."""
+    return 4.0 * A + 4.0 * n + 32.0 * n * (B // 64) + 32.0 * n
+
+
 def closeness_bytes(n, A, B, depth):
-    """Closeness, per batched launch: the forward half of the betweenness model,
-    (4A + 12n) + 17nB, plus the level-sum pass (depth slabs of 8nB/64 bytes read, the two
-    uint64 sums read and written, 32n)."""
+    """Closeness by a sweep with path counts (not what the library runs; levels_bytes is), per batch:
+    the forward half of the betweenness model, (4A + 12n) + 17nB, plus the level-sum pass (depth
+    slabs of 8nB/64 bytes read, the two uint64 sums read and written, 32n)."""
     return (4.0 * A + 12.0 * n) + 17.0 * n * B + 8.0 * n * (B // 64) * depth + 32.0 * n
 
 
@@ -458,14 +465,14 @@ def extension_legs(nk, torch, g, n, A, m, k, B, opts, stats, sseed, args, flush,
                 best = (Bx, t)
         return best[0]
 
-    # closeness (Table 1): forward sweep and level sums
+    # closeness (Table 1): level bitsets and level sums
     far_d = torch.empty(n, dtype=torch.float64, device="cuda")
     reach_d = torch.empty(n, dtype=torch.float64, device="cuda")
     Bc = fastest(lambda Bx: lambda: nk.closeness_sampled(g, sseed, k, width(base, Bx), out=(far_d, reach_d)))
     ms, lms, st = timed(lambda: nk.closeness_sampled(g, sseed, k, width(base, Bc), out=(far_d, reach_d)), reps)
     leg = {"value": m * k / (ms / 1e3) / 1e9, "unit": UNIT, "ms_per_step": ms, "batch": Bc,
-           "roofline": _roof(closeness_bytes(n, A, Bc, st["max_depth"] + 1), lms, peak, peak_kind, f"k_batch<W={Bc // 64}> forward only"),
-           "form": "batched forward sweep, sampled sources, scale n/k"}
+           "roofline": _roof(levels_bytes(n, A, Bc), lms, peak, peak_kind, f"k_levels<W={Bc // 64}>"),
+           "form": "level bitsets without path counts, sampled sources, scale n/k"}
     if ora:
         o, rp_o, col_o, src_o = ora
         pos = [0]
@@ -743,7 +750,7 @@ def run_ours(args, world, rank, local):
                       "max_depth": stats["max_depth"],
                       "td_levels": stats["td_levels"], "bu_levels": stats["bu_levels"],
                       "l2": l2_note(n, A, B),
-                      "sigma": "uint64",
+                      "sigma": "uint64, in 32-bit rows while a batch's counts fit",
                       "parallelism": (f"one sampled set split over {world} GPUs, one NCCL all-reduce of n doubles"
                                       if world > 1 else "1 GPU")},
            "roofline": roofline, "gpu_launches": int(gpu_launches),

@@ -70,3 +70,12 @@ def test_committed_traffic_follows_kernel_sources():
     assert bench.committed_traffic("rmat24", 128, False) == want
     assert bench.committed_traffic("rmat24", 64) is None
     assert bench.committed_traffic("rmat24", 128, True) is None
+
+
+def test_closeness_roofline_is_that_of_its_kernel():
+    """The closeness leg names the kernel that runs, with the bytes that it cannot do without."""
+    n, A = 1000, 16000
+    assert bench.levels_bytes(n, A, 256) == 4 * A + 4 * n + 32 * n * 4 + 32 * n
+    legs = open(bench.__file__).read()
+    leg = legs[legs.index("# closeness (Table 1)"):legs.index('legs["closeness"]')]
+    assert "levels_bytes(" in leg and "k_levels<" in leg and "k_batch" not in leg
