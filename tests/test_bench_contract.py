@@ -74,6 +74,7 @@ def test_committed_traffic_follows_kernel_sources():
 
 def test_closeness_roofline_is_that_of_its_kernel():
     """The closeness leg names the kernel that runs, with the bytes that it cannot do without."""
+    import bench
     n, A = 1000, 16000
     assert bench.levels_bytes(n, A, 256) == 4 * A + 4 * n + 32 * n * 4 + 32 * n
     legs = open(bench.__file__).read()
