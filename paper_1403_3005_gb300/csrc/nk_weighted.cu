@@ -426,23 +426,22 @@ int run_weighted(nk_graph *g, const int32_t *d_src, int32_t k, double *d_scores,
     }
     if (bps < 1) return set_error(NK_ERR_CUDA, "weighted kernel cannot be resident");
     const int total = std::max(1, bps * num_sms() / std::max(1, cfg.grid_div));
-    // sources without arcs add nothing and would leave their group idle
+    // CTAs that a search can use: one per 2^17 arcs, or per 384 vertices up to 57 (3 at least): a bucket of
+    // a small graph has no work for more, and every barrier waits for all.  3, 6, 14 and 57 CTAs, ms, with 3
+    // and with 8 sources: ER 1000 0.46, 0.51, 0.51, 0.51 and 0.56, 0.56, 0.57, 0.59; ER 2000 0.53, 0.58,
+    // 0.58, 0.59 and 0.64, 0.63, 0.64, 0.64; ER 5000 0.79, 0.69, 0.65, 0.67 and 0.79, 0.72, 0.69, 0.72; ER
+    // 10000 1.04, 0.87, 0.78, 0.77 and 1.05, 0.86, 0.78, 0.80; ER 20000 1.34, 1.12, 0.92, 0.83 and 1.51,
+    // 1.10, 0.90, 0.86; R-MAT 12 0.83, 0.73, 0.70, 0.73 and 0.83, 0.74, 0.70, 0.76
+    const int small = std::max(3, std::min(57, n / 384)), most = (int)std::max<int64_t>(small, std::min<int64_t>(total, g->A >> 17));
+    // sources without arcs add nothing and would leave their group idle, which costs the others CTAs unless
+    // each search has all that it can use: then the compaction (a kernel, a copy, a wait: ER 1000 with 3
+    // sources 0.57 -> 0.46 ms without it) is left out
     Tmp csrc, ccnt;
-    if (d_scores && !dist_out && !sigma_out) {
-        NK_TRY(csrc.alloc(sizeof(int32_t) * (size_t)k, s));
-        NK_TRY(ccnt.alloc(sizeof(int32_t), s));
-        NK_TRY(compact_sources(g, d_src, k, csrc.as<int32_t>(), ccnt.as<int32_t>(), s));
-        int32_t kk = 0;
-        NK_CUDA(cudaMemcpyAsync(&kk, ccnt.p, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-        NK_CUDA(cudaStreamSynchronize(s));
-        if (kk < 0 || kk > k) return set_error(NK_ERR_CUDA, "source compaction returned %d of %d", kk, k);
-        d_src = csrc.as<int32_t>();
-        k = kk;
-    }
+    if (d_scores && !dist_out && !sigma_out && (int64_t)k * (cfg.grid_ctas > 0 ? cfg.grid_ctas : most) > total)
+        NK_TRY(compact_list(g, &d_src, &k, csrc, ccnt, s));
     // CTAs per search: the sources in as few equal rounds as leave each search a CTA per 2^20 arcs (3
-    // at least), and no more CTAs than a search can use, one per 2^17 arcs (57 at least).  R-MAT 18, 64
-    // listed sources, groups x CTAs: 64 x 6 10.4 ms, 32 x 14 9.4, 15 x 30 10.4, 8 x 57 12.0; 8 listed: 8 x
-    // 30 2.26, 8 x 57 1.68, 4 x 114 2.66; ER 100003, 64: 64 x 4 4.35, 64 x 6 3.56, 32 x 14 3.66, 15 x 30 6.0; 8: 8 x
+    // at least), and no more CTAs than a search can use.  R-MAT 18, 64 listed sources, groups x CTAs:
+    // 64 x 6 10.4 ms, 32 x 14 9.4, 15 x 30 10.4, 8 x 57 12.0; 8 listed: 8 x 30 2.26, 8 x 57 1.68, 4 x 114 2.66; ER 100003, 64: 64 x 4 4.35, 64 x 6 3.56, 32 x 14 3.66, 15 x 30 6.0; 8: 8 x
     // 4 3.75, 8 x 57 1.09; R-MAT 20, 64: 32 x 14 39.5, 8 x 57 32.3, 3 x 120 40.0.  grid_ctas overrides it.
     // As many groups as fit, k at most, and their state within a quarter of the free memory.
     int cpg = cfg.grid_ctas;
@@ -450,7 +449,6 @@ int run_weighted(nk_graph *g, const int32_t *d_src, int32_t k, double *d_scores,
         const int least = (int)std::max<int64_t>(bps, std::min<int64_t>(total, g->A >> 20));
         int rounds = 1;
         while (total / ((std::max(k, 1) + rounds - 1) / rounds) < least && rounds < k) ++rounds;
-        const int most = (int)std::max<int64_t>(57, std::min<int64_t>(total, g->A >> 17));
         cpg = std::max(1, std::min(most, total / ((std::max(k, 1) + rounds - 1) / rounds)));
     }
     cpg = std::min(cpg, total);

@@ -369,3 +369,24 @@ def test_deep_searches_side_by_side_stay_within_their_memory(nk):
             below[1000 * p: 1000 * (p + 1)] = np.where(j > i, 999 - j, np.where(j < i, j + 1 + 999 * 1000, 0))
         want[1:] += below
     assert np.allclose(got, want, rtol=1e-9, atol=1e-12)
+
+
+@pytest.mark.parametrize("kind,n,params", [("er", 1151, dict(avg_deg=8.0)), ("er", 1152, dict(avg_deg=8.0)), ("ba", 21888, dict(m0=3)),
+                                           ("rmat", 10, dict(edge_factor=8))])
+def test_weighted_small_graphs(nk, kind, n, params):
+    """A search of a small graph gets no more CTAs than its vertices can use (3 to 57), and a few sources
+    are swept as they come, without a compaction: sampler, sweep, sum, scale.  R-MAT: some without arcs."""
+    g = nk.graph_generate(kind, n, 4, **params)
+    n, rp, col = oracle.generate(kind, n, 4, **params)
+    nk.random_weights(g, 5, 16)
+    before = nk.launch_count()
+    nk.sample_sources(n, 6, 4)
+    sampler = nk.launch_count() - before
+    for k in (1, 4, 40):
+        before = nk.launch_count()
+        got = nk.betweenness_weighted_sampled(g, 6, k)
+        if k == 4:
+            assert nk.launch_count() - before == sampler + 3
+        assert nk.last_run_stats()["tpv"] <= max(3, min(57, n // 384))
+        ref = oracle.betweenness_weighted_sampled(rp, col, nk.export_weights(g), 6, k)
+        assert np.allclose(got, ref, rtol=1e-9, atol=1e-12)
