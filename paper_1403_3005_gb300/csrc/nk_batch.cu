@@ -888,8 +888,10 @@ __global__ void __launch_bounds__(kThreads, min_ctas<W, EDGE>()) k_batch(BArgs a
                     part = dev::ff_add(part, dev::ff_mul(s, facc[k]));
                 }
             }
-            part = dev::group_sum_ff<32>(part);
-            if (!EDGE && lane == 0 && part.hi != 0.0f) atomicAdd(a.scores + v, dev::ff_to_double(part));
+            if constexpr (!EDGE) {
+                const double sum = dev::warp_sum(part);
+                if (lane == 0 && sum != 0.0) atomicAdd(a.scores + v, sum);
+            }
         };
         for_work(a, {ql >= 0 ? queue_of(a) + ql : nullptr, nl}, a.wq + (lv0 + l) * 8 + WQ_BACK, st.hand,
                  [&](bool on, int v, int beg, int dg, int chunk) {

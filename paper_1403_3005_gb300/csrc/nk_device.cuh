@@ -261,6 +261,30 @@ struct ff_sum {
     __device__ __forceinline__ double to_double() const { return (double)s + ((double)c + (double)l); }
 };
 
+// The sum over the warp of non-negative double-single numbers, rounded to FP64 once: every number is split
+// into whole numbers of 2^-25, 2^-49 and 2^-61 of the largest one's power of two (all conversions but the
+// last are exact), which add up exactly in any order, in one REDUX each; the sum is cut at 2^-56 of it.
+// Five exchanges and ff_adds leave up to five roundings of 48 bits in the sum of a batch's dependencies, which
+// no later addition averages out, and take 65 instructions against 30 here.
+__device__ __forceinline__ double warp_sum(ff x)
+{
+    const unsigned full = 0xffffffffu;
+    // biased exponent of the largest; 2^-102 and less (no dependency is below 2^-64) counts as that
+    const unsigned e = max(__reduce_max_sync(full, __float_as_uint(x.hi)) >> 23, 25u);
+    const float up = __uint_as_float((279u - e) << 23);  // the largest becomes [2^25, 2^26)
+    const float p = __fmul_rn(x.hi, up), q = __fmul_rn(__fmul_rn(x.lo, up), 16777216.0f);  // |q| <= 2^25
+    const int i1 = __float2int_rz(p);
+    const float r = __fmul_rn(__fsub_rn(p, __int2float_rn(i1)), 16777216.0f);  // fraction of p: |q| <= 2^23 if there is one
+    const int q2 = __float2int_rn(q), r2 = __float2int_rn(r);
+    const float rest = __fadd_rn(__fsub_rn(q, __int2float_rn(q2)), __fsub_rn(r, __int2float_rn(r2)));
+    const unsigned s1 = __reduce_add_sync(full, (unsigned)i1);                      // < 2^31
+    const int s2 = __reduce_add_sync(full, q2 + r2);                                // |s2| <= 2^30
+    const int s3 = __reduce_add_sync(full, __float2int_rn(__fmul_rn(rest, 4096.0f)));
+    const long long sum = ((long long)s1 << 31) + (long long)s2 * 128 + (s3 >> 5);  // units of 2^(e - 183)
+    if (sum == 0) return 0.0;
+    return __longlong_as_double(__double_as_longlong(__ll2double_rn(sum)) + ((long long)((int)e - 183) << 52));
+}
+
 __device__ __forceinline__ unsigned lanemask_lt()
 {
     unsigned m;

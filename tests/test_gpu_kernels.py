@@ -390,3 +390,21 @@ def test_weighted_small_graphs(nk, kind, n, params):
         assert nk.last_run_stats()["tpv"] <= max(3, min(57, n // 384))
         ref = oracle.betweenness_weighted_sampled(rp, col, nk.export_weights(g), 6, k)
         assert np.allclose(got, ref, rtol=1e-9, atol=1e-12)
+
+
+@pytest.mark.parametrize("kind,params", [("er", dict(avg_deg=8.0)), ("rmat", dict(edge_factor=8))])
+def test_dependencies_of_a_batch_are_summed_exactly(nk, kind, params):
+    """The scores of 64 sources in one batch against those of the same sources one to a batch, summed in
+    FP64: a source's dependencies are the same numbers either way.  What the batch may lose is one
+    double-single addition per lane, 2^-49 each and independent over 32 lanes (2e-16 in the mean square), and
+    the FP64 roundings (1e-16).  Joining the lanes in double-single too loses 1e-15."""
+    import math
+    g = nk.graph_generate(kind, 1000 if kind == "er" else 10, 4, **params)
+    src = np.argsort(-np.diff(g.export_csr()[0]), kind="stable")[40:104].astype(np.int32)
+    opts = nk.run_opts(mode=nk.MODE_BATCHED, batch=64)
+    one = np.array([nk.betweenness_sources(g, src[i:i + 1], 1.0, opts) for i in range(len(src))])
+    want = np.array([math.fsum(c) for c in one.T])
+    got = nk.betweenness_sources(g, src, 1.0, opts)
+    assert np.array_equal(got == 0.0, want == 0.0)
+    nz = want > 0.0
+    assert np.sqrt(np.mean(((got[nz] - want[nz]) / want[nz]) ** 2)) < 5e-16
