@@ -1,7 +1,7 @@
 // Batched multi-source betweenness: B = 64*W sources share one sweep, and several such batches
-// one persistent cooperative launch, a row of the grid each.  The paper parallelises Brandes' algorithm over sources with one dependency
-// array per thread, summed at the end (Section 3.2); on the GPU the sources of a batch
-// instead share every pass over the CSR, so the adjacency of a level is read once for
+// one persistent cooperative launch, a row of the grid each.  The paper parallelises Brandes'
+// algorithm over sources with one dependency array per thread, summed at the end (Section 3.2);
+// on the GPU the sources of a batch instead share every pass over the CSR, so the adjacency of a level is read once for
 // all B shortest-path trees.
 //
 // State of one batch, all in HBM (b = source slot 0..B-1, q = word 0..W-1):
@@ -874,7 +874,7 @@ __global__ void __launch_bounds__(kThreads, min_ctas<W, EDGE>()) k_batch(BArgs a
         // delta/psi/score of vertex v from its successor sums facc (whole warp; the lane's slots
         // nib, its path counts sg): psi_v = 1/sigma_v + acc and delta_v = sigma_v * acc (Brandes'
         // recurrence with sigma_v factored out), in double-single; the vertex's delta summed over
-        // its source slots goes to the FP64 score once per vertex and level.  One warp adds to a
+        // its source slots (exactly, over the lanes) goes to the FP64 score once per vertex and level.  One warp adds to a
         // vertex's score per level, so the atomic addition, which returns nothing and is not
         // waited for, keeps the order of the additions.
         auto finish = [&](unsigned v, unsigned nib, const RowPart<W, S32> &sg, const dev::ff (&facc)[2 * W]) {
@@ -1154,6 +1154,7 @@ int launch_batches(nk_graph *g, const int32_t *d_src, int32_t k, const int32_t *
     // more than one batch: similar sources share one.  R-MAT 18, 670 sources by 128: 65.2M
     // rows gathered in the order of the ids, 42.8M in this order, 18.3 -> 13.4 ms; R-MAT 24,
     // 271 sources: 493 -> 348 ms; BA 10^6, 512 sources: 40.2 -> 36.9 ms; ER (no hubs) equal
+    // (both sides one batch at a time, with the gather of that time: the calls now take 10.7, 300 and 29.4)
     Tmp osrc, okey;
     if (d_count && k > B && !cfg.keep_order) {
         NK_TRY(osrc.alloc(sizeof(int32_t) * (size_t)k, s));
