@@ -147,7 +147,8 @@ int nk_sssp_noalloc(int32_t n, const int32_t *row_ptr, const int32_t *col, int64
                                 last bits of its scores may differ from run to run (distances and
                                 path counts never do) */
 #define NK_MODE_BATCHED 2    /* bitset multi-source kernel, `batch` sources per batch, several
-                                batches per launch */
+                                batches per launch; its scores do not depend on how many of
+                                them a launch holds */
 
 #define NK_DIR_AUTO 0        /* direction-optimising: switch by alpha */
 #define NK_DIR_TOP_DOWN 1    /* every level top-down (push from the frontier) */
@@ -163,7 +164,10 @@ int nk_sssp_noalloc(int32_t n, const int32_t *row_ptr, const int32_t *col, int64
                                   on first use and replay it for later calls with the same
                                   graph, seed, k, options and output pointer; every replay
                                   re-executes all kernels.  Falls back to the regular path
-                                  when a BFS is deeper than the captured level slabs. */
+                                  when a BFS is deeper than the captured level slabs.  It
+                                  spares a small call its host work; its batches run one after
+                                  another (64 sources each without a width), so where the plain
+                                  call runs several side by side that is the faster one */
 
 typedef struct nk_run_opts {
     int32_t mode;      /* NK_MODE_* */
@@ -196,6 +200,14 @@ typedef struct nk_run_stats {
     int64_t bu_levels;
     double alpha;
 } nk_run_stats;
+
+/* Device memory of the calls below: a graph keeps the workspace of its largest call so far until it
+ * is freed, and later calls use it again.  For every batch that runs side by side with others it holds
+ * 12 bytes of rows per source and vertex, and bitsets of 8 bytes per 64 sources, vertex and level (48
+ * levels at first).  Batches are added until their rows reach 3300 MB together (the last may go beyond)
+ * or their state a quarter of the free memory.  Batches with deeper searches run again, with
+ * level bitsets in up to half of the free memory; below 16 sources in up to an eighth of it, 8 GB at
+ * most.  A call also takes, until it returns, n doubles (edge betweenness: A) per batch side by side. */
 
 /* Exact betweenness: all n sources, scores[n] = (1/2) sum_s delta_s(v). */
 int nk_betweenness_exact(const nk_graph *g, double *scores);
@@ -297,8 +309,7 @@ int nk_edge_betweenness_sampled(const nk_graph *g, uint64_t seed, int32_t k, dou
                                 const nk_run_opts *opts);
 
 /* ---------------------------------------------------------------- closeness (Table 1) */
-/* Closeness from the same forward sweep (Table 1: closeness by a shortest-path search from
- * each node, and the approximation after Eppstein and Wang from s sampled sources).  For
+/* Closeness (Table 1: closeness by a shortest-path search from each node, and the approximation after Eppstein and Wang from s sampled sources).  For
  * every vertex v, with S the source set:
  *     far[v]   = scale * sum of d(s, v) over the sources s in S, s != v, that reach v,
  *     reach[v] = scale * number of those sources,
