@@ -440,15 +440,7 @@ int run_thin(nk_graph *g, const int32_t *d_src, int32_t k, double *d_scores, con
              cudaStream_t s)
 {
     Tmp csrc, ccnt;
-    NK_TRY(csrc.alloc(sizeof(int32_t) * (size_t)k, s));
-    NK_TRY(ccnt.alloc(sizeof(int32_t), s));
-    NK_TRY(compact_sources(g, d_src, k, csrc.as<int32_t>(), ccnt.as<int32_t>(), s));
-    int32_t kk = 0;
-    NK_CUDA(cudaMemcpyAsync(&kk, ccnt.p, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-    NK_CUDA(cudaStreamSynchronize(s));
-    if (kk < 0 || kk > k) return set_error(NK_ERR_CUDA, "source compaction returned %d of %d", kk, k);
-    d_src = csrc.as<int32_t>();
-    k = kk;
+    NK_TRY(compact_list(g, &d_src, &k, csrc, ccnt, s));
     st->mode = NK_MODE_BATCHED;
     st->batch = kT;
     if (k == 0) return NK_OK;
